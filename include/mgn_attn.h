@@ -68,7 +68,9 @@ enum { MGN_MODE_STRICT_F32 = 0, MGN_MODE_FAST_BF16 = 1 };
  *   lse_i = log sum_j exp(s_ij)  (natural log, of the scaled and masked scores);
  *   o_i   = sum_j exp(s_ij - lse_i) v_j.
  * q,k,v: in.  o: out [B,H,S,D] (mode's element type).  lse: out [B,H,S] f32.
- * Strict mode computes in f32 FFMA; fast mode multiplies bf16 operands on the
+ * Strict mode computes to f32 accuracy: its products run in f32 FFMA, or on the tensor
+ * cores with every f32 operand split into three bf16 parts (24 bits) and six partial
+ * products per product, accumulated in f32.  Fast mode multiplies bf16 operands on the
  * tensor cores with f32 accumulation and f32 softmax statistics.
  * Range (fast mode): a row's running softmax reference may stay up to 2^60 below the
  * largest score seen so far, so the unnormalised sums reach 2^60 * S_k * max|v|; they
@@ -88,8 +90,8 @@ int mgn_attn_fwd(const void* q, const void* k, const void* v, void* o, float* ls
  * dq, dk, dv: out.  workspace: device scratch of at least
  * mgn_attn_bwd_workspace_bytes(...) bytes, 256-byte aligned, contents ignored on
  * entry and undefined on exit; two calls that may overlap on the GPU need
- * distinct workspaces.  dq is accumulated with floating-point atomics, so its
- * low-order bits can differ from run to run; dk, dv, and the forward are
+ * distinct workspaces.  dq may be accumulated with floating-point atomics, so
+ * its low-order bits can differ from run to run; dk, dv, and the forward are
  * deterministic.
  */
 int mgn_attn_bwd(const void* q, const void* k, const void* v, const void* o, const void* d_o,
@@ -112,7 +114,7 @@ size_t mgn_attn_bwd_workspace_bytes(int B, int H, int S, int D, int mode);
  *   bottom-right corner (the last query sees every key) and needs S_q <= S_k, else the call
  *   returns MGN_ERR_UNSUPPORTED (a query row without a visible key has no softmax).
  * Everything else -- element types per mode, alignment, ownership, stream semantics, error
- * order, dq accumulated with floating-point atomics -- is as for mgn_attn_fwd / mgn_attn_bwd,
+ * order, dq possibly accumulated with floating-point atomics -- is as for mgn_attn_fwd / mgn_attn_bwd,
  * which are these functions with H_kv = H and S_q = S_k = S.  H % H_kv != 0 is MGN_ERR_INVALID_ARG.
  * The workspace of mgn_attn_bwd_ext is mgn_attn_bwd_workspace_bytes(B, H, S_q, D, mode) bytes.
  */

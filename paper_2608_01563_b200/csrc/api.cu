@@ -208,7 +208,8 @@ int mgn_attn_bwd_ext(const void* q, const void* k, const void* v, const void* o,
     unsigned* sched = fast ? reinterpret_cast<unsigned*>(static_cast<char*>(workspace) + ws_delta_bytes(rows)) : nullptr;
     float* dq_acc = fast ? reinterpret_cast<float*>(static_cast<char*>(workspace) + ws_delta_bytes(rows) + kSchedBytes)
                          : static_cast<float*>(dq);
-    const bool no_acc = fast && mgn::fast_bwd_writes_dq_directly(p);     // single key block: nothing accumulates
+    // a single key block (fast), the tensor-core kernels (strict): nothing accumulates in memory
+    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : mgn::strict_bwd_on_tensor_cores(p);
     cudaError_t e = mgn::launch_bwd_preprocess(o, d_o, delta, no_acc ? nullptr : dq_acc, sched, rows, D, fast ? 1 : 0, st);
     if (e != cudaSuccess) return MGN_ERR_CUDA;
     MainKernelTimer timer(st);
@@ -248,6 +249,12 @@ int mgn_attn_bwd_deterministic(const void* q, const void* k, const void* v, cons
         e = mgn::launch_fast_dq(p, q, k, v, d_o, lse, delta, dq, status, st);
         return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
     }
+    if (mgn::strict_bwd_on_tensor_cores(p)) {
+        e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
+                                   static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
+                                   static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv), status, st);
+        return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
+    }
     e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
                                static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta, nullptr,
                                static_cast<float*>(dk), static_cast<float*>(dv), status, st);
@@ -276,8 +283,9 @@ int mgn_attn_bwd_given_delta(const void* q, const void* k, const void* v, const 
     unsigned* sched = fast ? reinterpret_cast<unsigned*>(static_cast<char*>(workspace) + ws_delta_bytes(rows)) : nullptr;
     float* dq_acc = fast ? reinterpret_cast<float*>(static_cast<char*>(workspace) + ws_delta_bytes(rows) + kSchedBytes)
                          : static_cast<float*>(dq);
-    const bool no_acc = fast && mgn::fast_bwd_writes_dq_directly(p);
-    cudaError_t e = mgn::launch_bwd_clear(no_acc ? nullptr : dq_acc, rows * D, sched, st);
+    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : mgn::strict_bwd_on_tensor_cores(p);
+    cudaError_t e = cudaSuccess;
+    if (fast || !no_acc) e = mgn::launch_bwd_clear(no_acc ? nullptr : dq_acc, rows * D, sched, st);
     if (e != cudaSuccess) return MGN_ERR_CUDA;
     MainKernelTimer timer(st);
     if (!fast)

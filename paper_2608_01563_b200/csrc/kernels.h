@@ -89,6 +89,15 @@ int make_tmap_3d(CUtensorMap* out, const void* base, int elem_bytes, int is_bf16
 // Strict (f32 FFMA) kernels.
 cudaError_t launch_strict_fwd(const Problem& p, const float* q, const float* k, const float* v,
                               float* o, float* lse, unsigned* status, cudaStream_t st);
+// The same on the tensor cores (D = 64 and 128): f32 products as six bf16 partial products each.
+inline bool strict_fwd_on_tensor_cores(const Problem& p) { return p.D != 32 && p.Sk >= 64; }
+cudaError_t launch_strict_tc_fwd(const Problem& p, const float* q, const float* k, const float* v,
+                                 float* o, float* lse, unsigned* status, cudaStream_t st);
+// Backward on the tensor cores: no floating-point atomics, dq, dk, dv need not be cleared.
+inline bool strict_bwd_on_tensor_cores(const Problem& p) { return p.D != 32 && p.Sk >= 64 && p.Sq >= 64; }
+cudaError_t launch_strict_tc_bwd(const Problem& p, const float* q, const float* k, const float* v, const float* d_o,
+                                 const float* lse, const float* delta, float* dq, float* dk, float* dv,
+                                 unsigned* status, cudaStream_t st);
 cudaError_t launch_strict_bwd(const Problem& p, const float* q, const float* k, const float* v,
                               const float* d_o, const float* lse, const float* delta,
                               float* dq, float* dk, float* dv, unsigned* status, cudaStream_t st);

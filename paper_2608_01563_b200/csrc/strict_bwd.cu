@@ -375,6 +375,7 @@ cudaError_t launch_strict_bwd(const Problem& p, const float* q, const float* k, 
                               const float* d_o, const float* lse, const float* delta,
                               float* dq, float* dk, float* dv, unsigned* status, cudaStream_t st)
 {
+    if (strict_bwd_on_tensor_cores(p)) return launch_strict_tc_bwd(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
     int BM, BN;
     strict_bwd_tiles(p, &BM, &BN);
     switch (p.D) {

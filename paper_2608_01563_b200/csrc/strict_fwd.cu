@@ -372,6 +372,7 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
 cudaError_t launch_strict_fwd(const Problem& p, const float* q, const float* k, const float* v,
                               float* o, float* lse, unsigned* status, cudaStream_t st)
 {
+    if (strict_fwd_on_tensor_cores(p)) return launch_strict_tc_fwd(p, q, k, v, o, lse, status, st);
     int BM, BN;
     strict_fwd_tiles(p, &BM, &BN);
     switch (p.D) {

@@ -1,0 +1,289 @@
+// Strict (f32) products on the tensor cores: every f32 operand is split into three bf16 parts,
+//     x = hi + mid + lo,   hi = bf16(x), mid = bf16(x - hi), lo = bf16(x - hi - mid),
+// which together hold all 24 significant bits (the differences are exact in f32, the parts have f32's
+// exponent range), and a product of two operands is the sum of the six partial products
+//     lo*hi + hi*lo + mid*mid + mid*hi + hi*mid + hi*hi
+// accumulated in f32, smallest first.  What is left out (mid*lo, lo*mid, lo*lo) is below 2^-25 of the
+// product.  The tensor core adds into its accumulator with truncation, so an accumulation chain is kept
+// to one 64-step tile (four hi*hi steps at 16 a step) and tiles are added up in registers, rounded to
+// nearest, where an FFMA kernel would chain its whole contraction.
+//
+// Operand tiles: R rows of D values in D/64 blocks of 64 columns, each block one part after the other
+// (128-byte lines, 128-byte swizzle); the same tile serves as K-major and as MN-major operand.
+//
+// A 16-deep step of 128 rows takes about 50 clocks for 32 and for 64 columns, 64 to 72 for 128: its A operand
+// has to be fetched whatever the width.  So steps are made wider by running one part of A against two or
+// three adjacent parts of B at once ("stacked": 64 rows of hi followed by 64 rows of mid are a 128-row B
+// operand); the column sets that come out are added in registers.  Stacked scores of 64 rows cost four
+// steps of 228 clocks together per 16 columns of D instead of six of 300.  f32 tensors are read with plain 16-byte loads and split by converter warps.
+#pragma once
+#include "kernels.h"
+#include "umma.cuh"
+
+namespace mgn {
+namespace stc {
+
+constexpr float kLog2e = 1.4426950408889634f;   // 1.4426950216293335 as a float
+constexpr float kLn2 = 0.6931471805599453f, kLn2Lo = static_cast<float>(0.6931471805599453 - 0.6931471824645996);
+
+
+// Factor folded into one operand of the scores, so that they come out in the log2 domain.  The tensor core's
+// truncation makes a score smaller by a fixed share on average -- measured on single-key problems, where
+// LSE is the score: 0.93 x 2^-24 over 64 columns, 1.65 x 2^-24 over 128 -- which the factor gives back.
+inline double score_factor(float scale, int D) {
+    return static_cast<double>(scale) * 1.4426950408889634 * (1.0 + (D == 64 ? 0.93 : 1.65) * 0x1p-24);
+}
+
+// x * (c_hi + c_lo), rounded once.
+__device__ __forceinline__ float scaled(float x, float c_hi, float c_lo) { return fmaf(x, c_hi, x * c_lo); }
+
+// A pair of f32 (a in the low half) -> three packed bf16 pairs.
+__device__ __forceinline__ void split3(uint64_t x, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    const uint64_t minus1 = f2_pack(-1.f, -1.f);
+    float a, b;
+    f2_unpack(x, a, b);
+    hi = pack_bf16(a, b);
+    x = f2_fma(f2_pack(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus1, x);
+    f2_unpack(x, a, b);
+    mid = pack_bf16(a, b);
+    x = f2_fma(f2_pack(__uint_as_float(mid << 16), __uint_as_float(mid & 0xffff0000u)), minus1, x);
+    f2_unpack(x, a, b);
+    lo = pack_bf16(a, b);
+}
+
+template <int R> __host__ __device__ constexpr uint32_t part_bytes() { return R * 128; }          // of one 64-column block
+template <int R> __host__ __device__ constexpr uint32_t block_bytes() { return 3 * R * 128; }     // a 64-column block
+template <int D, int R> __host__ __device__ constexpr uint32_t tile_bytes() { return D / 64 * 3 * R * 128; }
+
+// Eight consecutive f32 of a row -> the 16-byte pieces of the three parts of a split tile.
+template <int D, int R>
+__device__ __forceinline__ void store_unit(uint32_t dst, int r, int piece, const float4 x, const float4 y) {
+    uint32_t h[4], m[4], l[4];
+    split3(f2_pack(x.x, x.y), h[0], m[0], l[0]);
+    split3(f2_pack(x.z, x.w), h[1], m[1], l[1]);
+    split3(f2_pack(y.x, y.y), h[2], m[2], l[2]);
+    split3(f2_pack(y.z, y.w), h[3], m[3], l[3]);
+    const uint32_t a = dst + (piece >> 3) * block_bytes<R>() + r * 128 + (((piece & 7) ^ (r & 7)) << 4);
+    constexpr uint32_t PART = part_bytes<R>();
+    sts128(a, h[0], h[1], h[2], h[3]);
+    sts128(a + PART, m[0], m[1], m[2], m[3]);
+    sts128(a + 2 * PART, l[0], l[1], l[2], l[3]);
+}
+
+// A team of kTeam threads turns a stream of R x D f32 tiles into split operand tiles, 2048 values at a time
+// (a slot): six 16-byte quads a thread, each replaced by the same quad of the next slot as soon as it has
+// been split and stored, so that global latency is covered by a whole slot of work.
+// The loop is rolled over slots on purpose: every role of these kernels runs its own code on each scheduler,
+// and larger unrolled bodies made instruction fetch the top stall (5.3 stalled warps per issue).  Staging the
+// f32 values in shared memory is slower: a load from there queues behind the tensor core's operand traffic
+// (512 queries over 4096 keys, D = 128: forward 0.239 ms against 0.169).
+constexpr int kTeam = 96;
+
+template <int D, int R, bool SCALED = false>
+struct Converter {
+    static constexpr int QUADS = D / 4;                                             // 16-byte quads of a row
+    static constexpr int SLOT_ROWS = 2048 / D, SLOTS = R / SLOT_ROWS, STEP = kTeam / QUADS;
+    static constexpr int NQ = (SLOT_ROWS + STEP - 1) / STEP;                        // quads of a thread in a slot
+    static_assert(R % SLOT_ROWS == 0 && kTeam % QUADS == 0 && SLOT_ROWS % 8 == 0, "");
+
+    float4 buf[NQ];
+    uint32_t off[NQ];         // where they go in a slot of an operand tile
+    int row, quad;
+    float c_hi, c_lo;         // SCALED: what the values are multiplied by
+
+    __device__ __forceinline__ explicit Converter(int t, float hi = 1.f, float lo = 0.f)
+        : row(t / QUADS), quad(t % QUADS), c_hi(hi), c_lo(lo) {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            const int r = row + k * STEP;
+            off[k] = (quad >> 4) * block_bytes<R>() + r * 128 + ((((quad >> 1) & 7) ^ (r & 7)) << 4) + (quad & 1) * 8;
+        }
+    }
+    // Converts tiles 0 .. n-1.  src(i, rows) gives the first row of tile i and how many rows exist from there;
+    // dst(i) waits until the tile's stage is free and returns its address; done(i) follows the stores.
+    template <class Src, class Dst, class Done>
+    __device__ __forceinline__ void run(int n, Src src, Dst dst, Done done) {
+        int rows;
+        const float* g = src(0, rows) + row * D + quad * 4;
+        auto load = [&](int k) {
+            const int r = row + k * STEP;
+            buf[k] = r < min(rows, SLOT_ROWS) ? __ldg(reinterpret_cast<const float4*>(g + k * STEP * D))
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) load(k);
+        uint32_t d = 0;
+        int sl = 0, i = 0;
+#pragma unroll 1
+        while (i < n) {
+            if (sl == 0) d = dst(i);
+            if (sl == SLOTS - 1) {                       // the next slot is the first of the next tile
+                if (i + 1 < n) g = src(i + 1, rows) + row * D + quad * 4;
+                else rows = 0;
+            } else {
+                g += SLOT_ROWS * D;
+                rows -= SLOT_ROWS;
+            }
+#pragma unroll
+            for (int k = 0; k < NQ; ++k) {
+                if (row + k * STEP < SLOT_ROWS) {
+                    uint32_t h[2], m[2], l[2];
+                    if constexpr (SCALED)
+                        buf[k] = make_float4(scaled(buf[k].x, c_hi, c_lo), scaled(buf[k].y, c_hi, c_lo),
+                                             scaled(buf[k].z, c_hi, c_lo), scaled(buf[k].w, c_hi, c_lo));
+                    split3(f2_pack(buf[k].x, buf[k].y), h[0], m[0], l[0]);
+                    split3(f2_pack(buf[k].z, buf[k].w), h[1], m[1], l[1]);
+                    sts64(d + off[k], h[0], h[1]);
+                    sts64(d + off[k] + part_bytes<R>(), m[0], m[1]);
+                    sts64(d + off[k] + 2 * part_bytes<R>(), l[0], l[1]);
+                }
+                load(k);
+            }
+            d += SLOT_ROWS * 128;
+            if (++sl == SLOTS) {
+                fence_proxy_async_smem();
+                done(i);
+                ++i;
+                sl = 0;
+            }
+        }
+    }
+};
+
+// Splits `n32` groups of 32 consecutive f32 values of one row (null: zeros), times c_hi + c_lo, into tensor
+// memory: part a goes to columns t + a * part_cols.
+__device__ __forceinline__ void split_row_to_tmem(uint32_t t, int part_cols, const float* src, int n32, float c_hi, float c_lo) {
+#pragma unroll 1
+    for (int c = 0; c < n32; ++c) {
+        uint32_t h[16], m[16], l[16];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float4 x = src ? __ldg(reinterpret_cast<const float4*>(src + 32 * c) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+            split3(f2_pack(scaled(x.x, c_hi, c_lo), scaled(x.y, c_hi, c_lo)), h[2 * e], m[2 * e], l[2 * e]);
+            split3(f2_pack(scaled(x.z, c_hi, c_lo), scaled(x.w, c_hi, c_lo)), h[2 * e + 1], m[2 * e + 1], l[2 * e + 1]);
+        }
+        tmem_st16(t + 16 * c, h);
+        tmem_st16(t + part_cols + 16 * c, m);
+        tmem_st16(t + 2 * part_cols + 16 * c, l);
+    }
+}
+
+// The partial products as issued.  A term: part of A, first part of B, how many adjacent parts of B it runs
+// against, and the column set that its first one goes to.
+//  - Scores (the exponent of P): hi hi has a set of its own.  The forward and both backward kernels then round
+//    a score alike whichever operand is A, and P = exp(s - LSE) is as good as a difference of two equally
+//    rounded numbers even where both are large; with hi mid and mid hi split between the sets by operand, a
+//    row that attends to one key (scores near 130 in the log2 domain) had 2.5e-5 of error in P instead of 8e-6.
+//  - Everything else: smallest first, hi hi last.
+struct Term { uint32_t a, b, n, set; };
+template <bool SCORE, int ST> __device__ __forceinline__ Term term(int t) {
+    if constexpr (SCORE && ST == 2) {        // hi [hi mid], mid hi, mid mid, lo hi, hi lo
+        return {(0x02110u >> (4 * t)) & 3u, (0x20100u >> (4 * t)) & 3u, (0x11112u >> (4 * t)) & 3u, (0x11110u >> (4 * t)) & 3u};
+    } else if constexpr (SCORE) {            // hi [hi mid lo], mid [hi mid], lo hi
+        return {(0x210u >> (4 * t)) & 3u, 0u, (0x123u >> (4 * t)) & 3u, (0x210u >> (4 * t)) & 3u};
+    } else if constexpr (ST == 1) {          // lo hi, hi lo, mid mid, mid hi, hi mid, hi hi
+        return {(0x001102u >> (4 * t)) & 3u, (0x010120u >> (4 * t)) & 3u, 1u, 0u};
+    } else if constexpr (ST == 2) {          // mid [hi mid], lo hi, hi lo, hi [hi mid]
+        return {(0x0021u >> (4 * t)) & 3u, (0x0200u >> (4 * t)) & 3u, (0x2112u >> (4 * t)) & 3u, (0x0100u >> (4 * t)) & 3u};
+    } else {                                 // mid [hi mid lo], lo hi, hi [hi mid lo]
+        return {(0x021u >> (4 * t)) & 3u, 0u, (0x313u >> (4 * t)) & 3u, 0u};
+    }
+}
+template <bool SCORE, int ST> __device__ constexpr int n_terms() {
+    return SCORE && ST == 2 ? 5 : ST == 1 ? 6 : ST == 2 ? 4 : 3;
+}
+
+// A region of tensor memory that receives rows of N values in ST column sets and is later overwritten by the
+// three packed parts of what is formed from them.  The N/2 values of a half are worked on by one thread (or in
+// one go) and its parts stay within the columns that held those values (ST = 1: plus N/4 columns of a free
+// quarter in front), so a half never overwrites values of the other half.
+template <int N, int ST> __host__ __device__ constexpr uint32_t x_cols() { return ST == 1 ? 3 * N / 2 : ST * N; }
+template <int N, int ST> __host__ __device__ constexpr uint32_t x_value_col() { return ST == 1 ? N / 2 : 0; }   // of set 0
+template <int N, int ST> __host__ __device__ constexpr uint32_t x_half_part_col(int half, int part) {
+    return ST == 1 ? (part == 2 ? half * (N / 4) : N / 2 + half * (N / 2) + part * (N / 4))
+                   : (part == 2 ? N + half * (N / 2) : half * (N / 2) + part * (N / 4));
+}
+// columns of 16-value contraction step kk
+template <int N, int ST> __device__ __forceinline__ uint32_t x_part_col(uint32_t part, int kk) {
+    constexpr int SPH = N / 32;                          // steps per half
+    return x_half_part_col<N, ST>(kk / SPH, part) + (kk % SPH) * 8;
+}
+
+template <int N> __device__ __forceinline__ void tmem_load(uint32_t t, uint32_t (&v)[N]) {
+    static_assert(N == 16 || N == 32, "");
+    if constexpr (N == 32) tmem_ld32(t, v);
+    else tmem_ld16(t, v);
+}
+// W f32 columns of this thread's lane, summed over ST sets `stride` columns apart (the hi hi set last).
+template <int W, int ST> __device__ __forceinline__ void load_sets(uint32_t t, uint32_t stride, float (&v)[W]) {
+    uint32_t s[ST][W];
+#pragma unroll
+    for (int i = 0; i < ST; ++i) tmem_load<W>(t + i * stride, s[i]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int e = 0; e < W; e += 2) {
+        uint64_t x = f2_pack(__uint_as_float(s[ST - 1][e]), __uint_as_float(s[ST - 1][e + 1]));
+#pragma unroll
+        for (int i = ST - 2; i >= 0; --i) x = f2_add(x, f2_pack(__uint_as_float(s[i][e]), __uint_as_float(s[i][e + 1])));
+        f2_unpack(x, v[e], v[e + 1]);
+    }
+}
+// The values of one half of a region's row.
+template <int N, int ST> __device__ __forceinline__ void load_half(uint32_t x, int half, float (&v)[N / 2]) {
+    load_sets<N / 2, ST>(x + x_value_col<N, ST>() + half * (N / 2), N, v);
+}
+// The packed parts of a half row (N/2 values) into its columns.
+template <int N, int ST> __device__ __forceinline__ void store_half_parts(uint32_t x, int half, const uint32_t (&h)[N / 4],
+                                                                          const uint32_t (&m)[N / 4], const uint32_t (&l)[N / 4]) {
+    if constexpr (N == 64) {
+        tmem_st16(x + x_half_part_col<N, ST>(half, 0), h);
+        tmem_st16(x + x_half_part_col<N, ST>(half, 1), m);
+        tmem_st16(x + x_half_part_col<N, ST>(half, 2), l);
+    } else {
+        tmem_st8(x + x_half_part_col<N, ST>(half, 0), h);
+        tmem_st8(x + x_half_part_col<N, ST>(half, 1), m);
+        tmem_st8(x + x_half_part_col<N, ST>(half, 2), l);
+    }
+}
+
+// Sets of D[128 x R] = A B^T over D columns, at tensor-memory column d; B a split tile of R rows.  A in tensor
+// memory (part p at a + p * D / 2) or a split tile of 128 rows (a: its descriptor).  SCORE: see term().
+template <bool SCORE, int D, int R, int ST, typename A>
+__device__ __forceinline__ void issue_scores(uint32_t d, A a_at, uint64_t b_desc) {
+#pragma unroll 1
+    for (int t = 0; t < n_terms<SCORE, ST>(); ++t) {
+        const Term m = term<SCORE, ST>(t);
+        const uint32_t idesc = umma_idesc_bf16(128, R, false, false) + (m.n - 1) * ((R >> 3) << 17);
+        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
+        const uint32_t dt = d + m.set * R;
+#pragma unroll
+        for (int kk = 0; kk < D / 16; ++kk) {
+            const uint64_t bk = b + (((kk >> 2) * block_bytes<R>() + (kk & 3) * 32) >> 4);
+            const uint32_t add = (t > 0 || kk > 0) ? 1u : 0u;
+            if constexpr (sizeof(A) == 4) umma_ts(dt, a_at + m.a * (D / 2) + kk * 8, bk, idesc, add);
+            else umma_ss(dt, a_at + ((m.a * part_bytes<128>() + (kk >> 2) * block_bytes<128>() + (kk & 3) * 32) >> 4), bk, idesc, add);
+        }
+    }
+}
+// Sets of D[128 x D] = X B over the R rows of the split tile B (as MN-major operand, see rows_desc), X the parts
+// in a region of ST_X sets.  Stacking (ST = 2) needs adjacent parts to be D columns apart: D = 64.
+template <int D, int R> __device__ __forceinline__ uint64_t rows_desc(uint32_t tile) {
+    return umma_smem_desc(tile, D == 64 ? part_bytes<R>() : block_bytes<R>(), 1024);
+}
+template <int D, int R, int ST_X, int ST>
+__device__ __forceinline__ void issue_rows(uint32_t d, uint32_t x, uint64_t b_desc) {
+    static_assert(ST == 1 || D == 64, "");
+#pragma unroll 1
+    for (int t = 0; t < n_terms<false, ST>(); ++t) {
+        const Term m = term<false, ST>(t);
+        const uint32_t idesc = umma_idesc_bf16(128, D, false, true) + (m.n - 1) * ((D >> 3) << 17);
+        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
+        const uint32_t dt = d + m.set * D;
+#pragma unroll
+        for (int kk = 0; kk < R / 16; ++kk)
+            umma_ts(dt, x + x_part_col<R, ST_X>(m.a, kk), b + ((kk * 2048) >> 4), idesc, (t > 0 || kk > 0) ? 1u : 0u);
+    }
+}
+
+}  // namespace stc
+}  // namespace mgn

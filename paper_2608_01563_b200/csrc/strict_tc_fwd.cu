@@ -1,0 +1,332 @@
+// Strict forward on the tensor cores: O = softmax(scale Q K^T) V and LSE, f32 in and out, products as
+// six bf16 partial products per f32 product (strict_tc.cuh).
+//
+// One 512-thread CTA owns 128 query rows of one head and walks over key blocks (64 keys; 32
+// at D = 128, where tensor memory then has room for stacked scores).  Q is split once
+// into tensor memory (the A operand of the scores).  Roles:
+//   warp 0 / warp 4   one lane issues the score products / the P V products
+//   warps 1-3 / 5-7   split V blocks / K blocks into shared memory
+//   warps 8-11/12-15  softmax of the even / odd key blocks, one thread per query row
+// The two softmax warpgroups are independent online softmaxes over their halves of the keys: each thread
+// keeps its own maximum, sum and O accumulators (the P V product of every block is added up in registers,
+// rounded to nearest) and the halves meet once, in the epilogue, so no block needs an exchange.
+// A maximum is rounded up to a whole number (in the log2 domain), so that every rescaling factor is a power
+// of two and exact.
+// A barrier wait costs an issuing lane 250-350 clocks while the tensor core streams operands, and the core's
+// queue runs dry meanwhile.  Hence two issuing lanes with one wait per product: SGO(n) = K(n) split and
+// P(n-2) read, PGO(n) = V(n) split, P(n) written and the result of block n-1 read; and the completion of a
+// product also tells the converters that its stage is free.  (One lane with a barrier per condition: 512
+// queries over 4096 keys, D = 128, 0.213 ms.)
+// Tensor memory: Q parts 3 D/2 columns, two score regions, one P V result.
+#include "strict_tc.cuh"
+
+namespace mgn {
+namespace {
+
+using namespace stc;
+
+constexpr int kThreads = 512, kBM = 128;
+
+template <int D>
+struct Cfg {
+    static constexpr int NST = 2;                               // stages of K and of V: even and odd blocks
+    static constexpr int R = D == 64 ? 64 : 32;                 // keys of a block
+    static constexpr int STAGE = tile_bytes<D, R>();
+    static constexpr int OFF_K = 0, OFF_V = NST * STAGE, OFF_BAR = 2 * NST * STAGE;
+    static constexpr int SMEM = OFF_BAR + 512 + 1024;
+    static constexpr int PITCH = D + 1;                         // floats per row of the epilogue's exchange tile
+    static_assert(kBM * PITCH * 4 + kBM * 8 <= OFF_BAR, "the exchange tile lies over the K and V stages");
+    static_assert(SMEM <= 232448, "shared memory budget");
+    static constexpr int ST = D == 64 ? 2 : 3, STO = D == 64 ? 2 : 1;       // column sets of scores, of results
+    static constexpr uint32_t X = x_cols<R, ST>();
+    static constexpr uint32_t TM_Q = 0, TM_X = 3 * D / 2, TM_O = TM_X + 2 * X;
+    static_assert(TM_O + STO * D <= 512, "tensor memory budget");
+    // barriers, one per block parity: conditions of the score product, of the P V product; their completion
+    enum { SGO = 0, PGO = 2, SDONE = 4, PDONE = 6, QFULL = 8, COUNT = 9 };
+};
+
+// One query row by plain f32 arithmetic over its visible keys: rows whose split result is not finite take
+// it (an infinite or NaN input, or a product beyond the f32 range, where hi - hi parts would meet as NaN).
+template <int D>
+__device__ __noinline__ float plain_row(const float* q, const float* k, const float* v, int n_vis, float c2, float* out)
+{
+    auto score = [&](int j) {
+        float s = 0.f;
+        for (int d = 0; d < D; ++d) s = fmaf(q[d], k[static_cast<size_t>(j) * D + d], s);
+        return __fmul_rn(s, c2);       // rounded: contracted with the subtraction below, a huge maximum would not meet itself
+    };
+    float m = -INFINITY, l = 0.f;
+    for (int j = 0; j < n_vis; ++j) m = fmaxf(m, score(j));
+    for (int d = 0; d < D; ++d) out[d] = 0.f;
+    for (int j = 0; j < n_vis; ++j) {
+        const float p = ex2(score(j) - m);
+        l += p;
+        for (int d = 0; d < D; ++d) out[d] = fmaf(p, v[static_cast<size_t>(j) * D + d], out[d]);
+    }
+    const float inv = 1.0f / l;
+    for (int d = 0; d < D; ++d) out[d] *= inv;
+    return kLn2 * (m + lg2(l));
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1)
+strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
+                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int BH, int H, int G, int n_qt,
+                     int causal, float c_hi, float c_lo, unsigned* status)
+{
+    using C = Cfg<D>;
+    constexpr int R = C::R;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t base = smem_u32(smem);
+    const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
+    auto bar = [&](int i) { return bars + 8u * i; };
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
+
+    // Heaviest (last) query tiles first when causal.
+    const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / BH;
+    const int bh = static_cast<int>(blockIdx.x) % BH;
+    const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
+    const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
+    const int i0 = qt * kBM;
+    const int i_last = min(i0 + kBM, Sq) - 1;
+    const int n_kb = causal ? (i_last + off) / R + 1 : (Sk + R - 1) / R;
+    if (tid == 0) {
+        mbar_init(bar(C::QFULL), 256);
+        for (int w = 0; w < 2; ++w) {
+            mbar_init(bar(C::SGO + w), kTeam + 1);             // K split; P of two blocks back read
+            mbar_init(bar(C::PGO + w), kTeam + 256);           // V split; P written; last block's result read
+            mbar_init(bar(C::SDONE + w), 1);
+            mbar_init(bar(C::PDONE + w), 1);
+        }
+        fence_mbar_init();
+    }
+    __syncwarp();
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = lds32u(tmem_slot);
+
+    if (warp < 8) {
+        reg_dealloc<56>();
+        if (warp == 0) {
+            if (lane == 0) {
+                // -------------------------------------------------------------- score products
+                const uint64_t dK = umma_smem_desc(base + C::OFF_K, 16, 1024);
+                mbar_arrive(bar(C::SGO));                      // nothing to read yet in either score region
+                mbar_arrive(bar(C::SGO + 1));
+                mbar_wait(bar(C::QFULL), 0, status);
+#pragma unroll 1
+                for (int n = 0; n < n_kb; ++n) {
+                    const int w = n & 1;
+                    mbar_wait(bar(C::SGO + w), (n >> 1) & 1, status);
+                    tc_fence_after();
+                    issue_scores<true, D, R, C::ST>(tmem + C::TM_X + w * C::X, tmem + C::TM_Q,
+                                       dK + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                    umma_commit(bar(C::SDONE + w));
+                }
+            }
+            __syncwarp();
+        } else if (warp == 4) {
+            if (lane == 0) {
+                // -------------------------------------------------------------- P V products
+                const uint64_t mV = rows_desc<D, R>(base + C::OFF_V);
+#pragma unroll 1
+                for (int n = 0; n < n_kb; ++n) {
+                    const int w = n & 1;
+                    mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
+                    tc_fence_after();
+                    issue_rows<D, R, C::ST, C::STO>(tmem + C::TM_O, tmem + C::TM_X + w * C::X,
+                                     mV + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                    umma_commit(bar(C::PDONE + w));
+                    umma_commit(bar(C::SGO + w));
+                }
+            }
+            __syncwarp();
+        } else {
+            // ------------------------------------------------------------------ K and V converters (one code)
+            const bool is_k = warp >= 4;
+            const float* head = (is_k ? K : V) + static_cast<size_t>(bhk) * Sk * D;
+            const int full = is_k ? C::SGO : C::PGO, done = is_k ? C::SDONE : C::PDONE;
+            const uint32_t stages = base + (is_k ? C::OFF_K : C::OFF_V);
+            Converter<D, R> cv(is_k ? tid - 160 : tid - 32);
+            cv.run(n_kb,
+                   [&](int i, int& rows) {
+                       rows = Sk - i * R;
+                       return head + static_cast<size_t>(i) * R * D;
+                   },
+                   [&](int i) {
+                       if (i >= 2) mbar_wait(bar(done + (i & 1)), ((i >> 1) & 1) ^ 1, status);
+                       return stages + (i & 1) * C::STAGE;
+                   },
+                   [&](int i) { mbar_arrive(bar(full + (i & 1))); });
+        }
+    } else {
+        // ------------------------------------------------------------------ softmax
+        reg_alloc<200>();
+        const int w = (warp - 8) >> 2;
+        const int r = tid & 127;                               // row within the tile = tensor-memory lane
+        const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
+        const uint32_t tX = tmem + lane_base + C::TM_X + w * C::X, tO = tmem + lane_base + C::TM_O;
+        const int i = i0 + r;
+        const bool row_ok = i < Sq;
+        const float* qrow = Q + (static_cast<size_t>(bh) * Sq + i) * D;
+        split_row_to_tmem(tmem + lane_base + C::TM_Q + w * (D / 4), D / 2, row_ok ? qrow + w * (D / 2) : nullptr, D / 64,
+                          c_hi, c_lo);
+        tmem_st_wait();
+        tc_fence_before();
+        mbar_arrive(bar(C::QFULL));
+        if (w == 1) mbar_arrive(bar(C::PGO));                  // block 0 has no result before it to wait for
+
+        float m = -INFINITY, l = 0.f;
+        float acc[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) acc[d] = 0.f;
+        const int vis = min(Sk, causal ? i + off + 1 : Sk);    // keys this row sees
+
+        for (int n = w; n < n_kb; n += 2) {
+            const uint32_t ph = (n >> 1) & 1;
+            const int lim = vis - n * R;                   // visible columns of this block
+            const bool masked = (causal && n * R + R - 1 > i0 + off) || n * R + R > Sk;
+            mbar_wait(bar(C::SDONE + w), ph, status);
+            tc_fence_after();
+            // Blocks of 32 keep their scores in registers between the maximum and the exponentials; those of 64 are
+            // read twice, a half at a time (the loops stay rolled for the instruction cache).
+            constexpr int W = R / 2;
+            constexpr bool KEEP = R == 32;
+            float s[KEEP ? 2 : 1][W];
+            float mx = -INFINITY;
+            auto mask_half = [&](int h, float (&v)[W]) {          // ex2(-inf) = 0
+                if (masked) {
+#pragma unroll
+                    for (int e = 0; e < W; ++e)
+                        if (W * h + e >= lim) v[e] = -INFINITY;
+                }
+            };
+#pragma unroll(KEEP ? 2 : 1)
+            for (int h = 0; h < 2; ++h) {
+                float (&v)[W] = s[KEEP ? h : 0];
+                load_half<R, C::ST>(tX, h, v);
+                mask_half(h, v);
+#pragma unroll
+                for (int e = 0; e < W; ++e) mx = fmaxf(mx, v[e]);
+            }
+            const float m_new = fmaxf(m, ceilf(mx));
+            const float ref = m_new == -INFINITY ? 0.f : m_new;   // no visible key so far: every p is 0
+            const float corr = ex2(m - ref);
+            m = m_new;
+            const uint64_t nref = f2_pack(-ref, -ref);
+            uint64_t sum0 = f2_pack(0.f, 0.f), sum1 = sum0;
+#pragma unroll(KEEP ? 2 : 1)
+            for (int h = 0; h < 2; ++h) {
+                float (&v)[W] = s[KEEP ? h : 0];
+                if constexpr (!KEEP) {
+                    load_half<R, C::ST>(tX, h, v);
+                    mask_half(h, v);
+                }
+                uint32_t p0[W / 2], p1[W / 2], p2[W / 2];
+#pragma unroll
+                for (int e = 0; e < W; e += 2) {
+                    float a, b;
+                    f2_unpack(f2_add(f2_pack(v[e], v[e + 1]), nref), a, b);
+                    const uint64_t p = f2_pack(ex2(a), ex2(b));
+                    if (e & 2) sum1 = f2_add(sum1, p);
+                    else sum0 = f2_add(sum0, p);
+                    split3(p, p0[e / 2], p1[e / 2], p2[e / 2]);
+                }
+                store_half_parts<R, C::ST>(tX, h, p0, p1, p2);
+            }
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(bar(C::PGO + w));
+            float sa, sb;
+            f2_unpack(f2_add(sum0, sum1), sa, sb);
+            l = fmaf(l, corr, sa + sb);
+
+            mbar_wait(bar(C::PDONE + w), ph, status);
+            tc_fence_after();
+#pragma unroll
+            for (int h = 0; h < D / 32; ++h) {
+                float v[32];
+                load_sets<32, C::STO>(tO + 32 * h, D, v);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[32 * h + e] = fmaf(acc[32 * h + e], corr, v[e]);
+            }
+            tc_fence_before();
+            mbar_arrive(bar(C::PGO + (w ^ 1)));                // the next block's product may overwrite it
+        }
+
+        // ---- the two halves of the keys meet in shared memory (the K and V stages are dead)
+        float* tile = reinterpret_cast<float*>(smem);
+        float* stat = tile + kBM * C::PITCH;
+        float* row = tile + r * C::PITCH;
+        named_bar_sync(1, 256);
+        if (w == 1) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) row[d] = acc[d];
+            stat[r] = m;
+            stat[kBM + r] = l;
+        }
+        named_bar_sync(1, 256);
+        if (w == 0) {
+            const float m1 = stat[r], l1 = stat[kBM + r];
+            const float mm = fmaxf(m, m1);
+            const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+            const float lt = fmaf(l, a0, l1 * a1);
+            const float inv = 1.0f / lt;
+            const float b0 = a0 * inv, b1 = a1 * inv;
+            // mm is a whole number: its share of the natural logarithm is formed with one rounding
+            float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, lg2(lt) * kLn2));
+            float bad = 0.f;                                   // NaN once an output is not finite
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const float x = fmaf(acc[d], b0, row[d] * b1);
+                row[d] = x;
+                bad = fmaf(x, 0.f, bad);
+            }
+            if (row_ok) {
+                if (bad != 0.f || !(fabsf(lse) < INFINITY)) lse = plain_row<D>(qrow, K + static_cast<size_t>(bhk) * Sk * D, V + static_cast<size_t>(bhk) * Sk * D, vis,
+                                       c_hi, row);
+                LSE[static_cast<size_t>(bh) * Sq + i] = lse;
+            }
+        }
+        named_bar_sync(1, 256);
+        float* og = O + (static_cast<size_t>(bh) * Sq + i0) * D;
+        const int n_rows = min(kBM, Sq - i0);
+        for (int x = tid - 256; x < n_rows * D; x += 256) og[x] = tile[(x / D) * C::PITCH + x % D];
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+template <int D>
+cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse,
+                   unsigned* status, cudaStream_t st)
+{
+    using C = Cfg<D>;
+    auto kern = strict_tc_fwd_kernel<D>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_fwd attributes");
+    const int n_qt = (p.Sq + kBM - 1) / kBM;
+    const long long blocks = static_cast<long long>(n_qt) * p.BH();
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const double c = score_factor(p.scale, D);
+    const float c_hi = static_cast<float>(c), c_lo = static_cast<float>(c - c_hi);
+    kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(q, k, v, o, lse, p.Sq, p.Sk, p.BH(), p.H, p.group(),
+                                                                   n_qt, p.causal, c_hi, c_lo, status);
+    return MGN_FAIL(cudaGetLastError(), "strict_tc_fwd launch");
+}
+
+}  // namespace
+
+cudaError_t launch_strict_tc_fwd(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse,
+                                 unsigned* status, cudaStream_t st)
+{
+    return p.D == 64 ? launch<64>(p, q, k, v, o, lse, status, st) : launch<128>(p, q, k, v, o, lse, status, st);
+}
+
+}  // namespace mgn

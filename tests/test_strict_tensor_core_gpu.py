@@ -1,0 +1,84 @@
+"""Strict mode on the tensor cores (D = 64 and 128): f32 products formed from three bf16 parts per
+operand.  Sizes at the edges of its tiles (128 lane rows; streamed blocks of 64 rows, 32 at D = 128 in
+the backward), operands of very different magnitude, and inputs that are not finite."""
+import math
+
+import pytest
+import torch
+
+from paper_2608_01563_b200 import binding as mgn
+from paper_2608_01563_b200 import inputs as synth
+
+import helpers as hp
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # B, H, Hkv, Sq, Sk, D, causal
+    (1, 2, 2, 64, 64, 64, True),         # one block, half a lane tile
+    (1, 2, 2, 65, 65, 128, True),        # one row into the second block
+    (2, 2, 1, 128, 192, 64, True),       # whole tiles, an odd number of blocks, grouped heads
+    (1, 3, 3, 129, 127, 128, False),     # one row into the second lane tile, one short of whole blocks
+    (1, 4, 2, 97, 353, 128, True),       # causal offset 256, one row into a 32-row block
+    (1, 4, 1, 321, 448, 64, True),       # group of four, offset 127
+    (1, 2, 2, 700, 96, 64, False),       # many query blocks over two key blocks
+]
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", CASES)
+@pytest.mark.parametrize("scale_sign", [1.0, -1.0])
+def test_edges_of_the_tiles(B, H, Hkv, Sq, Sk, D, causal, scale_sign):
+    scale = scale_sign / math.sqrt(D)
+    q, _, _, d_o = synth.random_inputs(700, B, H, Sq, D)
+    _, k, v, _ = synth.random_inputs(701, B, Hkv, Sk, D)
+    got = hp.run_cuda_ext(q, k, v, d_o, causal, scale, mgn.MODE_STRICT_F32)
+    ref = hp.run_oracle_ext(q, k, v, d_o, causal, scale)
+    hp.check_strict(got, ref, literal_max_abs=False, label=f"strict tensor-core {B,H,Hkv,Sq,Sk,D,causal} ")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_rows_of_very_different_magnitude(D):
+    """The parts carry f32's exponent range: a row a million times larger than its neighbours costs the others
+    nothing.  Errors are taken row by row.  O is normalised, so the whole-tensor gate holds for each row; P of
+    the backward is exp(s - LSE) with both near 64 (92 in the log2 domain), each good to about two units of
+    2^-24, so a row of dV is good to 2 * 2 * 92 * 2^-24 = 2.2e-5."""
+    B, H, S = 1, 2, 200
+    q, k, v, d_o = synth.random_inputs(710, B, H, S, D)
+    v[:, :, 5::7] *= 1e6
+    d_o[:, :, 3::5] *= 1e-6
+    # every query attends to its own key almost alone, so O rows keep the magnitude of their V rows
+    k.copy_(q / q.norm(dim=-1, keepdim=True) * 8.0)
+    got = hp.run_cuda_ext(q, k, v, d_o, False, 1.0, mgn.MODE_STRICT_F32)
+    ref = hp.run_oracle_ext(q, k, v, d_o, False, 1.0)
+    for name, bound in (("O", 1e-5), ("dV", 2.2e-5)):
+        for a, b in zip(got[name].reshape(-1, D), ref[name].reshape(-1, D)):
+            assert hp.rel_l2(a, b) < bound, name
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_inputs_that_are_not_finite(D):
+    """Infinities and overflowing scores give what f32 arithmetic gives: hi - hi parts must not meet as NaN."""
+    B, H, S = 1, 1, 150
+    q, k, v, _ = synth.random_inputs(720, B, H, S, D)
+    v[0, 0, 70, 3] = math.inf                    # column 3 of every row that sees key 70
+    v[0, 0, 20, 9] = 3.4028e38                   # rounds to infinity in 8 bits
+    q[0, 0, 100, :] = -1e25                      # scores of -1e50 against key 10: probability 0
+    k[0, 0, 10, :] = 1e25
+    q[0, 0, 101, 0] = math.nan
+    # finite scores elsewhere: only the large query meets the large key
+    q[0, 0, :, :] = torch.where(torch.arange(S)[:, None] >= 100, q[0, 0], torch.zeros(()))
+    c = [t.cuda() for t in (q, k, v)]
+    o = torch.empty_like(c[0])
+    lse = torch.empty(B, H, S, device="cuda")
+    mgn.mgn_attn_fwd(c[0], c[1], c[2], o, lse, True, 1.0 / math.sqrt(D), mgn.MODE_STRICT_F32)
+    mgn.mgn_attn_check()
+    # the same arithmetic in f32, row by row over the visible keys
+    for i in (0, 19, 20, 69, 70, 99, 100, 101):
+        s = (k[0, 0, :i + 1].double() @ q[0, 0, i].double() / math.sqrt(D)).float()
+        p = torch.softmax(s, 0)
+        ref = (p[:, None] * v[0, 0, :i + 1]).sum(0)
+        got = o[0, 0, i].cpu()
+        assert torch.equal(torch.isnan(got), torch.isnan(ref)), i
+        assert torch.equal(torch.isinf(got), torch.isinf(ref)), i
+        ok = torch.isfinite(ref)
+        assert torch.allclose(got[ok], ref[ok], rtol=1e-5, atol=1e-6), i
