@@ -36,6 +36,9 @@ inline double score_factor(float scale, int D) {
 
 // x * (c_hi + c_lo), rounded once.
 __device__ __forceinline__ float scaled(float x, float c_hi, float c_lo) { return fmaf(x, c_hi, x * c_lo); }
+__device__ __forceinline__ float4 scaled(float4 x, float c_hi, float c_lo) {
+    return make_float4(scaled(x.x, c_hi, c_lo), scaled(x.y, c_hi, c_lo), scaled(x.z, c_hi, c_lo), scaled(x.w, c_hi, c_lo));
+}
 
 // A pair of f32 (a in the low half) -> three packed bf16 pairs.
 __device__ __forceinline__ void split3(uint64_t x, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
@@ -55,19 +58,20 @@ template <int R> __host__ __device__ constexpr uint32_t part_bytes() { return R 
 template <int R> __host__ __device__ constexpr uint32_t block_bytes() { return 3 * R * 128; }     // a 64-column block
 template <int D, int R> __host__ __device__ constexpr uint32_t tile_bytes() { return D / 64 * 3 * R * 128; }
 
-// Eight consecutive f32 of a row -> the 16-byte pieces of the three parts of a split tile.
-template <int D, int R>
-__device__ __forceinline__ void store_unit(uint32_t dst, int r, int piece, const float4 x, const float4 y) {
-    uint32_t h[4], m[4], l[4];
+// Four consecutive f32 of a row -> the 8-byte pieces of the three parts of a split tile of R rows.  `at` is where
+// the hi piece goes.
+template <int R>
+__device__ __forceinline__ uint32_t quad_offset(int r, int quad) {
+    return (quad >> 4) * block_bytes<R>() + r * 128 + ((((quad >> 1) & 7) ^ (r & 7)) << 4) + (quad & 1) * 8;
+}
+template <int R>
+__device__ __forceinline__ void store_quad(uint32_t at, const float4 x) {
+    uint32_t h[2], m[2], l[2];
     split3(f2_pack(x.x, x.y), h[0], m[0], l[0]);
     split3(f2_pack(x.z, x.w), h[1], m[1], l[1]);
-    split3(f2_pack(y.x, y.y), h[2], m[2], l[2]);
-    split3(f2_pack(y.z, y.w), h[3], m[3], l[3]);
-    const uint32_t a = dst + (piece >> 3) * block_bytes<R>() + r * 128 + (((piece & 7) ^ (r & 7)) << 4);
-    constexpr uint32_t PART = part_bytes<R>();
-    sts128(a, h[0], h[1], h[2], h[3]);
-    sts128(a + PART, m[0], m[1], m[2], m[3]);
-    sts128(a + 2 * PART, l[0], l[1], l[2], l[3]);
+    sts64(at, h[0], h[1]);
+    sts64(at + part_bytes<R>(), m[0], m[1]);
+    sts64(at + 2 * part_bytes<R>(), l[0], l[1]);
 }
 
 // A team of kTeam threads turns a stream of R x D f32 tiles into split operand tiles, 2048 values at a time
@@ -95,8 +99,7 @@ struct Converter {
         : row(t / QUADS), quad(t % QUADS), c_hi(hi), c_lo(lo) {
 #pragma unroll
         for (int k = 0; k < NQ; ++k) {
-            const int r = row + k * STEP;
-            off[k] = (quad >> 4) * block_bytes<R>() + r * 128 + ((((quad >> 1) & 7) ^ (r & 7)) << 4) + (quad & 1) * 8;
+            off[k] = quad_offset<R>(row + k * STEP, quad);
         }
     }
     // Converts tiles 0 .. n-1.  src(i, rows) gives the first row of tile i and how many rows exist from there;
@@ -127,15 +130,8 @@ struct Converter {
 #pragma unroll
             for (int k = 0; k < NQ; ++k) {
                 if (row + k * STEP < SLOT_ROWS) {
-                    uint32_t h[2], m[2], l[2];
-                    if constexpr (SCALED)
-                        buf[k] = make_float4(scaled(buf[k].x, c_hi, c_lo), scaled(buf[k].y, c_hi, c_lo),
-                                             scaled(buf[k].z, c_hi, c_lo), scaled(buf[k].w, c_hi, c_lo));
-                    split3(f2_pack(buf[k].x, buf[k].y), h[0], m[0], l[0]);
-                    split3(f2_pack(buf[k].z, buf[k].w), h[1], m[1], l[1]);
-                    sts64(d + off[k], h[0], h[1]);
-                    sts64(d + off[k] + part_bytes<R>(), m[0], m[1]);
-                    sts64(d + off[k] + 2 * part_bytes<R>(), l[0], l[1]);
+                    if constexpr (SCALED) buf[k] = scaled(buf[k], c_hi, c_lo);
+                    store_quad<R>(d + off[k], buf[k]);
                 }
                 load(k);
             }
@@ -150,23 +146,68 @@ struct Converter {
     }
 };
 
-// Splits `n32` groups of 32 consecutive f32 values of one row (null: zeros), times c_hi + c_lo, into tensor
-// memory: part a goes to columns t + a * part_cols.
-__device__ __forceinline__ void split_row_to_tmem(uint32_t t, int part_cols, const float* src, int n32, float c_hi, float c_lo) {
-#pragma unroll 1
-    for (int c = 0; c < n32; ++c) {
-        uint32_t h[16], m[16], l[16];
+// The 128 rows of D f32 that a CTA owns, read and written by its 256 element-wise threads (t) as 16-byte quads
+// in row order: a thread per row instead touches 32 lines with each load or store, which alone took 4000
+// clocks per tensor and CTA (dK+dV of a 197-token head: 10000 clocks to the first split tile, 5500 after the
+// last product, of 41000).
+template <int D>
+struct OwnRows {
+    static constexpr int NQ = 128 * D / 4 / 256, PITCH = D * 4 + 16;     // bytes of a row in the exchange tile
+    float4 q[NQ];
+    // src: the first row, of which `rows` exist
+    __device__ __forceinline__ void load(const float* src, int rows, int t) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float4 x = src ? __ldg(reinterpret_cast<const float4*>(src + 32 * c) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-            split3(f2_pack(scaled(x.x, c_hi, c_lo), scaled(x.y, c_hi, c_lo)), h[2 * e], m[2 * e], l[2 * e]);
-            split3(f2_pack(scaled(x.z, c_hi, c_lo), scaled(x.w, c_hi, c_lo)), h[2 * e + 1], m[2 * e + 1], l[2 * e + 1]);
+        for (int k = 0; k < NQ; ++k) {
+            const int u = t + 256 * k, r = u / (D / 4), c = u % (D / 4);
+            q[k] = r < rows ? __ldg(reinterpret_cast<const float4*>(src + r * D + 4 * c)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        tmem_st16(t + 16 * c, h);
-        tmem_st16(t + part_cols + 16 * c, m);
-        tmem_st16(t + 2 * part_cols + 16 * c, l);
     }
-}
+    __device__ __forceinline__ void scale(float c_hi, float c_lo) {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) q[k] = scaled(q[k], c_hi, c_lo);
+    }
+    // into a split tile of 128 rows
+    __device__ __forceinline__ void to_tile(uint32_t tile, int t) const {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            const int u = t + 256 * k;
+            store_quad<128>(tile + quad_offset<128>(u / (D / 4), u % (D / 4)), q[k]);
+        }
+    }
+    // into the exchange tile
+    __device__ __forceinline__ void to_exchange(uint32_t ex, int t) const {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            const int u = t + 256 * k;
+            sts128f(ex + (u / (D / 4)) * PITCH + (u % (D / 4)) * 16, q[k].x, q[k].y, q[k].z, q[k].w);
+        }
+    }
+    // from the exchange tile to global memory
+    static __device__ __forceinline__ void store(float* dst, int rows, uint32_t ex, int t) {
+#pragma unroll 4
+        for (int k = 0; k < NQ; ++k) {
+            const int u = t + 256 * k, r = u / (D / 4), c = u % (D / 4);
+            if (r < rows) *reinterpret_cast<float4*>(dst + r * D + 4 * c) = lds128(ex + r * PITCH + c * 16);
+        }
+    }
+    // half h of row r of the exchange tile, split into tensor memory: part a at columns t + a * D / 2
+    static __device__ __forceinline__ void half_row_to_tmem(uint32_t ex, int r, int h, uint32_t tm) {
+#pragma unroll 1
+        for (int c = 0; c < D / 64; ++c) {
+            uint32_t p0[16], p1[16], p2[16];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 x = lds128(ex + r * PITCH + h * (D * 2) + c * 128 + e * 16);
+                split3(f2_pack(x.x, x.y), p0[2 * e], p1[2 * e], p2[2 * e]);
+                split3(f2_pack(x.z, x.w), p0[2 * e + 1], p1[2 * e + 1], p2[2 * e + 1]);
+            }
+            const uint32_t at = tm + h * (D / 4) + 16 * c;
+            tmem_st16(at, p0);
+            tmem_st16(at + D / 2, p1);
+            tmem_st16(at + D, p2);
+        }
+    }
+};
 
 // The partial products as issued.  A term: part of A, first part of B, how many adjacent parts of B it runs
 // against, and the column set that its first one goes to.

@@ -57,22 +57,6 @@ struct KvCfg {
     enum { S_GO = 0, P_GO = 2, V_GO = 4, K_GO = 6, S_DONE = 7, P_DONE = 8, V_DONE = 9, K_DONE = 10, KV = 12, COUNT = 13 };
 };
 
-// Splits this thread's half of row r (null: zeros), times c_hi + c_lo, into a 128-row operand tile.
-template <int D>
-__device__ __forceinline__ void split_row_to_tile(uint32_t tile, int r, int h, const float* src, float c_hi, float c_lo) {
-#pragma unroll 1
-    for (int u = 0; u < D / 16; ++u) {
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-        if (src) {
-            x = __ldg(reinterpret_cast<const float4*>(src + 8 * u));
-            y = __ldg(reinterpret_cast<const float4*>(src + 8 * u) + 1);
-        }
-        x = make_float4(scaled(x.x, c_hi, c_lo), scaled(x.y, c_hi, c_lo), scaled(x.z, c_hi, c_lo), scaled(x.w, c_hi, c_lo));
-        y = make_float4(scaled(y.x, c_hi, c_lo), scaled(y.y, c_hi, c_lo), scaled(y.z, c_hi, c_lo), scaled(y.w, c_hi, c_lo));
-        store_unit<D, 128>(tile, r, h * (D / 16) + u, x, y);
-    }
-}
-
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
@@ -89,7 +73,6 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     auto bar = [&](int i) { return bars + 8u * i; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_launch_dependents();                               // the dQ kernel may fill SMs as this one drains
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
 
     // First key blocks first: under a causal mask they see the most queries.
     const int kb = static_cast<int>(blockIdx.x) / BHkv, bhk = static_cast<int>(blockIdx.x) % BHkv;
@@ -115,10 +98,16 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     }
     __syncwarp();
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    if (tid == 32) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = lds32u(tmem_slot);
+    if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tmem, 512);
+        return;
+    }
 
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
@@ -224,14 +213,23 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
         const uint32_t tl = tmem + lane_base;
         const int j = j0 + r;
-        const bool row_ok = j < Sk;
-        const size_t row_at = (static_cast<size_t>(bhk) * Sk + j) * D + h * (D / 2);
-        const float* krow = row_ok ? K + row_at : nullptr;
-        const float* vrow = row_ok ? V + row_at : nullptr;
-        split_row_to_tile<D>(base + C::OFF_K, r, h, krow, 1.f, 0.f);
-        if constexpr (C::V_TMEM) split_row_to_tmem(tl + C::TM_V + h * (D / 4), D / 2, vrow, D / 64, 1.f, 0.f);
-        else split_row_to_tile<D>(base + C::OFF_V, r, h, vrow, 1.f, 0.f);
-        fence_proxy_async_smem();
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bhk) * Sk + j0) * D;
+        {
+            OwnRows<D> kr, vr;
+            vr.load(V + own_at, Sk - j0, t);
+            kr.load(K + own_at, Sk - j0, t);
+            if constexpr (C::V_TMEM) {                     // by way of K's place
+                vr.to_exchange(base + C::OFF_K, t);
+                named_bar_sync(1, kCompute);
+                OwnRows<D>::half_row_to_tmem(base + C::OFF_K, r, h, tl + C::TM_V);
+                named_bar_sync(1, kCompute);
+            } else {
+                vr.to_tile(base + C::OFF_V, t);
+            }
+            kr.to_tile(base + C::OFF_K, t);
+            fence_proxy_async_smem();
+        }
         tmem_st_wait();
         tc_fence_before();
         mbar_arrive(bar(C::KV));
@@ -337,13 +335,18 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         mbar_wait(bar(C::K_DONE + ((n_blk - 1) & 1)), ((n_blk - 1) >> 1) & 1, status);
         tc_fence_after();
         add_result(C::TM_ZK, accK);
-        if (row_ok) {
+        // every product has completed: the operand tiles are dead
+        constexpr uint32_t EX = 128 * OwnRows<D>::PITCH;
+        static_assert(2 * EX <= C::OFF_STAT, "two exchange tiles");
+        const uint32_t ex = base + r * OwnRows<D>::PITCH + h * (D * 2);
 #pragma unroll
-            for (int d = 0; d < D / 2; d += 4) {
-                *reinterpret_cast<float4*>(dK + row_at + d) = make_float4(accK[d] * dk_factor, accK[d + 1] * dk_factor, accK[d + 2] * dk_factor, accK[d + 3] * dk_factor);
-                *reinterpret_cast<float4*>(dV + row_at + d) = make_float4(accV[d], accV[d + 1], accV[d + 2], accV[d + 3]);
-            }
+        for (int d = 0; d < D / 2; d += 4) {
+            sts128f(ex + d * 4, accK[d] * dk_factor, accK[d + 1] * dk_factor, accK[d + 2] * dk_factor, accK[d + 3] * dk_factor);
+            sts128f(ex + EX + d * 4, accV[d], accV[d + 1], accV[d + 2], accV[d + 3]);
         }
+        named_bar_sync(1, kCompute);
+        OwnRows<D>::store(dK + own_at, Sk - j0, base, t);
+        OwnRows<D>::store(dV + own_at, Sk - j0, base + EX, t);
     }
 
     tc_fence_before();
@@ -387,7 +390,6 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
 
     // Heaviest (last) query tiles first when causal.
     const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / BH;
@@ -412,10 +414,17 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     }
     __syncwarp();
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    if (tid == 32) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = lds32u(tmem_slot);
+    if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tmem, 512);
+        pdl_wait();
+        return;
+    }
 
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
@@ -488,14 +497,25 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
         const uint32_t tl = tmem + (static_cast<uint32_t>(r & ~31) << 16);
         const int i = i0 + r;
         const bool row_ok = i < Sq;
-        const size_t row_at = (static_cast<size_t>(bh) * Sq + i) * D + h * (D / 2);
-        const float* qrow = row_ok ? Q + row_at : nullptr;
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
         mbar_arrive(bar(C::P_GO));                         // block 0 has no dP before it
-        const float* orow = row_ok ? dO + row_at : nullptr;
-        split_row_to_tile<D>(base + C::OFF_Q, r, h, qrow, c_hi, c_lo);
-        if constexpr (C::DO_TMEM) split_row_to_tmem(tl + C::TM_DO + h * (D / 4), D / 2, orow, D / 64, 1.f, 0.f);
-        else split_row_to_tile<D>(base + C::OFF_DO, r, h, orow, 1.f, 0.f);
-        fence_proxy_async_smem();
+        {
+            OwnRows<D> qr, orr;
+            orr.load(dO + own_at, Sq - i0, t);
+            qr.load(Q + own_at, Sq - i0, t);
+            if constexpr (C::DO_TMEM) {                    // by way of Q's place
+                orr.to_exchange(base + C::OFF_Q, t);
+                named_bar_sync(1, kCompute);
+                OwnRows<D>::half_row_to_tmem(base + C::OFF_Q, r, h, tl + C::TM_DO);
+                named_bar_sync(1, kCompute);
+            } else {
+                orr.to_tile(base + C::OFF_DO, t);
+            }
+            qr.scale(c_hi, c_lo);
+            qr.to_tile(base + C::OFF_Q, t);
+            fence_proxy_async_smem();
+        }
         tmem_st_wait();
         tc_fence_before();
         mbar_arrive(bar(C::QDO));
@@ -560,11 +580,13 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
             mbar_arrive(bar(C::Q_GO));
         }
         add_result(n_blk - 1);
-        if (row_ok) {
+        // every product has completed: the operand tiles are dead
+        const uint32_t ex = base + r * OwnRows<D>::PITCH + h * (D * 2);
 #pragma unroll
-            for (int d = 0; d < D / 2; d += 4)
-                *reinterpret_cast<float4*>(dQ + row_at + d) = make_float4(acc[d] * scale, acc[d + 1] * scale, acc[d + 2] * scale, acc[d + 3] * scale);
-        }
+        for (int d = 0; d < D / 2; d += 4)
+            sts128f(ex + d * 4, acc[d] * scale, acc[d + 1] * scale, acc[d + 2] * scale, acc[d + 3] * scale);
+        named_bar_sync(1, kCompute);
+        OwnRows<D>::store(dQ + own_at, Sq - i0, base, t);
     }
 
     tc_fence_before();

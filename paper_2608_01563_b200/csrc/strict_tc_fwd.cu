@@ -32,10 +32,9 @@ struct Cfg {
     static constexpr int NST = 2;                               // stages of K and of V: even and odd blocks
     static constexpr int R = D == 64 ? 64 : 32;                 // keys of a block
     static constexpr int STAGE = tile_bytes<D, R>();
-    static constexpr int OFF_K = 0, OFF_V = NST * STAGE, OFF_BAR = 2 * NST * STAGE;
+    static constexpr int OFF_K = 0, OFF_V = NST * STAGE, OFF_EX = 2 * NST * STAGE,
+                         OFF_BAR = OFF_EX + 128 * OwnRows<D>::PITCH + 2 * 128 * 4;      // exchange tile, row statistics
     static constexpr int SMEM = OFF_BAR + 512 + 1024;
-    static constexpr int PITCH = D + 1;                         // floats per row of the epilogue's exchange tile
-    static_assert(kBM * PITCH * 4 + kBM * 8 <= OFF_BAR, "the exchange tile lies over the K and V stages");
     static_assert(SMEM <= 232448, "shared memory budget");
     static constexpr int ST = D == 64 ? 2 : 3, STO = D == 64 ? 2 : 1;       // column sets of scores, of results
     static constexpr uint32_t X = x_cols<R, ST>();
@@ -82,7 +81,6 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
 
     // Heaviest (last) query tiles first when causal.
     const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / BH;
@@ -104,10 +102,16 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     }
     __syncwarp();
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    if (tid == 32) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = lds32u(tmem_slot);
+    if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tmem, 512);
+        return;
+    }
 
     if (warp < 8) {
         reg_dealloc<56>();
@@ -172,9 +176,17 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         const uint32_t tX = tmem + lane_base + C::TM_X + w * C::X, tO = tmem + lane_base + C::TM_O;
         const int i = i0 + r;
         const bool row_ok = i < Sq;
-        const float* qrow = Q + (static_cast<size_t>(bh) * Sq + i) * D;
-        split_row_to_tmem(tmem + lane_base + C::TM_Q + w * (D / 4), D / 2, row_ok ? qrow + w * (D / 2) : nullptr, D / 64,
-                          c_hi, c_lo);
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
+        const uint32_t ex = base + C::OFF_EX;
+        {
+            OwnRows<D> qr;
+            qr.load(Q + own_at, Sq - i0, t);
+            qr.scale(c_hi, c_lo);
+            qr.to_exchange(ex, t);
+            named_bar_sync(1, 256);
+            OwnRows<D>::half_row_to_tmem(ex, r, w, tmem + lane_base + C::TM_Q);
+        }
         tmem_st_wait();
         tc_fence_before();
         mbar_arrive(bar(C::QFULL));
@@ -258,20 +270,18 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
             mbar_arrive(bar(C::PGO + (w ^ 1)));                // the next block's product may overwrite it
         }
 
-        // ---- the two halves of the keys meet in shared memory (the K and V stages are dead)
-        float* tile = reinterpret_cast<float*>(smem);
-        float* stat = tile + kBM * C::PITCH;
-        float* row = tile + r * C::PITCH;
-        named_bar_sync(1, 256);
+        // ---- the two halves of the keys meet in the exchange tile
+        const uint32_t row = ex + r * OwnRows<D>::PITCH, stat = ex + 128 * OwnRows<D>::PITCH + r * 8;
+        named_bar_sync(1, 256);                                // both warpgroups have read their Q rows from it
         if (w == 1) {
 #pragma unroll
-            for (int d = 0; d < D; ++d) row[d] = acc[d];
-            stat[r] = m;
-            stat[kBM + r] = l;
+            for (int d = 0; d < D; d += 4) sts128f(row + d * 4, acc[d], acc[d + 1], acc[d + 2], acc[d + 3]);
+            sts32(stat, m);
+            sts32(stat + 4, l);
         }
         named_bar_sync(1, 256);
         if (w == 0) {
-            const float m1 = stat[r], l1 = stat[kBM + r];
+            const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
             const float mm = fmaxf(m, m1);
             const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
             const float lt = fmaf(l, a0, l1 * a1);
@@ -281,21 +291,23 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
             float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, lg2(lt) * kLn2));
             float bad = 0.f;                                   // NaN once an output is not finite
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                const float x = fmaf(acc[d], b0, row[d] * b1);
-                row[d] = x;
-                bad = fmaf(x, 0.f, bad);
+            for (int d = 0; d < D; d += 4) {
+                float4 x = lds128(row + d * 4);
+                x = make_float4(fmaf(acc[d], b0, x.x * b1), fmaf(acc[d + 1], b0, x.y * b1), fmaf(acc[d + 2], b0, x.z * b1),
+                                fmaf(acc[d + 3], b0, x.w * b1));
+                sts128f(row + d * 4, x.x, x.y, x.z, x.w);
+                bad = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, bad))));
             }
             if (row_ok) {
-                if (bad != 0.f || !(fabsf(lse) < INFINITY)) lse = plain_row<D>(qrow, K + static_cast<size_t>(bhk) * Sk * D, V + static_cast<size_t>(bhk) * Sk * D, vis,
-                                       c_hi, row);
+                if (bad != 0.f || !(fabsf(lse) < INFINITY))
+                    lse = plain_row<D>(Q + own_at + static_cast<size_t>(r) * D, K + static_cast<size_t>(bhk) * Sk * D,
+                                       V + static_cast<size_t>(bhk) * Sk * D, vis, c_hi,
+                                       reinterpret_cast<float*>(smem + C::OFF_EX + r * OwnRows<D>::PITCH));
                 LSE[static_cast<size_t>(bh) * Sq + i] = lse;
             }
         }
         named_bar_sync(1, 256);
-        float* og = O + (static_cast<size_t>(bh) * Sq + i0) * D;
-        const int n_rows = min(kBM, Sq - i0);
-        for (int x = tid - 256; x < n_rows * D; x += 256) og[x] = tile[(x / D) * C::PITCH + x % D];
+        OwnRows<D>::store(O + own_at, Sq - i0, ex, t);
     }
 
     tc_fence_before();
