@@ -5,15 +5,17 @@
 // here, which makes seven matrix products per tile pair instead of the fused kernel's five.
 //
 // One CTA owns one 128-row query tile of one head, keeps its Q and dO tiles in shared memory and
-// streams the 128-key blocks of K and V through a two-stage ring.  Per key block:
+// streams the 128-key blocks of K (three stages) and V (two).  Per key block:
 //   MMA  S  = Q K^T   -> tensor memory S        MMA  dP = dO V^T -> tensor memory P
 //   compute (256 threads, two per query row, 64 key columns each):
 //        P = exp2(S c - LSE), dS = P (dP - delta) -> bf16, written over S (the A operand of the next product)
 //   MMA  dQ += dS K   (A from tensor memory, K as the MN-major shared-memory operand)
-// The products of one block and the arithmetic of that block alternate (one buffer each for S and
-// dP): this pass favours simplicity over overlap.  Epilogue: dQ * scale -> bf16 -> shared memory
-// (the dead Q tile) -> TMA store.
-// Warp roles (384 threads): warp 0 TMA producer, warp 1 MMA issuer, warps 4-11 compute.
+// S has two regions: S(n+1) and dQ(n-1) run while the arithmetic of block n does, and dP(n+1) follows
+// as soon as dP(n) has been read, so a block costs its arithmetic; with one S region the products and the
+// arithmetic took turns.  (4,32,1024,128) causal, forward and deterministic backward: 261 -> 253 us.
+// Epilogue: dQ * scale -> bf16 -> shared memory (the dead Q tile) -> TMA store.
+// Warp roles (384 threads): warp 0 TMA producer, warps 1 and 2 one MMA-issuing lane each (S and dP; dQ),
+// warps 4-11 compute.
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -34,16 +36,18 @@ struct Cfg {
     static constexpr int CHUNK_BYTES = BLK * 128;
     static constexpr int OFF_Q = 0;
     static constexpr int OFF_DO = OFF_Q + TILE_BYTES;
-    static constexpr int OFF_K = OFF_DO + TILE_BYTES;          // two stages
-    static constexpr int OFF_V = OFF_K + 2 * TILE_BYTES;       // two stages
+    static constexpr int OFF_K = OFF_DO + TILE_BYTES;          // three stages: K is needed again by dQ
+    static constexpr int OFF_V = OFF_K + 3 * TILE_BYTES;       // two stages
     static constexpr int OFF_BAR = OFF_V + 2 * TILE_BYTES;
     static constexpr int SMEM = OFF_BAR + 256 + 1024;
     static_assert(SMEM <= 232448, "shared memory budget");
-    static constexpr uint32_t TM_S = 0, TM_P = 128, TM_DQ = 256, TM_COLS = 512;
+    static constexpr uint32_t TM_S = 0, TM_P = 256, TM_DQ = 384, TM_COLS = 512;   // S: two regions
 };
 
-enum { B_Q = 0, B_KFULL = 1, B_KEMPTY = 3, B_VFULL = 5, B_VEMPTY = 7, B_SPFULL = 9, B_DSFULL = 10, B_DQFULL = 11,
-       B_COUNT = 12 };
+// Conditions of the products and their completion; pairs are indexed by the parity of the key block.
+//   B_KFULL[3]: K landed   B_SFREE[2]: dS of two blocks back read   B_PGO[2]: V landed and the last dP read
+//   B_QGO: dS written      B_SDONE[2], B_PDONE: S, dP complete      B_QDONE[3]: dQ complete (K, V, dS free)
+enum { B_Q = 0, B_KFULL = 1, B_SFREE = 4, B_PGO = 6, B_QGO = 8, B_SDONE = 9, B_PDONE = 11, B_QDONE = 12, B_COUNT = 15 };
 
 
 template <int D>
@@ -75,7 +79,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const float c2 = scale * kLog2e;
 
     if (tid == 0) {
-        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), i == B_DSFULL ? 256u : 1u);
+        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), i == B_QGO ? 256u : (i == B_PGO || i == B_PGO + 1) ? 257u : 1u);
         fence_mbar_init();
     }
     __syncwarp();
@@ -96,55 +100,63 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 tma_load_3d(sdO + ch * C::CHUNK_BYTES, &tmdO, bar(B_Q), ch * 64, i0, bh);
             }
             for (int n = 0; n < n_kb; ++n) {
-                const int st = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                mbar_wait(bar(B_KEMPTY + st), ph ^ 1, status);
-                mbar_arrive_expect_tx(bar(B_KFULL + st), C::TILE_BYTES);
+                const int sk = n % 3, sv = n & 1;
+                if (n >= 3) mbar_wait(bar(B_QDONE + sk), (n / 3 - 1) & 1, status);
+                mbar_arrive_expect_tx(bar(B_KFULL + sk), C::TILE_BYTES);
 #pragma unroll
                 for (int ch = 0; ch < C::NCH; ++ch)
-                    tma_load_3d(sK + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmK, bar(B_KFULL + st), ch * 64, n * BLK, bhk);
-                mbar_wait(bar(B_VEMPTY + st), ph ^ 1, status);
-                mbar_arrive_expect_tx(bar(B_VFULL + st), C::TILE_BYTES);
+                    tma_load_3d(sK + sk * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmK, bar(B_KFULL + sk), ch * 64, n * BLK, bhk);
+                // dP(n-2), the last reader of this V stage, is complete when the dS formed from it has been used
+                if (n >= 2) mbar_wait(bar(B_QDONE + (n - 2) % 3), ((n - 2) / 3) & 1, status);
+                mbar_arrive_expect_tx(bar(B_PGO + sv), C::TILE_BYTES);
 #pragma unroll
                 for (int ch = 0; ch < C::NCH; ++ch)
-                    tma_load_3d(sV + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmV, bar(B_VFULL + st), ch * 64, n * BLK, bhk);
+                    tma_load_3d(sV + sv * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmV, bar(B_PGO + sv), ch * 64, n * BLK, bhk);
             }
         } else if (warp == 1 && lane == 0) {
-            // ------------------------------------------------------------------ MMA issuer
-            constexpr uint32_t idesc_s = umma_idesc_bf16(BLK, BLK, false, false);    // S, dP: both operands K-major
-            constexpr uint32_t idesc_q = umma_idesc_bf16(BLK, D, false, true);       // dQ: A from tensor memory, B MN-major
+            // ------------------------------------------------------------------ S and dP
+            constexpr uint32_t idesc_s = umma_idesc_bf16(BLK, BLK, false, false);    // both operands K-major
             const uint64_t dQd = umma_smem_desc(sQ, 16, 1024), dOd = umma_smem_desc(sdO, 16, 1024);
             const uint64_t dK0 = umma_smem_desc(sK, 16, 1024), dV0 = umma_smem_desc(sV, 16, 1024);
-            const uint64_t mK0 = umma_smem_desc(sK, C::CHUNK_BYTES, 1024);
-            const uint32_t tS = tmem + C::TM_S, tP = tmem + C::TM_P, tDQ = tmem + C::TM_DQ;
+            const uint32_t tP = tmem + C::TM_P;
             auto koff = [](int kk) { return static_cast<uint64_t>(((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32) >> 4); };
+            mbar_arrive(bar(B_SFREE));
+            mbar_arrive(bar(B_SFREE + 1));
             mbar_wait(bar(B_Q), 0, status);
             for (int n = 0; n < n_kb; ++n) {
-                const int st = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                const uint64_t stoff = static_cast<uint64_t>((st * C::TILE_BYTES) >> 4);
-                // S(n): its region held dS(n-1), read by the dQ product issued just before (same thread: in order)
-                mbar_wait(bar(B_KFULL + st), ph, status);
+                const int w = n & 1;
+                const uint32_t tS = tmem + C::TM_S + BLK * w;
+                const uint64_t kst = dK0 + static_cast<uint64_t>(((n % 3) * C::TILE_BYTES) >> 4);
+                const uint64_t vst = dV0 + static_cast<uint64_t>((w * C::TILE_BYTES) >> 4);
+                mbar_wait(bar(B_KFULL + n % 3), (n / 3) & 1, status);
+                mbar_wait(bar(B_SFREE + w), (n >> 1) & 1, status);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tS, dQd + koff(kk), dK0 + stoff + koff(kk), idesc_s, kk > 0);
-                // dP(n): the compute warps finished reading dP(n-1) before they signalled dS(n-1)
-                mbar_wait(bar(B_VFULL + st), ph, status);
+                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tS, dQd + koff(kk), kst + koff(kk), idesc_s, kk > 0);
+                umma_commit(bar(B_SDONE + w));
+                mbar_wait(bar(B_PGO + w), (n >> 1) & 1, status);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tP, dOd + koff(kk), dV0 + stoff + koff(kk), idesc_s, kk > 0);
-                umma_commit(bar(B_SPFULL));
-                umma_commit(bar(B_VEMPTY + st));
-                // dQ += dS(n) K(n)
-                mbar_wait(bar(B_DSFULL), n & 1, status);
+                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tP, dOd + koff(kk), vst + koff(kk), idesc_s, kk > 0);
+                umma_commit(bar(B_PDONE));
+            }
+        } else if (warp == 2 && lane == 0) {
+            // ------------------------------------------------------------------ dQ
+            constexpr uint32_t idesc_q = umma_idesc_bf16(BLK, D, false, true);       // A from tensor memory, B MN-major
+            const uint64_t mK0 = umma_smem_desc(sK, C::CHUNK_BYTES, 1024);
+            const uint32_t tDQ = tmem + C::TM_DQ;
+            for (int n = 0; n < n_kb; ++n) {
+                const uint32_t tS = tmem + C::TM_S + BLK * (n & 1);
+                const uint64_t kst = mK0 + static_cast<uint64_t>(((n % 3) * C::TILE_BYTES) >> 4);
+                mbar_wait(bar(B_QGO), n & 1, status);
                 tc_fence_after();
 #pragma unroll
                 for (int kk = 0; kk < BLK / 16; ++kk)
-                    umma_ts(tDQ, tS + (kk >> 2) * 64 + (kk & 3) * 8, mK0 + stoff + static_cast<uint64_t>((kk * 2048) >> 4),
-                            idesc_q, (kk > 0 || n > 0) ? 1u : 0u);
-                umma_commit(bar(B_KEMPTY + st));
+                    umma_ts(tDQ, tS + (kk >> 2) * 64 + (kk & 3) * 8, kst + static_cast<uint64_t>((kk * 2048) >> 4), idesc_q,
+                            (kk > 0 || n > 0) ? 1u : 0u);
+                umma_commit(bar(B_QDONE + n % 3));
+                umma_commit(bar(B_SFREE + (n & 1)));
             }
-            umma_commit(bar(B_DQFULL));
         }
         __syncwarp();
     } else {
@@ -153,7 +165,8 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const int h = (warp - 4) >> 2;                     // which 64 key columns of every block
         const int r = (tid - 128) & 127;                   // row within the tile = tensor-memory lane
         const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
-        const uint32_t tS = tmem + lane_base + C::TM_S + 64 * h, tP = tmem + lane_base + C::TM_P + 64 * h;
+        const uint32_t tS0 = tmem + lane_base + C::TM_S + 64 * h, tP = tmem + lane_base + C::TM_P + 64 * h;
+        mbar_arrive(bar(B_PGO));                           // block 0 has no dP before it
         const int i = i0 + r;
         const bool row_ok = i < dm.Sq;
         const float lse2 = row_ok ? LSE[static_cast<size_t>(bh) * dm.Sq + i] * kLog2e : INFINITY;   // P = 0 past the end
@@ -163,40 +176,45 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const int j0 = n * BLK + 64 * h;
             const bool masked = causal && (j0 + 63 > i0 + dm.off);
             const int jmax = i + dm.off - j0;              // causal: columns c <= jmax of this half are visible
-            mbar_wait(bar(B_SPFULL), n & 1, status);
+            const uint32_t tS = tS0 + BLK * (n & 1);
+            mbar_wait(bar(B_SDONE + (n & 1)), (n >> 1) & 1, status);
             tc_fence_after();
-            uint32_t pk[32];
+            float p[64];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                uint32_t s[32], dp[32];
+                uint32_t s[32];
                 tmem_ld32(tS + 32 * c, s);
-                tmem_ld32(tP + 32 * c, dp);
                 tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    float p0 = ex2(fmaf(__uint_as_float(s[e]), c2, -lse2));
-                    float p1 = ex2(fmaf(__uint_as_float(s[e + 1]), c2, -lse2));
-                    if (masked) {
-                        if (32 * c + e > jmax) p0 = 0.f;
-                        if (32 * c + e + 1 > jmax) p1 = 0.f;
-                    }
-                    pk[16 * c + e / 2] = pack_bf16(p0 * (__uint_as_float(dp[e]) - dl), p1 * (__uint_as_float(dp[e + 1]) - dl));
+                for (int e = 0; e < 32; ++e) {
+                    p[32 * c + e] = ex2(fmaf(__uint_as_float(s[e]), c2, -lse2));
+                    if (masked && 32 * c + e > jmax) p[32 * c + e] = 0.f;
                 }
             }
+            mbar_wait(bar(B_PDONE), n & 1, status);
+            tc_fence_after();
+            uint32_t dp[2][32];
+            tmem_ld32(tP, dp[0]);
+            tmem_ld32(tP + 32, dp[1]);
+            tmem_ld_wait();
+            tc_fence_before();
+            mbar_arrive(bar(B_PGO + ((n + 1) & 1)));       // dP of the next block may overwrite it
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 uint32_t u[16];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) u[e] = pk[16 * c + e];
+                for (int e = 0; e < 32; e += 2)
+                    u[e / 2] = pack_bf16(p[32 * c + e] * (__uint_as_float(dp[c][e]) - dl),
+                                         p[32 * c + e + 1] * (__uint_as_float(dp[c][e + 1]) - dl));
                 tmem_st16(tS + 16 * c, u);                 // dS of this half: packed columns [64h, 64h + 32)
             }
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(bar(B_DSFULL));
+            mbar_arrive(bar(B_QGO));
         }
 
         // ---- epilogue: dQ * scale -> bf16 -> shared memory (the Q tile is dead) -> TMA store
-        mbar_wait(bar(B_DQFULL), 0, status);
+        mbar_wait(bar(B_QDONE + (n_kb - 1) % 3), ((n_kb - 1) / 3) & 1, status);
         tc_fence_after();
         {
             const uint32_t tDQ = tmem + lane_base + C::TM_DQ + (D / 2) * h;
