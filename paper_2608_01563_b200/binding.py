@@ -101,9 +101,16 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# The current stream's handle without a torch.cuda.Stream object around it: 0.3 us instead of 3.0 us, where a
+# whole small call takes 10 us of host time.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream: Optional[int]) -> Optional[int]:
     if stream is not None:
         return stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch._C._cuda_getDevice())
     return torch.cuda.current_stream().cuda_stream
 
 
