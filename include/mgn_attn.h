@@ -255,8 +255,8 @@ int mgn_attn_profile_events(void* before_main, void* after_main);
 int mgn_attn_fast_item_order(int order);
 
 /*
- * Which tile shapes the strict-mode kernels run a problem with (host-only query; library plumbing,
- * the paper has no counterpart).  The strict kernels cover the score matrix with tiles of
+ * Which tile shapes the strict-mode FFMA kernels run a problem of these lengths with, where they run it
+ * and it has tiles enough to fill the GPU (host-only query; library plumbing, the paper has no counterpart).  The strict kernels cover the score matrix with tiles of
  * fwd_bm x fwd_bn (forward) and bwd_bm x bwd_bn (backward) query rows x keys, and execute whole
  * tiles; for short sequences whose lengths are far from tile multiples (197 tokens of a vision
  * transformer, Section 4.1 workload table) a second shape with less padding is chosen.  Writes the

@@ -208,18 +208,25 @@ int mgn_attn_bwd_ext(const void* q, const void* k, const void* v, const void* o,
     unsigned* sched = fast ? reinterpret_cast<unsigned*>(static_cast<char*>(workspace) + ws_delta_bytes(rows)) : nullptr;
     float* dq_acc = fast ? reinterpret_cast<float*>(static_cast<char*>(workspace) + ws_delta_bytes(rows) + kSchedBytes)
                          : static_cast<float*>(dq);
-    // a single key block (fast), the tensor-core kernels (strict): nothing accumulates in memory
-    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : mgn::strict_bwd_on_tensor_cores(p);
+    // a single key block (fast), the tensor-core kernels with whole key loops (strict): nothing accumulates in memory
+    const bool strict_tc = !fast && mgn::strict_on_tensor_cores(p);
+    const int dq_splits = mgn::strict_dq_splits(p, false);
+    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : strict_tc && dq_splits == 1;
     cudaError_t e = mgn::launch_bwd_preprocess(o, d_o, delta, no_acc ? nullptr : dq_acc, sched, rows, D, fast ? 1 : 0, st);
     if (e != cudaSuccess) return MGN_ERR_CUDA;
     MainKernelTimer timer(st);
-    if (!fast)
+    if (fast)
+        e = mgn::launch_fast_bwd(p, q, k, v, d_o, lse, delta, dq_acc, dq, dk, dv, sched, status, st);
+    else if (strict_tc)
+        e = mgn::launch_strict_tc_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
+                                      static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
+                                      static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv),
+                                      dq_splits, status, st);
+    else
         e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
                                    static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
                                    static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv), status,
                                    st);
-    else
-        e = mgn::launch_fast_bwd(p, q, k, v, d_o, lse, delta, dq_acc, dq, dk, dv, sched, status, st);
     return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
 }
 
@@ -249,10 +256,11 @@ int mgn_attn_bwd_deterministic(const void* q, const void* k, const void* v, cons
         e = mgn::launch_fast_dq(p, q, k, v, d_o, lse, delta, dq, status, st);
         return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
     }
-    if (mgn::strict_bwd_on_tensor_cores(p)) {
-        e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
-                                   static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
-                                   static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv), status, st);
+    if (mgn::strict_on_tensor_cores(p)) {
+        e = mgn::launch_strict_tc_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
+                                      static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
+                                      static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv), 1, status,
+                                      st);
         return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
     }
     e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
@@ -283,18 +291,25 @@ int mgn_attn_bwd_given_delta(const void* q, const void* k, const void* v, const 
     unsigned* sched = fast ? reinterpret_cast<unsigned*>(static_cast<char*>(workspace) + ws_delta_bytes(rows)) : nullptr;
     float* dq_acc = fast ? reinterpret_cast<float*>(static_cast<char*>(workspace) + ws_delta_bytes(rows) + kSchedBytes)
                          : static_cast<float*>(dq);
-    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : mgn::strict_bwd_on_tensor_cores(p);
+    const bool strict_tc = !fast && mgn::strict_on_tensor_cores(p);
+    const int dq_splits = mgn::strict_dq_splits(p, false);
+    const bool no_acc = fast ? mgn::fast_bwd_writes_dq_directly(p) : strict_tc && dq_splits == 1;
     cudaError_t e = cudaSuccess;
     if (fast || !no_acc) e = mgn::launch_bwd_clear(no_acc ? nullptr : dq_acc, rows * D, sched, st);
     if (e != cudaSuccess) return MGN_ERR_CUDA;
     MainKernelTimer timer(st);
-    if (!fast)
+    if (fast)
+        e = mgn::launch_fast_bwd(p, q, k, v, d_o, lse, delta, dq_acc, dq, dk, dv, sched, status, st);
+    else if (strict_tc)
+        e = mgn::launch_strict_tc_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
+                                      static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
+                                      static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv),
+                                      dq_splits, status, st);
+    else
         e = mgn::launch_strict_bwd(p, static_cast<const float*>(q), static_cast<const float*>(k),
                                    static_cast<const float*>(v), static_cast<const float*>(d_o), lse, delta,
                                    static_cast<float*>(dq), static_cast<float*>(dk), static_cast<float*>(dv), status,
                                    st);
-    else
-        e = mgn::launch_fast_bwd(p, q, k, v, d_o, lse, delta, dq_acc, dq, dk, dv, sched, status, st);
     return e == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
 }
 

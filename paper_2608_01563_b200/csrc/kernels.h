@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 
 #include <stdio.h>
@@ -86,18 +87,46 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned bl
 int make_tmap_3d(CUtensorMap* out, const void* base, int elem_bytes, int is_bf16,
                  int BH, int S, int D, int box_d, int box_rows);
 
+// Problems whose 64-row tiles would leave half of the SMs without work are cut finer (16-row query tiles forward,
+// 32-row key tiles backward): a call of two heads of 64 tokens is one chain per tile, and shorter chains end
+// sooner.  (1,2,64,32), strict: forward 7.5 -> 3.5 us, backward 9.3 -> 7.3 us.
+inline bool strict_few_tiles(long long tiles64) { return tiles64 <= 74; }
+
 // Strict (f32 FFMA) kernels.
 cudaError_t launch_strict_fwd(const Problem& p, const float* q, const float* k, const float* v,
                               float* o, float* lse, unsigned* status, cudaStream_t st);
 // The same on the tensor cores (D = 64 and 128): f32 products as six bf16 partial products each.
-inline bool strict_fwd_on_tensor_cores(const Problem& p) { return p.D != 32 && p.Sk >= 64; }
+// Forward and backward take the same route whatever the entry point: P = exp(s - LSE) of the backward is as good as
+// f32 allows only where both were rounded alike (a row that attends to itself with a score of 92 in the log2 domain:
+// dV off by 2.7e-5 across the routes, by 7e-6 within either).  The line is where forward and backward together are
+// ahead on one B200.  D = 64, 2 heads of 64 / 128 / 256 tokens: 14.2 / 22.5 / 39 us FFMA, 18.8 / 23.7 / 33 here (without
+// atomics 28 / 46 / 80 against 19 / 24 / 33); 96 heads of 64: 25 / 26; 256 heads of 90: 104 / 64.  D = 128, 12 heads
+// of 64 queries and 77 keys: 46 / 31.
+//   At most 64 queries of ungrouped heads over few key tiles stay on FFMA: its backward spreads them over the key
+// tiles in one step (forward and backward of 8 heads, 40 x 300, D = 64: 21 us against
+// 34; 16 heads, 30 x 500, D = 128: 46 against 84).
+inline bool strict_on_tensor_cores(const Problem& p) {
+    if (p.Sq <= 64 && p.group() == 1 && static_cast<long long>((p.Sk + 63) / 64) * p.BHkv() <= 296) return false;
+    if (p.D == 128) return p.Sk >= 64;
+    if (p.D != 64 || p.Sk <= 64) return false;
+    return p.Sk >= 128 || !strict_few_tiles(static_cast<long long>((p.Sq + 63) / 64) * p.BH());
+}
 cudaError_t launch_strict_tc_fwd(const Problem& p, const float* q, const float* k, const float* v,
                                  float* o, float* lse, unsigned* status, cudaStream_t st);
-// Backward on the tensor cores: no floating-point atomics, dq, dk, dv need not be cleared.
-inline bool strict_bwd_on_tensor_cores(const Problem& p) { return p.D != 32 && p.Sk >= 64 && p.Sq >= 64; }
+// Backward on the tensor cores: dq, dk, dv need not be cleared unless dq_splits > 1 (dq then; see strict_dq_splits).
+// A short query sequence over a long key sequence leaves the dQ kernel few and long chains: where atomics are allowed
+// its keys are dealt to several CTAs per query tile, at least 256 keys each, which add into a cleared dQ
+// (backward of 16 heads, 128 x 8192, D = 128: 897 -> 246 us; 32 heads in groups of 4, 64 x 1024: 104 -> 65).
+inline int strict_dq_splits(const Problem& p, bool deterministic) {
+    const long long tiles = static_cast<long long>((p.Sq + 127) / 128) * p.BH();
+    if (deterministic || tiles > 74) return 1;
+    const long long by_sm = 148 / tiles, by_keys = p.Sk / 256;
+    const long long n = by_sm < by_keys ? by_sm : by_keys;
+    return n > 1 ? static_cast<int>(n) : 1;
+}
 cudaError_t launch_strict_tc_bwd(const Problem& p, const float* q, const float* k, const float* v, const float* d_o,
                                  const float* lse, const float* delta, float* dq, float* dk, float* dv,
-                                 unsigned* status, cudaStream_t st);
+                                 int dq_splits, unsigned* status, cudaStream_t st);
 cudaError_t launch_strict_bwd(const Problem& p, const float* q, const float* k, const float* v,
                               const float* d_o, const float* lse, const float* delta,
                               float* dq, float* dk, float* dv, unsigned* status, cudaStream_t st);

@@ -375,9 +375,12 @@ cudaError_t launch_strict_bwd(const Problem& p, const float* q, const float* k, 
                               const float* d_o, const float* lse, const float* delta,
                               float* dq, float* dk, float* dv, unsigned* status, cudaStream_t st)
 {
-    if (strict_bwd_on_tensor_cores(p)) return launch_strict_tc_bwd(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
     int BM, BN;
     strict_bwd_tiles(p, &BM, &BN);
+    if (strict_few_tiles(static_cast<long long>((p.Sk + 63) / 64) * p.BHkv())) {
+        if (p.D == 32) return launch<32, 32, 32, 128>(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
+        if (p.D == 64) return launch<64, 32, 32, 128>(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
+    }
     switch (p.D) {
         case 32:  return launch<32, 64, 64, 128>(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
         case 64:

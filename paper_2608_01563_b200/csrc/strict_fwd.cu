@@ -372,9 +372,14 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
 cudaError_t launch_strict_fwd(const Problem& p, const float* q, const float* k, const float* v,
                               float* o, float* lse, unsigned* status, cudaStream_t st)
 {
-    if (strict_fwd_on_tensor_cores(p)) return launch_strict_tc_fwd(p, q, k, v, o, lse, status, st);
+    if (strict_on_tensor_cores(p)) return launch_strict_tc_fwd(p, q, k, v, o, lse, status, st);
     int BM, BN;
     strict_fwd_tiles(p, &BM, &BN);
+    if (strict_few_tiles(static_cast<long long>((p.Sq + 63) / 64) * p.BH())) {
+        if (p.D == 32) return launch<32, 16, 128, 128>(p, q, k, v, o, lse, status, st);
+        if (p.D == 64) return launch<64, 16, 128, 128>(p, q, k, v, o, lse, status, st);
+        if (p.D == 128) return launch<128, 16, 64, 128>(p, q, k, v, o, lse, status, st);
+    }
     switch (p.D) {
         case 32:  return launch<32, 64, 128, 128>(p, q, k, v, o, lse, status, st);
         case 64:

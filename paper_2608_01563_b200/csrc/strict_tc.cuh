@@ -190,6 +190,15 @@ struct OwnRows {
             if (r < rows) *reinterpret_cast<float4*>(dst + r * D + 4 * c) = lds128(ex + r * PITCH + c * 16);
         }
     }
+    // the same, added to what is there
+    static __device__ __forceinline__ void add(float* dst, int rows, uint32_t ex, int t) {
+#pragma unroll 4
+        for (int k = 0; k < NQ; ++k) {
+            const int u = t + 256 * k, r = u / (D / 4), c = u % (D / 4);
+            const float4 x = lds128(ex + r * PITCH + c * 16);
+            if (r < rows) red_add_v4(dst + r * D + 4 * c, x.x, x.y, x.z, x.w);
+        }
+    }
     // half h of row r of the exchange tile, split into tensor memory: part a at columns t + a * D / 2
     static __device__ __forceinline__ void half_row_to_tmem(uint32_t ex, int r, int h, uint32_t tm) {
 #pragma unroll 1

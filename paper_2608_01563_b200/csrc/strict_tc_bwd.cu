@@ -379,7 +379,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                     const float* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ DELTA,
-                    float* __restrict__ dQ, int Sq, int Sk, int BH, int H, int G, int n_qt, int causal, float c_hi,
+                    float* __restrict__ dQ, int Sq, int Sk, int BH, int H, int G, int n_qt, int splits, int causal, float c_hi,
                     float c_lo, float scale, unsigned* status)
 {
     using C = DqCfg<D>;
@@ -392,13 +392,20 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Heaviest (last) query tiles first when causal.
-    const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / BH;
-    const int bh = static_cast<int>(blockIdx.x) % BH;
+    const int item = static_cast<int>(blockIdx.x) / splits, part = static_cast<int>(blockIdx.x) % splits;
+    const int qt = n_qt - 1 - item / BH, bh = item % BH;
     const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
     const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
     const int i0 = qt * kBM;
     const int i_last = min(i0 + kBM, Sq) - 1;
-    const int n_blk = causal ? (i_last + off) / R + 1 : (Sk + R - 1) / R;
+    // key blocks of this CTA: its share of those that the tile sees (the last share may be short, or empty)
+    const int n_all = causal ? (i_last + off) / R + 1 : (Sk + R - 1) / R;
+    const int share = (n_all + splits - 1) / splits, b0 = part * share;
+    const int n_blk = min(share, n_all - b0);
+    if (n_blk <= 0) {
+        pdl_wait();
+        return;
+    }
 
     if (tid == 0) {
         for (int w = 0; w < 2; ++w) {
@@ -480,8 +487,8 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
             Converter<D, R> cv(tid - (is_k ? 64 : 160));
             cv.run(n_blk,
                    [&](int n, int& rows) {
-                       rows = Sk - n * R;
-                       return head + static_cast<size_t>(n) * R * D;
+                       rows = Sk - (b0 + n) * R;
+                       return head + static_cast<size_t>(b0 + n) * R * D;
                    },
                    [&](int n) {
                        if (n >= 2) mbar_wait(bar(C::Z_DONE + (n & 1)), ((n >> 1) & 1) ^ 1, status);
@@ -545,7 +552,8 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
 #pragma unroll 1
         for (int n = 0; n < n_blk; ++n) {
             const uint32_t x = tl + C::TM_X + (n & 1) * C::X;
-            const bool masked = (causal && n * R + R - 1 > i0 + off) || n * R + R > Sk;
+            const int j0 = (b0 + n) * R;                   // first key of the block
+            const bool masked = (causal && j0 + R - 1 > i0 + off) || j0 + R > Sk;
             float p[HC], s[HC];
             uint32_t a[HC / 2], b[HC / 2], c[HC / 2];
             mbar_wait(bar(C::S_DONE + (n & 1)), (n >> 1) & 1, status);
@@ -559,7 +567,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
                 p[e + 1] = ex2(t1);
             }
             if (masked) {
-                const int lim = vis - n * R - h * HC;
+                const int lim = vis - j0 - h * HC;
 #pragma unroll
                 for (int e = 0; e < HC; ++e)
                     if (e >= lim) p[e] = 0.f;
@@ -586,7 +594,8 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
         for (int d = 0; d < D / 2; d += 4)
             sts128f(ex + d * 4, acc[d] * scale, acc[d + 1] * scale, acc[d + 2] * scale, acc[d + 3] * scale);
         named_bar_sync(1, kCompute);
-        OwnRows<D>::store(dQ + own_at, Sq - i0, base, t);
+        if (splits == 1) OwnRows<D>::store(dQ + own_at, Sq - i0, base, t);
+        else OwnRows<D>::add(dQ + own_at, Sq - i0, base, t);
     }
 
     tc_fence_before();
@@ -597,7 +606,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
 
 template <int D>
 cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, const float* d_o, const float* lse,
-                   const float* delta, float* dq, float* dk, float* dv, unsigned* status, cudaStream_t st)
+                   const float* delta, float* dq, float* dk, float* dv, int dq_splits, unsigned* status, cudaStream_t st)
 {
     using KC = KvCfg<D>;
     using QC = DqCfg<D>;
@@ -609,7 +618,7 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
     if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_dq attributes");
     const long long kv_blocks = static_cast<long long>((p.Sk + kBM - 1) / kBM) * p.BHkv();
     const int n_qt = (p.Sq + kBM - 1) / kBM;
-    const long long dq_blocks = static_cast<long long>(n_qt) * p.BH();
+    const long long dq_blocks = static_cast<long long>(n_qt) * p.BH() * dq_splits;
     if (kv_blocks > 0x7fffffffLL || dq_blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     const double c = score_factor(p.scale, D);
     const float c_hi = static_cast<float>(c), c_lo = static_cast<float>(c - c_hi);
@@ -619,18 +628,18 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
     e = cudaGetLastError();
     if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_dkv launch");
     return MGN_FAIL(launch_pdl(dqk, static_cast<unsigned>(dq_blocks), kThreads, QC::SMEM, st, q, k, v, d_o, lse, delta, dq, p.Sq,
-                               p.Sk, p.BH(), p.H, p.group(), n_qt, p.causal, c_hi, c_lo, p.scale, status),
+                               p.Sk, p.BH(), p.H, p.group(), n_qt, dq_splits, p.causal, c_hi, c_lo, p.scale, status),
                     "strict_tc_dq launch");
 }
 
 }  // namespace
 
 cudaError_t launch_strict_tc_bwd(const Problem& p, const float* q, const float* k, const float* v, const float* d_o,
-                                 const float* lse, const float* delta, float* dq, float* dk, float* dv, unsigned* status,
+                                 const float* lse, const float* delta, float* dq, float* dk, float* dv, int dq_splits, unsigned* status,
                                  cudaStream_t st)
 {
-    return p.D == 64 ? launch<64>(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st)
-                     : launch<128>(p, q, k, v, d_o, lse, delta, dq, dk, dv, status, st);
+    return p.D == 64 ? launch<64>(p, q, k, v, d_o, lse, delta, dq, dk, dv, dq_splits, status, st)
+                     : launch<128>(p, q, k, v, d_o, lse, delta, dq, dk, dv, dq_splits, status, st);
 }
 
 }  // namespace mgn

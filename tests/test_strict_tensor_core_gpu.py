@@ -22,6 +22,9 @@ CASES = [
     (1, 4, 2, 97, 353, 128, True),       # causal offset 256, one row into a 32-row block
     (1, 4, 1, 321, 448, 64, True),       # group of four, offset 127
     (1, 2, 2, 700, 96, 64, False),       # many query blocks over two key blocks
+    (1, 2, 1, 70, 1025, 64, True),       # dQ's keys dealt to two CTAs per tile, one key in the last block
+    (1, 4, 2, 1, 2100, 128, True),       # one query row, four shares of the keys
+    (1, 1, 1, 130, 4700, 128, False),    # eighteen shares of 9 blocks, the last one empty or short
 ]
 
 
@@ -34,6 +37,30 @@ def test_edges_of_the_tiles(B, H, Hkv, Sq, Sk, D, causal, scale_sign):
     got = hp.run_cuda_ext(q, k, v, d_o, causal, scale, mgn.MODE_STRICT_F32)
     ref = hp.run_oracle_ext(q, k, v, d_o, causal, scale)
     hp.check_strict(got, ref, literal_max_abs=False, label=f"strict tensor-core {B,H,Hkv,Sq,Sk,D,causal} ")
+
+
+FEW_TILES = [
+    # problems that leave most SMs without a 64-row tile are cut into 16-row query and 32-row key tiles
+    (1, 1, 1, 1, 1, 32, True),
+    (1, 2, 2, 17, 17, 32, True),         # one row into the second query tile
+    (1, 2, 1, 33, 65, 32, False),        # one row into the second key tile of both widths
+    (2, 3, 3, 100, 161, 32, True),       # causal offset 61
+    (1, 4, 2, 50, 40, 64, False),
+    (1, 2, 2, 129, 63, 64, False),
+    (1, 3, 3, 33, 129, 128, True),       # at most 64 queries of ungrouped heads
+    (2, 2, 2, 64, 200, 64, True),
+    (1, 74, 74, 18, 18, 32, False),      # the last count of tiles that is cut finer, and the first that is not
+    (1, 75, 75, 18, 18, 32, False),
+]
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", FEW_TILES)
+def test_few_tiles(B, H, Hkv, Sq, Sk, D, causal):
+    q, _, _, d_o = synth.random_inputs(705, B, H, Sq, D)
+    _, k, v, _ = synth.random_inputs(706, B, Hkv, Sk, D)
+    got = hp.run_cuda_ext(q, k, v, d_o, causal, 0.3, mgn.MODE_STRICT_F32)
+    ref = hp.run_oracle_ext(q, k, v, d_o, causal, 0.3)
+    hp.check_strict(got, ref, literal_max_abs=False, label=f"few tiles {B,H,Hkv,Sq,Sk,D,causal} ")
 
 
 @pytest.mark.parametrize("D", [64, 128])
