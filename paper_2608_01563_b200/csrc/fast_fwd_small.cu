@@ -6,13 +6,15 @@
 // small (Section 7.3).  The persistent kernel in fast_fwd.cu is built for long items: with one or two
 // key blocks per item its fill, hand-offs and epilogue (about 5 us per item, one item at a time per SM)
 // are all there is.  Here one small CTA owns one 128-row query tile of one head and up to four of them
-// share an SM (two at D = 128), so the latencies of neighbouring tiles overlap:
+// share an SM (two at D = 128 or with two key blocks), so the latencies of neighbouring tiles overlap:
 //   warp 0, one lane   TMA loads (Q once; K and V per block, single buffers) and all tensor-core issue
 //   warps 1-4          softmax, ONE THREAD PER ROW (tensor-memory lane): the row maximum, the running
 //                      sum and the rescaling factor are thread-local, so the classic online softmax
 //                      needs no exchange between threads and no speculation
 // Tensor memory (256 columns): S [0,128), O [128,128+D).  P (bf16) overwrites S, keys 0-127 at S[0,64),
-// each 16-column piece written over columns the thread has already read.  The output tile leaves through
+// each 16-column piece written over columns the thread has already read.  With a single key block at D = 64
+// (ONE) the columns S[64,128) are dead when the product with V is issued, so O takes them: 128 columns, four
+// CTAs per SM instead of two ((16,8,1024 x 77,64), forward and backward: 55.5 -> 49.5 us).  The output tile leaves through
 // the Q buffer (dead after the last score product) and a TMA store.
 #include "kernels.h"
 #include "fast_items.cuh"
@@ -26,25 +28,27 @@ constexpr int BM = 128, BN = 128;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
-template <int D>
+template <int D, bool ONE>
 struct Cfg {
+    static constexpr bool SHARE = ONE && D == 64;
     static constexpr int NCH = D / 64;
     static constexpr int TILE_BYTES = 128 * D * 2;
     static constexpr int CHUNK_BYTES = 128 * 128;
     static constexpr int OFF_Q = 0, OFF_K = TILE_BYTES, OFF_V = 2 * TILE_BYTES, OFF_BAR = 3 * TILE_BYTES;
     static constexpr int PAYLOAD = OFF_BAR + 64;
     static constexpr int SMEM = PAYLOAD + 1024;
-    static constexpr uint32_t TM_S = 0, TM_O = 128, TM_COLS = 256;
+    static constexpr uint32_t TM_S = 0, TM_O = SHARE ? 64 : 128, TM_COLS = SHARE ? 128 : 256;
+    static constexpr int CTAS = SHARE ? 4 : 2;
 };
 enum { B_Q = 0, B_K = 1, B_V = 2, B_SFULL = 3, B_PFULL = 4, B_PVDONE = 5, B_COUNT = 6 };
 
-template <int D, bool GEN>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int D, bool GEN, bool ONE>
+__global__ void __launch_bounds__(kThreads, Cfg<D, ONE>::CTAS)
 fast_fwd_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                       float* __restrict__ LSE, const Dims dm, int n_qt, int causal, float c2, unsigned* status)
 {
-    using C = Cfg<D>;
+    using C = Cfg<D, ONE>;
     extern __shared__ uint8_t smem_raw[];
     if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -57,7 +61,7 @@ fast_fwd_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const int bh = static_cast<int>(blockIdx.x) / n_qt;
     const int row0 = (n_qt - 1 - static_cast<int>(blockIdx.x) % n_qt) * BM;       // last (heaviest) tiles of a head first
     const int bhk = GEN ? (bh / dm.H) * (dm.H / dm.G) + (bh % dm.H) / dm.G : bh;
-    const int n_kb = (Sk + BN - 1) / BN;
+    const int n_kb = ONE ? 1 : (Sk + BN - 1) / BN;
     const int nb = causal ? min(n_kb, (min(row0 + BM, Sq) - 1 + coff) / BN + 1) : n_kb;   // key blocks this tile sees (>= 1)
 
     if (tid == 0) {
@@ -227,17 +231,17 @@ fast_fwd_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     if (warp == 0) tmem_dealloc(tmem, C::TM_COLS);
 }
 
-template <int D, bool GEN>
+template <int D, bool GEN, bool ONE>
 cudaError_t launch_gen(const Problem& p, const void* q, const void* k, const void* v, void* o, float* lse,
                        unsigned* status, cudaStream_t st)
 {
-    using C = Cfg<D>;
+    using C = Cfg<D, ONE>;
     CUtensorMap tq, tk, tv, to;
     if (make_tmap_3d(&tq, q, 2, 1, p.BH(), p.Sq, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map q");
     if (make_tmap_3d(&tk, k, 2, 1, p.BHkv(), p.Sk, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map k");
     if (make_tmap_3d(&tv, v, 2, 1, p.BHkv(), p.Sk, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map v");
     if (make_tmap_3d(&to, o, 2, 1, p.BH(), p.Sq, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map o");
-    auto kern = fast_fwd_small_kernel<D, GEN>;
+    auto kern = fast_fwd_small_kernel<D, GEN, ONE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return MGN_FAIL(e, "cudaFuncSetAttribute");
     const int n_qt = (p.Sq + BM - 1) / BM;
@@ -253,8 +257,12 @@ template <int D>
 cudaError_t launch(const Problem& p, const void* q, const void* k, const void* v, void* o, float* lse,
                    unsigned* status, cudaStream_t st)
 {
-    return (p.Hkv != p.H || p.Sq != p.Sk) ? launch_gen<D, true>(p, q, k, v, o, lse, status, st)
-                                          : launch_gen<D, false>(p, q, k, v, o, lse, status, st);
+    const bool gen = p.Hkv != p.H || p.Sq != p.Sk;
+    if (p.Sk <= BN)
+        return gen ? launch_gen<D, true, true>(p, q, k, v, o, lse, status, st)
+                   : launch_gen<D, false, true>(p, q, k, v, o, lse, status, st);
+    return gen ? launch_gen<D, true, false>(p, q, k, v, o, lse, status, st)
+               : launch_gen<D, false, false>(p, q, k, v, o, lse, status, st);
 }
 
 }  // namespace
