@@ -61,7 +61,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                      const float* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ DELTA,
-                     float* __restrict__ dK, float* __restrict__ dV, int Sq, int Sk, int BHkv, int G, int causal,
+                     float* __restrict__ dK, float* __restrict__ dV, int Sq, int Sk, int BHkv, int G, int Hg, int causal,
                      float c_hi, float c_lo, float dk_factor, unsigned* status)
 {
     using C = KvCfg<D>;
@@ -75,7 +75,8 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     pdl_launch_dependents();                               // the dQ kernel may fill SMs as this one drains
 
     // First key blocks first: under a causal mask they see the most queries.
-    const int kb = static_cast<int>(blockIdx.x) / BHkv, bhk = static_cast<int>(blockIdx.x) % BHkv;
+    int kb, bhk;
+    item_of_block(static_cast<int>(blockIdx.x), (Sk + kBM - 1) / kBM, BHkv, Hg, kb, bhk);
     const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
     const int j0 = kb * kBM;
     const int m0 = causal ? max(0, j0 - off) / R : 0;      // first query block that sees a key of this block
@@ -379,7 +380,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
                     const float* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ DELTA,
-                    float* __restrict__ dQ, int Sq, int Sk, int BH, int H, int G, int n_qt, int splits, int causal, float c_hi,
+                    float* __restrict__ dQ, int Sq, int Sk, int BH, int H, int G, int n_qt, int Hg, int splits, int causal, float c_hi,
                     float c_lo, float scale, unsigned* status)
 {
     using C = DqCfg<D>;
@@ -393,7 +394,9 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
 
     // Heaviest (last) query tiles first when causal.
     const int item = static_cast<int>(blockIdx.x) / splits, part = static_cast<int>(blockIdx.x) % splits;
-    const int qt = n_qt - 1 - item / BH, bh = item % BH;
+    int tile, bh;
+    item_of_block(item, n_qt, BH, Hg, tile, bh);
+    const int qt = n_qt - 1 - tile;
     const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
     const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
     const int i0 = qt * kBM;
@@ -624,11 +627,12 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
     const float c_hi = static_cast<float>(c), c_lo = static_cast<float>(c - c_hi);
     const float dk_factor = c == 0.0 ? 0.f : static_cast<float>(p.scale / c);    // dK was summed over c Q
     kv<<<static_cast<unsigned>(kv_blocks), kThreads, KC::SMEM, st>>>(q, k, v, d_o, lse, delta, dk, dv, p.Sq, p.Sk, p.BHkv(),
-                                                                     p.group(), p.causal, c_hi, c_lo, dk_factor, status);
+                                                                     p.group(), head_group(8.0 * p.Sq * D * p.group(), p.BHkv()), p.causal, c_hi, c_lo, dk_factor, status);
     e = cudaGetLastError();
     if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_dkv launch");
     return MGN_FAIL(launch_pdl(dqk, static_cast<unsigned>(dq_blocks), kThreads, QC::SMEM, st, q, k, v, d_o, lse, delta, dq, p.Sq,
-                               p.Sk, p.BH(), p.H, p.group(), n_qt, dq_splits, p.causal, c_hi, c_lo, p.scale, status),
+                               p.Sk, p.BH(), p.H, p.group(), n_qt,
+                               head_group(8.0 * p.Sk * D / p.group(), p.BH()), dq_splits, p.causal, c_hi, c_lo, p.scale, status),
                     "strict_tc_dq launch");
 }
 

@@ -70,7 +70,7 @@ __device__ __noinline__ float plain_row(const float* q, const float* k, const fl
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
-                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int BH, int H, int G, int n_qt,
+                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int BH, int H, int G, int n_qt, int Hg,
                      int causal, float c_hi, float c_lo, unsigned* status)
 {
     using C = Cfg<D>;
@@ -83,8 +83,9 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Heaviest (last) query tiles first when causal.
-    const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / BH;
-    const int bh = static_cast<int>(blockIdx.x) % BH;
+    int tile, bh;
+    item_of_block(static_cast<int>(blockIdx.x), n_qt, BH, Hg, tile, bh);
+    const int qt = n_qt - 1 - tile;
     const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
     const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
     const int i0 = qt * kBM;
@@ -329,7 +330,7 @@ cudaError_t launch(const Problem& p, const float* q, const float* k, const float
     const double c = score_factor(p.scale, D);
     const float c_hi = static_cast<float>(c), c_lo = static_cast<float>(c - c_hi);
     kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(q, k, v, o, lse, p.Sq, p.Sk, p.BH(), p.H, p.group(),
-                                                                   n_qt, p.causal, c_hi, c_lo, status);
+                                                                   n_qt, head_group(8.0 * p.Sk * D / p.group(), p.BH()), p.causal, c_hi, c_lo, status);
     return MGN_FAIL(cudaGetLastError(), "strict_tc_fwd launch");
 }
 

@@ -28,6 +28,23 @@ CASES = [
 ]
 
 
+GROUPED_HEADS = [
+    # K and V (Q and dO) of all heads exceed half of L2: heads in groups of 6, 6 and 5
+    (1, 17, 17, 130, 4096, 128, False),
+    (1, 17, 17, 4096, 130, 128, False),
+]
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", GROUPED_HEADS)
+def test_heads_in_groups(B, H, Hkv, Sq, Sk, D, causal):
+    scale = 1.0 / math.sqrt(D)
+    q, _, _, d_o = synth.random_inputs(702, B, H, Sq, D)
+    _, k, v, _ = synth.random_inputs(703, B, Hkv, Sk, D)
+    got = hp.run_cuda_ext(q, k, v, d_o, causal, scale, mgn.MODE_STRICT_F32)
+    ref = hp.run_oracle_ext(q, k, v, d_o, causal, scale)
+    hp.check_strict(got, ref, literal_max_abs=False, label=f"grouped heads {B,H,Hkv,Sq,Sk,D,causal} ")
+
+
 @pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", CASES)
 @pytest.mark.parametrize("scale_sign", [1.0, -1.0])
 def test_edges_of_the_tiles(B, H, Hkv, Sq, Sk, D, causal, scale_sign):
