@@ -33,8 +33,8 @@ METRIC = "attention fwd+bwd TFLOP/s per B200 (strict f32, bf16) and % of matchin
 # ncu summary named beside it (same workload and launch configuration as the bench; re-taken when that
 # kernel changes -- the record carries the file so that a stale figure can be told)
 NCU_TRAFFIC = {
-    ("strict", "gpt2_small"): (140.9e6 + 41.3e6, "profiles/strict_fwd_bwd_gpt2_small.md",
-                               "strict_bwd_kernel<64,64,64,128,false,true>"),
+    ("strict", "gpt2_small"): (105.4e6 + 18.5e6 + 107.5e6 + 8.2e6, "profiles/strict_tensor_core.md",
+                               "strict_tc_dkv_kernel<64> + strict_tc_dq_kernel<64>"),
     ("fast", "long_context"): (203.3e6 + 88.7e6, "profiles/fast_fwd_bwd_long_context.md",
                                "fast_bwd_kernel<128,false,true>"),
 }
@@ -774,9 +774,13 @@ def main():
         fl_sum = flops(w, "sum")
         value = whole_job_tflops(w, world, K, total_ms_max)
         if args.mode == "strict":
-            peak = fp32_peak_tflops(peaks)
-            bound = "alu"
-            peak_note = f"{SM_COUNT} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {peaks.get('sm_max_mhz', 1965.0):.0f} MHz"
+            # D = 64 and 128 form an f32 product from six bf16 partial products; D = 32 runs on FFMA
+            tensor_route = w.D != 32
+            peak = peaks["bf16_tflops"] / 6.0 if tensor_route else fp32_peak_tflops(peaks)
+            bound = "tensor" if tensor_route else "alu"
+            ffma_note = f"{SM_COUNT} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {peaks.get('sm_max_mhz', 1965.0):.0f} MHz"
+            peak_note = (f"{peak_src} dense bf16 burst / 6: an f32 product is six bf16 partial products "
+                         f"(FP32 FFMA peak, {ffma_note}: {fp32_peak_tflops(peaks):.2f} TFLOP/s)") if tensor_route else ffma_note
         else:
             peak = peaks["bf16_tflops"]
             bound = "tensor"
@@ -798,7 +802,7 @@ def main():
             "fwd_tflops": flops(w, "fwd") / (fwd_call_ms * 1e-3) / 1e12,
             "bwd_tflops": flops(w, "bwd") / (bwd_call_ms * 1e-3) / 1e12,
             "fwd_ms": fwd_call_ms, "bwd_ms": bwd_call_ms,
-            "roofline": {"kernel": "bwd_main (fused dK/dV/dQ)", "bound": bound, "achieved": bwd_main_tflops,
+            "roofline": {"kernel": "bwd_main (dK+dV and dQ)", "bound": bound, "achieved": bwd_main_tflops,
                          "peak": peak, "unit": "TFLOP/s", "frac": bwd_main_tflops / peak,
                          "traffic": NCU_TRAFFIC.get((args.mode, w.name), (None,))[0],
                          "traffic_unit": "bytes per launch (ncu dram read+write)",
@@ -807,7 +811,7 @@ def main():
                          "ms_per_launch": bwd_main_ms, "peak_source": peak_note,
                          "fwd_kernel": {"achieved": fwd_main_tflops, "frac": fwd_main_tflops / peak,
                                         "ms_per_launch": fwd_main_ms}},
-            "gpu_launches": (3 if args.mode == "strict" else 4) * K,
+            "gpu_launches": (3 if args.mode == "strict" and w.D == 32 else 4) * K,
             "clocks": clocks,
         }
         if e2e_ms is not None:
