@@ -263,20 +263,18 @@ template <bool SCORE, int ST> __device__ constexpr int n_terms() {
     return SCORE && ST == 2 ? 5 : ST == 1 ? 6 : ST == 2 ? 4 : 3;
 }
 
-// A region of tensor memory that receives rows of N values in ST column sets and is later overwritten by the
-// three packed parts of what is formed from them.  The N/2 values of a half are worked on by one thread (or in
-// one go) and its parts stay within the columns that held those values (ST = 1: plus N/4 columns of a free
-// quarter in front), so a half never overwrites values of the other half.
-template <int N, int ST> __host__ __device__ constexpr uint32_t x_cols() { return ST == 1 ? 3 * N / 2 : ST * N; }
-template <int N, int ST> __host__ __device__ constexpr uint32_t x_value_col() { return ST == 1 ? N / 2 : 0; }   // of set 0
-template <int N, int ST> __host__ __device__ constexpr uint32_t x_half_part_col(int half, int part) {
-    return ST == 1 ? (part == 2 ? half * (N / 4) : N / 2 + half * (N / 2) + part * (N / 4))
-                   : (part == 2 ? N + half * (N / 2) : half * (N / 2) + part * (N / 4));
+// A region of tensor memory that receives rows of N values in ST column sets (two or three) and is later overwritten
+// by the three packed parts of what is formed from them.  The N/2 values of a half are worked on by one thread (or
+// in one go) and its parts stay within the columns that held those values, so a half never overwrites values of the
+// other half.
+template <int N, int ST> __host__ __device__ constexpr uint32_t x_cols() { return ST * N; }
+template <int N> __host__ __device__ constexpr uint32_t x_half_part_col(int half, int part) {
+    return part == 2 ? N + half * (N / 2) : half * (N / 2) + part * (N / 4);
 }
 // columns of 16-value contraction step kk
-template <int N, int ST> __device__ __forceinline__ uint32_t x_part_col(uint32_t part, int kk) {
+template <int N> __device__ __forceinline__ uint32_t x_part_col(uint32_t part, int kk) {
     constexpr int SPH = N / 32;                          // steps per half
-    return x_half_part_col<N, ST>(kk / SPH, part) + (kk % SPH) * 8;
+    return x_half_part_col<N>(kk / SPH, part) + (kk % SPH) * 8;
 }
 
 template <int N> __device__ __forceinline__ void tmem_load(uint32_t t, uint32_t (&v)[N]) {
@@ -300,19 +298,19 @@ template <int W, int ST> __device__ __forceinline__ void load_sets(uint32_t t, u
 }
 // The values of one half of a region's row.
 template <int N, int ST> __device__ __forceinline__ void load_half(uint32_t x, int half, float (&v)[N / 2]) {
-    load_sets<N / 2, ST>(x + x_value_col<N, ST>() + half * (N / 2), N, v);
+    load_sets<N / 2, ST>(x + half * (N / 2), N, v);
 }
 // The packed parts of a half row (N/2 values) into its columns.
-template <int N, int ST> __device__ __forceinline__ void store_half_parts(uint32_t x, int half, const uint32_t (&h)[N / 4],
+template <int N> __device__ __forceinline__ void store_half_parts(uint32_t x, int half, const uint32_t (&h)[N / 4],
                                                                           const uint32_t (&m)[N / 4], const uint32_t (&l)[N / 4]) {
     if constexpr (N == 64) {
-        tmem_st16(x + x_half_part_col<N, ST>(half, 0), h);
-        tmem_st16(x + x_half_part_col<N, ST>(half, 1), m);
-        tmem_st16(x + x_half_part_col<N, ST>(half, 2), l);
+        tmem_st16(x + x_half_part_col<N>(half, 0), h);
+        tmem_st16(x + x_half_part_col<N>(half, 1), m);
+        tmem_st16(x + x_half_part_col<N>(half, 2), l);
     } else {
-        tmem_st8(x + x_half_part_col<N, ST>(half, 0), h);
-        tmem_st8(x + x_half_part_col<N, ST>(half, 1), m);
-        tmem_st8(x + x_half_part_col<N, ST>(half, 2), l);
+        tmem_st8(x + x_half_part_col<N>(half, 0), h);
+        tmem_st8(x + x_half_part_col<N>(half, 1), m);
+        tmem_st8(x + x_half_part_col<N>(half, 2), l);
     }
 }
 
@@ -336,11 +334,11 @@ __device__ __forceinline__ void issue_scores(uint32_t d, A a_at, uint64_t b_desc
     }
 }
 // Sets of D[128 x D] = X B over the R rows of the split tile B (as MN-major operand, see rows_desc), X the parts
-// in a region of ST_X sets.  Stacking (ST = 2) needs adjacent parts to be D columns apart: D = 64.
+// in a region of scores.  Stacking (ST = 2) needs adjacent parts to be D columns apart: D = 64.
 template <int D, int R> __device__ __forceinline__ uint64_t rows_desc(uint32_t tile) {
     return umma_smem_desc(tile, D == 64 ? part_bytes<R>() : block_bytes<R>(), 1024);
 }
-template <int D, int R, int ST_X, int ST>
+template <int D, int R, int ST>
 __device__ __forceinline__ void issue_rows(uint32_t d, uint32_t x, uint64_t b_desc) {
     static_assert(ST == 1 || D == 64, "");
 #pragma unroll 1
@@ -351,7 +349,7 @@ __device__ __forceinline__ void issue_rows(uint32_t d, uint32_t x, uint64_t b_de
         const uint32_t dt = d + m.set * D;
 #pragma unroll
         for (int kk = 0; kk < R / 16; ++kk)
-            umma_ts(dt, x + x_part_col<R, ST_X>(m.a, kk), b + ((kk * 2048) >> 4), idesc, (t > 0 || kk > 0) ? 1u : 0u);
+            umma_ts(dt, x + x_part_col<R>(m.a, kk), b + ((kk * 2048) >> 4), idesc, (t > 0 || kk > 0) ? 1u : 0u);
     }
 }
 

@@ -148,12 +148,12 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
                     const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
                     mbar_wait(bar(C::V_GO + w), (n >> 1) & 1, status);
                     tc_fence_after();
-                    issue_rows<D, R, C::ST, C::STZ>(tmem + C::TM_ZV, tmem + C::TM_X, mO + so);
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZV, tmem + C::TM_X, mO + so);
                     umma_commit(bar(C::V_DONE));
                     umma_commit(bar(C::S_GO + (w ^ 1)));
                     mbar_wait(bar(C::K_GO), n & 1, status);
                     tc_fence_after();
-                    issue_rows<D, R, C::ST, C::STZ>(tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so);
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so);
                     umma_commit(bar(C::K_DONE + w));       // both products of the block: its tiles are free too
                     umma_commit(bar(C::P_GO + (w ^ 1)));
                 }
@@ -283,7 +283,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
                 }
 #pragma unroll
                 for (int e = 0; e < HC; e += 2) split3(f2_pack(p[e], p[e + 1]), a[e / 2], b[e / 2], c[e / 2]);
-                store_half_parts<R, C::ST>(tl + C::TM_X, h, a, b, c);
+                store_half_parts<R>(tl + C::TM_X, h, a, b, c);
             }
             if constexpr (C::SHARED_Z) {
                 if (n > 0) {
@@ -317,7 +317,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
                     split3(f2_mul(f2_pack(p[e + 2], p[e + 3]), f2_add(f2_pack(s[e + 2], s[e + 3]), nd.hi)),
                            a[e / 2 + 1], b[e / 2 + 1], c[e / 2 + 1]);
                 }
-                store_half_parts<R, C::ST>(tl + C::TM_Y, h, a, b, c);
+                store_half_parts<R>(tl + C::TM_Y, h, a, b, c);
             }
             if constexpr (!C::SHARED_Z) {
                 tmem_st_wait();
@@ -474,7 +474,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
                     const int w = n & 1;
                     mbar_wait(bar(C::Q_GO), n & 1, status);
                     tc_fence_after();
-                    issue_rows<D, R, C::ST, C::STZ>(tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
                                         mK + static_cast<uint64_t>((w * C::STAGE) >> 4));
                     umma_commit(bar(C::Z_DONE + w));       // S, dP (whose results it was formed from) and dQ: tiles free
                     umma_commit(bar(C::S_GO + w));
@@ -584,7 +584,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
             for (int e = 0; e < HC; e += 2)
                 split3(f2_mul(f2_pack(p[e], p[e + 1]), f2_add(f2_pack(s[e], s[e + 1]), nd)),
                        a[e / 2], b[e / 2], c[e / 2]);
-            store_half_parts<R, C::ST>(x, h, a, b, c);
+            store_half_parts<R>(x, h, a, b, c);
             if (n > 0) add_result(n - 1);
             tmem_st_wait();
             tc_fence_before();

@@ -143,7 +143,7 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
                     const int w = n & 1;
                     mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
                     tc_fence_after();
-                    issue_rows<D, R, C::ST, C::STO>(tmem + C::TM_O, tmem + C::TM_X + w * C::X,
+                    issue_rows<D, R, C::STO>(tmem + C::TM_O, tmem + C::TM_X + w * C::X,
                                      mV + static_cast<uint64_t>((w * C::STAGE) >> 4));
                     umma_commit(bar(C::PDONE + w));
                     umma_commit(bar(C::SGO + w));
@@ -249,7 +249,7 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
                     else sum0 = f2_add(sum0, p);
                     split3(p, p0[e / 2], p1[e / 2], p2[e / 2]);
                 }
-                store_half_parts<R, C::ST>(tX, h, p0, p1, p2);
+                store_half_parts<R>(tX, h, p0, p1, p2);
             }
             tmem_st_wait();
             tc_fence_before();
