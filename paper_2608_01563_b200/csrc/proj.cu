@@ -19,12 +19,18 @@
 // The last two take the gradients with respect to the UNROTATED projection: the rotation depends on the
 // position, i.e. on the row of the operand, and cannot be folded into either product; rope_bwd_kernel
 // applies the opposite rotation to dQ and dK in place first (a streaming pass over those two tensors).
-// Persistent: one CTA per SM walks over 128 x 256 output tiles (tile t, t + grid, ...; neighbouring tiles
-// share their row block, so the CTAs running at one time share operand tiles in L2).  Warp 0 streams
-// 64-wide contraction slices of both operands through a four-stage TMA ring that keeps running across
-// tiles (a lane of warp 6 does the same for the other operand), one lane of warp 1 issues the products
-// into one of two 256-column tensor-memory accumulators, warps 2-5 (one thread per accumulator row) read
-// the other one out meanwhile.
+// Persistent, in pairs of CTAs (cta_group::2): a pair walks over 256 x 256 output tiles (tile t, t + pairs, ...;
+// neighbouring tiles share their rows, so the pairs running at one time share operand tiles in L2).  A CTA holds
+// 128 rows of A, its half of the tile, and 128 of the 256 columns of B, and each SM's tensor core reads the columns
+// from both: per 64-wide piece of the contraction and 512 clocks of products an SM fetches 32 KB from L2, where a
+// CTA with a 128 x 256 tile of its own fetched 48 KB -- 94 bytes per clock wanted, of which it got about 55 (a layer of
+// 2 x 4096 positions, E = 2048, forward and backward: 1505 -> 1427 us).
+// The two row tiles of a pair need not be neighbours: they are consecutive in the list of the 128-row tiles of all
+// batch elements, so short sequences pay no padding to 256 rows.
+// Per CTA: a lane of warp 0 and one of warp 6 stream the two operands through a three-stage TMA ring (two 64-wide
+// pieces a stage: every barrier wait of the issuing lane costs the tensor core about 150 clocks) that keeps running
+// across tiles; one lane of the first CTA's warp 1 issues the products of both into one of two 256-column
+// tensor-memory accumulators; warps 2-5 (one thread per accumulator row) read the other one out meanwhile.
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -34,13 +40,15 @@ namespace mgn {
 namespace {
 
 constexpr int kThreads = 224;
-constexpr int TM = 128, TN = 256, TK = 64, kStages = 4;
-constexpr int A_BYTES = TM * TK * 2;          // 16 KB
-constexpr int B_BYTES = TN * TK * 2;          // 32 KB
+constexpr int TM = 128, TN = 256, TNC = TN / 2, TK = 64;        // rows of a CTA, columns of a pair and of a CTA's share of B
+constexpr int kPieces = 2, kStages = 3;                         // 64-wide pieces of the contraction in a stage
+constexpr int A_PIECE = TM * TK * 2, B_PIECE = TNC * TK * 2;    // 16 KB each
+constexpr int A_BYTES = kPieces * A_PIECE, B_BYTES = kPieces * B_PIECE;
 constexpr int OFF_A = 0, OFF_B = kStages * A_BYTES, OFF_BAR = OFF_B + kStages * B_BYTES;
 constexpr int PAYLOAD = OFF_BAR + 128;
 constexpr int SMEM = PAYLOAD + 1024;
 enum { B_FULL = 0, B_EMPTY = kStages, B_ACCFULL = 2 * kStages, B_ACCEMPTY = 2 * kStages + 2, B_COUNT = 2 * kStages + 4 };
+static_assert(B_COUNT * 8 + 8 <= PAYLOAD - OFF_BAR && SMEM <= 232448, "shared memory budget");
 enum { V_FWD = 0, V_DO = 1, V_DW = 2, V_QKV = 3, V_DX = 4, V_DWX = 5 };
 
 struct ProjArgs {
@@ -144,24 +152,27 @@ __device__ __forceinline__ void epilogue_qkv_head(const ProjArgs& a, uint32_t ta
 }
 
 template <int V>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 proj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
             const __grid_constant__ CUtensorMap tmA3, const __grid_constant__ CUtensorMap tmB, const ProjArgs a,
             unsigned* status)
 {
     extern __shared__ uint8_t smem_raw[];
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;       // the same offset in both CTAs of a pair
     const uint32_t sA = base + OFF_A, sB = base + OFF_B, bars = base + OFF_BAR;
     const uint32_t tmem_slot = bars + B_COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // tile t: TN output columns from n0; TM rows from r0 (positions s of batch element b, or for DW, DWX rows of d_w)
+    const uint32_t rank = cluster_ctarank();                           // CTA of the pair; the first one issues the products
+    // tile t: TN output columns from n0; for each CTA TM rows from r0 (positions s of batch element b, or for DW, DWX rows of d_w)
     const int HD = a.H * a.D, F = (a.H + 2 * a.Hkv) * a.D;             // features: of the heads of O; of query | key | value
-    const int n_sc = (a.S + TK - 1) / TK;                              // DW, DWX: 64-position slices per batch element
+    constexpr bool WGRAD = V == V_DW || V == V_DWX;
+    const int n_sc = (a.S + TK - 1) / TK;                              // DW, DWX: 64-position pieces per batch element
     const int N = V == V_DO ? HD : V == V_QKV ? F : a.E;
-    const int n_kt = V == V_FWD ? HD / TK : V == V_DX ? F / TK : (V == V_DW || V == V_DWX) ? a.B * n_sc : (a.E + TK - 1) / TK;
+    const int n_kp = V == V_FWD ? HD / TK : V == V_DX ? F / TK : WGRAD ? a.B * n_sc : (a.E + TK - 1) / TK;     // pieces
+    const int n_kt = (n_kp + kPieces - 1) / kPieces;                   // stages a tile takes; the last may hold one piece
     const int rows = V == V_DW ? HD : V == V_DWX ? F : a.S;
+    auto pieces_of = [&](int kt) { return min(kPieces, n_kp - kt * kPieces); };
     // DX, DWX: 64 consecutive features of the concatenation (query | key | value heads) starting at f lie in one
     // head of one of three tensors; `idx` is that head's index in its tensor for batch element bb.  Past the
     // last head the index runs off the value tensor, and the load returns zeros.
@@ -174,21 +185,33 @@ proj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     };
 
     const int tiles_n = (N + TN - 1) / TN, tiles_m = (rows + TM - 1) / TM;
-    const int n_tiles = tiles_n * tiles_m * ((V == V_DW || V == V_DWX) ? 1 : a.B);
-    const int t0 = static_cast<int>(blockIdx.x), dt = static_cast<int>(gridDim.x);
+    const int row_tiles = tiles_m * (WGRAD ? 1 : a.B);
+    const int n_tiles = tiles_n * ((row_tiles + 1) / 2);
+    const int t0 = static_cast<int>(blockIdx.x >> 1), dt = static_cast<int>(gridDim.x >> 1);
+    // An odd number of row tiles leaves the second CTA of the last pairs without one: its batch element b is then
+    // past the last (zeros are loaded and nothing is stored; DW, DWX: rows past the last, of which nothing is stored).
     auto tile_at = [&](int t, int& n0, int& r0, int& b) {
         n0 = (t % tiles_n) * TN;
-        r0 = ((t / tiles_n) % tiles_m) * TM;
-        b = t / (tiles_n * tiles_m);
+        const int rt = 2 * (t / tiles_n) + static_cast<int>(rank);
+        b = WGRAD ? 0 : rt / tiles_m;
+        r0 = (rt - b * tiles_m) * TM;
     };
 
     if (tid == 0) {
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), (i == B_ACCEMPTY || i == B_ACCEMPTY + 1) ? 128 : (i >= B_FULL && i < B_FULL + kStages) ? 2 : 1);
+            mbar_init(bar(i), (i == B_ACCEMPTY || i == B_ACCEMPTY + 1) ? 8 : (i >= B_FULL && i < B_FULL + kStages) ? 2 : 1);
         fence_mbar_init();
+        sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
     }
     __syncwarp();
-    if (warp == 0) tmem_alloc(tmem_slot, 2 * TN);
+    cluster_sync();
+    // Whether an earlier wait on this device gave up: the first CTA's reading counts for both, so that they go on or
+    // end together.
+    if (lds_cluster_u32(cluster_map(tmem_slot + 4, 0)) != 0) {
+        cluster_sync();                                // not before the other has read it
+        return;
+    }
+    if (warp == 0) tmem_alloc_pair(tmem_slot, 2 * TN);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -196,85 +219,93 @@ proj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     if ((warp == 0 || warp == 6) && lane == 0) {
         // ---------------------------------------------------------------- TMA producers
-        // Two lanes, one per operand (warp 0: A, warp 6: B).  A lane's turn per slice is a barrier wait (250-350
-        // clocks while the tensor core streams operands from shared memory) plus up to six copy instructions,
-        // and the products of a slice take 512 clocks: one lane for both operands was the limit of the
-        // variants that fetch their operands in 64-wide blocks.
+        // Two lanes, one per operand (warp 0: A, warp 6: B), since a lane's turn is a barrier wait (250-350 clocks
+        // while the tensor core streams operands from shared memory) plus up to four copy instructions.  Both CTAs'
+        // copies report to the first CTA's barrier, which its lanes arm for the bytes of both.
         const bool opA = warp == 0;
-        int g = 0;                                     // slices loaded so far (all tiles): stage and phase of the ring
+        int g = 0;                                     // stages filled so far (all tiles): stage and phase of the ring
         for (int t = t0; t < n_tiles; t += dt) {
         int n0, r0, b;
         tile_at(t, n0, r0, b);
-        int bb = 0, s0 = 0;                            // DW, DWX: batch element and first position of the slice
+        const int nc = n0 + static_cast<int>(rank) * TNC;                // this CTA's columns of B
+        int bb = 0, s0 = 0;                            // DW, DWX: batch element and first position of the piece
         for (int kt = 0; kt < n_kt; ++kt, ++g) {
-            const int st = g % kStages, k0 = kt * TK;
+            const int st = g % kStages, np = pieces_of(kt);
             if (g >= kStages) mbar_wait(bar(B_EMPTY + st), ((g / kStages) - 1) & 1, status);
-            mbar_arrive_expect_tx(bar(B_FULL + st), opA ? A_BYTES : B_BYTES);
-            const uint32_t dA = sA + st * A_BYTES, dB = sB + st * B_BYTES, full = bar(B_FULL + st);
-            if constexpr (V == V_DO || V == V_QKV) {
-                if (opA) tma_load_3d(dA, &tmA, full, k0, r0, b);                         // 128 positions x 64 e
-                else tma_load_3d(dB, &tmB, full, k0, n0, 0);                             // 256 rows n x 64 e
-            } else if constexpr (V == V_FWD || V == V_DX) {
-                if (opA) {
-                    if constexpr (V == V_FWD) {
-                        tma_load_3d(dA, &tmA, full, k0 % a.D, r0, b * a.H + k0 / a.D);   // 128 positions x 64 d of one head
-                    } else {
-                        int idx;
-                        const CUtensorMap* m = head_of(k0, b, idx);
-                        tma_load_3d(dA, m, full, k0 % a.D, r0, idx);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < TN / 64; ++c)                                     // four blocks of 64 k rows x 64 n
-                        tma_load_3d(dB + c * (TK * 128), &tmB, full, n0 + 64 * c, k0, 0);
-                }
-            } else {
-                if (opA) {
-#pragma unroll
-                    for (int c = 0; c < TM / 64; ++c) {                                   // two blocks of 64 positions x 64 rows m
-                        const int m = r0 + 64 * c;
-                        if constexpr (V == V_DW) {
-                            tma_load_3d(dA + c * (TK * 128), &tmA, full, m % a.D, s0, bb * a.H + m / a.D);
+            if (rank == 0) mbar_arrive_expect_tx(bar(B_FULL + st), 2 * np * (opA ? A_PIECE : B_PIECE));
+            const uint32_t full = cluster_map(bar(B_FULL + st), 0);
+            for (int p = 0; p < np; ++p) {
+                const int k0 = (kt * kPieces + p) * TK;
+                const uint32_t dA = sA + st * A_BYTES + p * A_PIECE, dB = sB + st * B_BYTES + p * B_PIECE;
+                if constexpr (V == V_DO || V == V_QKV) {
+                    if (opA) tma_load_3d_pair(dA, &tmA, full, k0, r0, b);                         // 128 positions x 64 e
+                    else tma_load_3d_pair(dB, &tmB, full, k0, nc, 0);                             // 128 rows n x 64 e
+                } else if constexpr (V == V_FWD || V == V_DX) {
+                    if (opA) {
+                        if constexpr (V == V_FWD) {
+                            tma_load_3d_pair(dA, &tmA, full, k0 % a.D, r0, b * a.H + k0 / a.D);   // 128 positions x 64 d of one head
                         } else {
                             int idx;
-                            const CUtensorMap* mp = head_of(m, bb, idx);
-                            tma_load_3d(dA + c * (TK * 128), mp, full, m % a.D, s0, idx);
+                            const CUtensorMap* m = head_of(k0, b, idx);
+                            tma_load_3d_pair(dA, m, full, k0 % a.D, r0, idx);
                         }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < TNC / 64; ++c)                                        // two blocks of 64 k rows x 64 n
+                            tma_load_3d_pair(dB + c * (TK * 128), &tmB, full, nc + 64 * c, k0, 0);
                     }
                 } else {
+                    if (opA) {
 #pragma unroll
-                    for (int c = 0; c < TN / 64; ++c)                                     // four blocks of 64 positions x 64 e
-                        tma_load_3d(dB + c * (TK * 128), &tmB, full, n0 + 64 * c, s0, bb);
+                        for (int c = 0; c < TM / 64; ++c) {                                       // two blocks of 64 positions x 64 rows m
+                            const int m = r0 + 64 * c;
+                            if constexpr (V == V_DW) {
+                                tma_load_3d_pair(dA + c * (TK * 128), &tmA, full, m % a.D, s0, bb * a.H + m / a.D);
+                            } else {
+                                int idx;
+                                const CUtensorMap* mp = head_of(m, bb, idx);
+                                tma_load_3d_pair(dA + c * (TK * 128), mp, full, m % a.D, s0, idx);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < TNC / 64; ++c)                                        // two blocks of 64 positions x 64 e
+                            tma_load_3d_pair(dB + c * (TK * 128), &tmB, full, nc + 64 * c, s0, bb);
+                    }
+                    s0 += TK;                          // pieces run over the positions of batch element 0, then 1, ...
+                    if (s0 >= n_sc * TK) { s0 = 0; ++bb; }
                 }
-                s0 += TK;                              // slices run over the positions of batch element 0, then 1, ...
-                if (s0 >= n_sc * TK) { s0 = 0; ++bb; }
             }
         }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------------------------------------------------------- MMA issuer
-        constexpr bool A_MN = V == V_DW || V == V_DWX, B_MN = V == V_FWD || V == V_DW || V == V_DX || V == V_DWX;
-        constexpr uint32_t idesc = umma_idesc_bf16(TM, TN, A_MN, B_MN);
+        // the stages' last releases arrive from the other CTA's products: not after this CTA has gone
+        for (int j = max(0, g - kStages); j < g; ++j) mbar_wait(bar(B_EMPTY + j % kStages), (j / kStages) & 1, status);
+    } else if (warp == 1 && lane == 0 && rank == 0) {
+        // ---------------------------------------------------------------- MMA issuer (for both CTAs)
+        constexpr bool A_MN = WGRAD, B_MN = V == V_FWD || V == V_DX || WGRAD;
+        constexpr uint32_t idesc = umma_idesc_bf16(2 * TM, TN, A_MN, B_MN);
         const uint64_t dA = A_MN ? umma_smem_desc(sA, TK * 128, 1024) : umma_smem_desc(sA, 16, 1024);
         const uint64_t dB = B_MN ? umma_smem_desc(sB, TK * 128, 1024) : umma_smem_desc(sB, 16, 1024);
-        int g = 0, ti = 0;                             // slices and tiles so far
+        int g = 0, ti = 0;                             // stages and tiles so far
         for (int t = t0; t < n_tiles; t += dt, ++ti) {
             const int acc = ti & 1;
-            mbar_wait(bar(B_ACCEMPTY + acc), ((ti >> 1) & 1) ^ 1, status);   // the tile two back has been read out
+            mbar_wait_cluster(bar(B_ACCEMPTY + acc), ((ti >> 1) & 1) ^ 1, status);   // the tile two back has been read out, by both
             tc_fence_after();
             for (int kt = 0; kt < n_kt; ++kt, ++g) {
-                const int st = g % kStages;
+                const int st = g % kStages, np = pieces_of(kt);
                 mbar_wait(bar(B_FULL + st), (g / kStages) & 1, status);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < TK / 16; ++kk) {
-                    const uint64_t da = dA + static_cast<uint64_t>((st * A_BYTES + (A_MN ? kk * 2048 : kk * 32)) >> 4);
-                    const uint64_t db = dB + static_cast<uint64_t>((st * B_BYTES + (B_MN ? kk * 2048 : kk * 32)) >> 4);
-                    umma_ss(tmem + acc * TN, da, db, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 0; kk < kPieces * TK / 16; ++kk) {
+                    const int p = kk / (TK / 16), q = kk % (TK / 16);
+                    if (p >= np) break;
+                    const uint64_t da = dA + static_cast<uint64_t>((st * A_BYTES + p * A_PIECE + (A_MN ? q * 2048 : q * 32)) >> 4);
+                    const uint64_t db = dB + static_cast<uint64_t>((st * B_BYTES + p * B_PIECE + (B_MN ? q * 2048 : q * 32)) >> 4);
+                    umma_ss_pair(tmem + acc * TN, da, db, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
                 }
-                umma_commit(bar(B_EMPTY + st));
+                umma_commit_pair(bar(B_EMPTY + st));
             }
-            umma_commit(bar(B_ACCFULL + acc));
+            umma_commit_pair(bar(B_ACCFULL + acc));
         }
     } else if (warp >= 2 && warp < 6) {
         // ---------------------------------------------------------------- epilogue: one thread per row
@@ -284,16 +315,17 @@ proj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         int n0, r0, b;
         tile_at(t, n0, r0, b);
         const int row = r0 + r, acc = ti & 1;
+        const bool row_ok = row < rows && b < a.B;
         const uint32_t tacc = tmem + (static_cast<uint32_t>(32 * q4) << 16) + acc * TN;
         mbar_wait(bar(B_ACCFULL + acc), (ti >> 1) & 1, status);
         tc_fence_after();
         if constexpr (V == V_QKV) {
             if (a.D == 128) {
 #pragma unroll 1
-                for (int hh = 0; hh < TN / 128; ++hh) epilogue_qkv_head<128>(a, tacc + 128 * hh, b, row, n0 / 128 + hh, row < rows);
+                for (int hh = 0; hh < TN / 128; ++hh) epilogue_qkv_head<128>(a, tacc + 128 * hh, b, row, n0 / 128 + hh, row_ok);
             } else {
 #pragma unroll 1
-                for (int hh = 0; hh < TN / 64; ++hh) epilogue_qkv_head<64>(a, tacc + 64 * hh, b, row, n0 / 64 + hh, row < rows);
+                for (int hh = 0; hh < TN / 64; ++hh) epilogue_qkv_head<64>(a, tacc + 64 * hh, b, row, n0 / 64 + hh, row_ok);
             }
         } else {
             float dl = 0.f;
@@ -303,16 +335,18 @@ proj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 tmem_ld32(tacc + 32 * c, v);          // whole warp, whatever the row
                 tmem_ld_wait();
                 const int n = n0 + 32 * c;
-                if (row < rows && n < N) epilogue_plain<V>(a, v, b, row, n, dl);
+                if (row_ok && n < N) epilogue_plain<V>(a, v, b, row, n, dl);
             }
         }
         tc_fence_before();
-        mbar_arrive(bar(B_ACCEMPTY + acc));             // this accumulator may be overwritten
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(cluster_map(bar(B_ACCEMPTY + acc), 0));     // this accumulator may be overwritten
         }
     }
     tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 2 * TN);
+    __syncwarp();
+    cluster_sync();                                    // neither CTA leaves while the other's products read its tiles
+    if (warp == 0) tmem_dealloc_pair(tmem, 2 * TN);
 }
 
 template <int V>
@@ -325,14 +359,14 @@ cudaError_t launch3(const CUtensorMap& ta, const CUtensorMap& ta2, const CUtenso
     const int F = (a.H + 2 * a.Hkv) * a.D;
     const int N = V == V_DO ? a.H * a.D : V == V_QKV ? F : a.E;
     const int rows = V == V_DW ? a.H * a.D : V == V_DWX ? F : a.S;
-    const long long tiles = static_cast<long long>((N + TN - 1) / TN) * ((rows + TM - 1) / TM) *
-                            ((V == V_DW || V == V_DWX) ? 1 : a.B);
+    const long long row_tiles = static_cast<long long>((rows + TM - 1) / TM) * ((V == V_DW || V == V_DWX) ? 1 : a.B);
+    const long long tiles = static_cast<long long>((N + TN - 1) / TN) * ((row_tiles + 1) / 2);
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms <= 0 || tiles > 0x7fffffffLL)
+        sms <= 1 || tiles > 0x3fffffffLL)
         return cudaErrorInvalidValue;
-    const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);     // persistent: one CTA per SM
-    kern<<<grid, kThreads, SMEM, st>>>(ta, ta2, ta3, tb, a, status);
+    const unsigned pairs = static_cast<unsigned>(tiles < sms / 2 ? tiles : sms / 2);     // persistent: one CTA per SM
+    kern<<<2 * pairs, kThreads, SMEM, st>>>(ta, ta2, ta3, tb, a, status);
     return cudaGetLastError();
 }
 template <int V>
@@ -393,7 +427,7 @@ cudaError_t launch_out_proj_bwd_data(const void* d_y, const void* w, const void*
 {
     CUtensorMap ta, tb;
     if (make_tmap_3d(&ta, d_y, 2, 1, B, S, E, 64, TM)) return cudaErrorInvalidValue;
-    if (make_tmap_3d(&tb, w, 2, 1, 1, H * D, E, 64, TN)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tb, w, 2, 1, 1, H * D, E, 64, TNC)) return cudaErrorInvalidValue;
     ProjArgs a{static_cast<__nv_bfloat16*>(d_o), nullptr, nullptr, static_cast<const __nv_bfloat16*>(o), delta, nullptr,
                nullptr, B, H, H, S, D, E};
     return launch<V_DO>(ta, tb, a, status, st);
@@ -414,7 +448,7 @@ cudaError_t launch_qkv_rope(const void* x, const void* w, const float* cos_t, co
 {
     CUtensorMap ta, tb;
     if (make_tmap_3d(&ta, x, 2, 1, B, S, E, 64, TM)) return cudaErrorInvalidValue;
-    if (make_tmap_3d(&tb, w, 2, 1, 1, (H + 2 * Hkv) * D, E, 64, TN)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tb, w, 2, 1, 1, (H + 2 * Hkv) * D, E, 64, TNC)) return cudaErrorInvalidValue;
     ProjArgs a{static_cast<__nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(k), static_cast<__nv_bfloat16*>(v), nullptr,
                nullptr, cos_t, sin_t, B, H, Hkv, S, D, E};
     return launch<V_QKV>(ta, tb, a, status, st);

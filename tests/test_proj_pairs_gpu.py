@@ -1,0 +1,57 @@
+"""The projection kernel's pairs of CTAs (csrc/proj.cu) at several tiles per pair: an odd number of 128-row tiles over the
+batch, so that the last pair has one tile and pairs span batch elements, column tiles past the last column, a contraction
+whose last stage holds one 64-wide piece."""
+import math
+
+import pytest
+import torch
+
+from oracle import attn_oracle as orc
+from paper_2608_01563_b200 import binding as mgn
+
+import helpers as hp
+
+pytestmark = pytest.mark.gpu
+MODE, BF = mgn.MODE_FAST_BF16, torch.bfloat16
+
+
+def _close(got, ref):
+    err = hp.rel_l2(got.double().numpy(), ref)
+    assert err <= hp.FAST_REL_L2, err
+
+
+@pytest.mark.parametrize("B,S,E,H,Hkv,D", [(3, 900, 72, 16, 16, 128),      # QKV: 12 pairs x 24 column tiles, two pieces
+                                            (5, 129, 4104, 3, 1, 64)])      # out-projection: 5 pairs x 17 column tiles, three pieces
+def test_all_products(B, S, E, H, Hkv, D):
+    g = torch.Generator().manual_seed(S)
+    x, d_y = (torch.randn(B, S, E, generator=g).to(BF) for _ in range(2))
+    w_qkv = (torch.randn((H + 2 * Hkv) * D, E, generator=g) / math.sqrt(E)).to(BF)
+    w_o = (torch.randn(H * D, E, generator=g) / math.sqrt(H * D)).to(BF)
+    o, gq = (torch.randn(B, H, S, D, generator=g).to(BF) for _ in range(2))
+    gk, gv = (torch.randn(B, Hkv, S, D, generator=g).to(BF) for _ in range(2))
+    cos_t, sin_t = torch.ones(S, D // 2), torch.zeros(S, D // 2)
+    f64 = lambda t: t.double().numpy()
+    xd, dyd, wqd, wod, od, gqd, gkd, gvd = (t.cuda() for t in (x, d_y, w_qkv, w_o, o, gq, gk, gv))
+
+    q, k, v = (hp.Guarded((B, h, S, D), BF) for h in (H, Hkv, Hkv))
+    mgn.mgn_qkv_rope_fwd(xd, wqd, cos_t.cuda(), sin_t.cuda(), q.view, k.view, v.view, MODE)
+    y, d_o, delta = hp.Guarded((B, S, E), BF), hp.Guarded((B, H, S, D), BF), hp.Guarded((B, H, S), torch.float32)
+    mgn.mgn_out_proj_fwd(od, wod, y.view, MODE)
+    mgn.mgn_out_proj_bwd_data(dyd, wod, od, d_o.view, delta.view, MODE)
+    d_wo, d_x, d_wqkv = hp.Guarded((H * D, E), BF), hp.Guarded((B, S, E), BF), hp.Guarded(((H + 2 * Hkv) * D, E), BF)
+    mgn.mgn_out_proj_bwd_weight(od, dyd, d_wo.view, MODE)
+    mgn.mgn_qkv_bwd_data(gqd, gkd, gvd, wqd, d_x.view, MODE)
+    mgn.mgn_qkv_bwd_weight(gqd, gkd, gvd, xd, d_wqkv.view, MODE)
+    mgn.mgn_attn_check()
+
+    c64, s64 = f64(cos_t), f64(sin_t)
+    for got, ref in zip((q, k, v), orc.qkv_rope(f64(x), f64(w_qkv), c64, s64, H, Hkv, D)):
+        _close(got.check("QKV"), ref)
+    _close(y.check("Y"), orc.out_proj_fwd(f64(o), f64(w_o)))
+    r_do, r_delta, r_dwo = orc.out_proj_bwd(f64(d_y), f64(w_o), f64(o))
+    _close(d_o.check("dO"), r_do)
+    _close(delta.check("delta"), r_delta)
+    _close(d_wo.check("dWo"), r_dwo)
+    rdx, rdw, _ = orc.qkv_rope_bwd(f64(gq), f64(gk), f64(gv), f64(x), f64(w_qkv), c64, s64)
+    _close(d_x.check("dX"), rdx)
+    _close(d_wqkv.check("dWqkv"), rdw)
