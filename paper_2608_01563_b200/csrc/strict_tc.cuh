@@ -48,13 +48,10 @@ inline ScoreFactor score_factor(float scale, int D) {
     return {hi, static_cast<float>(c - hi), static_cast<float>(ldexp(1.0, e)), static_cast<float>(1.0 / log2e)};
 }
 
-// x * (c_hi + c_lo), rounded once; two values an instruction.
+// x * (c_hi + c_lo), rounded once.
+__device__ __forceinline__ float scaled(float x, float c_hi, float c_lo) { return fmaf(x, c_hi, x * c_lo); }
 __device__ __forceinline__ float4 scaled(float4 x, float c_hi, float c_lo) {
-    const uint64_t hi = f2_pack(c_hi, c_hi), lo = f2_pack(c_lo, c_lo);
-    const uint64_t a = f2_pack(x.x, x.y), b = f2_pack(x.z, x.w);
-    f2_unpack(f2_fma(a, hi, f2_mul(a, lo)), x.x, x.y);
-    f2_unpack(f2_fma(b, hi, f2_mul(b, lo)), x.z, x.w);
-    return x;
+    return make_float4(scaled(x.x, c_hi, c_lo), scaled(x.y, c_hi, c_lo), scaled(x.z, c_hi, c_lo), scaled(x.w, c_hi, c_lo));
 }
 
 // A pair of f32 (a in the low half) -> three packed bf16 pairs.  hi saturates: a finite x near the end of the range
@@ -132,30 +129,28 @@ struct Converter {
     float4 buf[NQ];
     uint32_t off[NQ];         // where they go in a slot of an operand tile
     int row, quad;
-    const float* g;           // this thread's first quad of the slot in buf
-    int rows;                 // rows that exist from the slot's first one on
+    float c_hi, c_lo;         // SCALED: what the values are multiplied by
 
-    // Asks for the first slot, of the tile at `tile`, of which `n_rows` rows exist: before a CTA sets itself up, so that the
-    // two latencies overlap.
-    __device__ __forceinline__ void start(int t, const float* tile, int n_rows) {
-        row = t / QUADS;
-        quad = t % QUADS;
-        g = tile + row * D + quad * 4;
-        rows = n_rows;
+    __device__ __forceinline__ explicit Converter(int t, float hi = 1.f, float lo = 0.f)
+        : row(t / QUADS), quad(t % QUADS), c_hi(hi), c_lo(lo) {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            off[k] = quad_offset<R>(row + k * STEP, quad);
+        }
+    }
+    // Converts tiles 0 .. n-1.  src(i, rows) gives the first row of tile i and how many rows exist from there;
+    // dst(i) waits until the tile's stage is free and returns its address; done(i) follows the stores.
+    template <class Src, class Dst, class Done>
+    __device__ __forceinline__ void run(int n, Src src, Dst dst, Done done) {
+        int rows;
+        const float* g = src(0, rows) + row * D + quad * 4;
+        auto load = [&](int k) {
+            const int r = row + k * STEP;
+            buf[k] = r < min(rows, SLOT_ROWS) ? __ldg(reinterpret_cast<const float4*>(g + k * STEP * D))
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
 #pragma unroll
         for (int k = 0; k < NQ; ++k) load(k);
-    }
-    __device__ __forceinline__ void load(int k) {
-        const int r = row + k * STEP;
-        buf[k] = r < min(rows, SLOT_ROWS) ? __ldg(reinterpret_cast<const float4*>(g + k * STEP * D)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    // Converts tiles 0 .. n-1; the first one has been started.  src(i, rows) gives the first row of tile i and how many rows
-    // exist from there; dst(i) waits until the tile's stage is free and returns its address; done(i) follows the stores.
-    // SCALED: the values are multiplied by c_hi + c_lo.
-    template <class Src, class Dst, class Done>
-    __device__ __forceinline__ void run(int n, float c_hi, float c_lo, Src src, Dst dst, Done done) {
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) off[k] = quad_offset<R>(row + k * STEP, quad);
         uint32_t d = 0;
         int sl = 0, i = 0;
 #pragma unroll 1
@@ -338,41 +333,39 @@ template <int N> __device__ __forceinline__ void store_half_parts(uint32_t x, in
 // Sets of D[128 x R] = A B^T over D columns, at tensor-memory column d; B a split tile of R rows.  A in tensor
 // memory (part p at a + p * D / 2) or a split tile of 128 rows (a: its descriptor).  SCORE: see term().
 template <bool SCORE, int D, int R, int ST, typename A>
-__device__ __forceinline__ void issue_scores(uint32_t leader, uint32_t d, A a_at, uint64_t b_desc) {
+__device__ __forceinline__ void issue_scores(uint32_t d, A a_at, uint64_t b_desc) {
 #pragma unroll 1
     for (int t = 0; t < n_terms<SCORE, ST>(); ++t) {
         const Term m = term<SCORE, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, R, false, false) + (m.n - 1) * ((R >> 3) << 17);
-        const uint64_t b = desc_at(b_desc, m.b * part_bytes<R>());
+        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
         const uint32_t dt = d + m.set * R;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t bk = desc_at(b, (kk >> 2) * block_bytes<R>() + (kk & 3) * 32);
+            const uint64_t bk = b + (((kk >> 2) * block_bytes<R>() + (kk & 3) * 32) >> 4);
             const uint32_t add = (t > 0 || kk > 0) ? 1u : 0u;
-            if constexpr (sizeof(A) == 4) umma_ts_warp(leader, dt, a_at + m.a * (D / 2) + kk * 8, bk, idesc, add);
-            else umma_ss_warp(leader, dt, desc_at(a_at, m.a * part_bytes<128>() + (kk >> 2) * block_bytes<128>() + (kk & 3) * 32), bk, idesc, add);
+            if constexpr (sizeof(A) == 4) umma_ts(dt, a_at + m.a * (D / 2) + kk * 8, bk, idesc, add);
+            else umma_ss(dt, a_at + ((m.a * part_bytes<128>() + (kk >> 2) * block_bytes<128>() + (kk & 3) * 32) >> 4), bk, idesc, add);
         }
     }
 }
-// 16-row steps of a block of R rows of which `rows` exist.
-template <int R> __device__ __forceinline__ int row_steps(int rows) { return (min(rows, R) + 15) >> 4; }
-// Sets of D[128 x D] = X B over the first 16 `steps` rows of the split tile B (as MN-major operand, see rows_desc; the
-// rows behind are past the end of their sequence and would add zeros), X the parts in a region of scores.  Stacking (ST = 2) needs adjacent parts to be D columns apart: D = 64.
+// Sets of D[128 x D] = X B over the R rows of the split tile B (as MN-major operand, see rows_desc), X the parts
+// in a region of scores.  Stacking (ST = 2) needs adjacent parts to be D columns apart: D = 64.
 template <int D, int R> __device__ __forceinline__ uint64_t rows_desc(uint32_t tile) {
     return umma_smem_desc(tile, D == 64 ? part_bytes<R>() : block_bytes<R>(), 1024);
 }
 template <int D, int R, int ST>
-__device__ __forceinline__ void issue_rows(uint32_t leader, uint32_t d, uint32_t x, uint64_t b_desc, int steps) {
+__device__ __forceinline__ void issue_rows(uint32_t d, uint32_t x, uint64_t b_desc) {
     static_assert(ST == 1 || D == 64, "");
 #pragma unroll 1
     for (int t = 0; t < n_terms<false, ST>(); ++t) {
         const Term m = term<false, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, D, false, true) + (m.n - 1) * ((D >> 3) << 17);
-        const uint64_t b = desc_at(b_desc, m.b * part_bytes<R>());
+        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
         const uint32_t dt = d + m.set * D;
 #pragma unroll
         for (int kk = 0; kk < R / 16; ++kk)
-            umma_ts_warp(kk < steps ? leader : 0u, dt, x + x_part_col<R>(m.a, kk), desc_at(b, kk * 2048), idesc, (t > 0 || kk > 0) ? 1u : 0u);
+            umma_ts(dt, x + x_part_col<R>(m.a, kk), b + ((kk * 2048) >> 4), idesc, (t > 0 || kk > 0) ? 1u : 0u);
     }
 }
 

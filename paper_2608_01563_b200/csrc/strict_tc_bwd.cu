@@ -190,7 +190,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_launch_dependents();                               // the dQ kernel may fill SMs as this one drains
 
     // First key blocks first: under a causal mask they see the most queries.
@@ -201,20 +201,6 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const int m0 = causal ? max(0, j0 - off) / R : 0;      // first query block that sees a key of this block
     const int n_m = (Sq + R - 1) / R - m0;
     const int n_blk = n_m * G;
-
-    // Own rows and the first streamed tile are asked for before the set-up (at D = 128 registers allow one own tensor).
-    const int t_own = tid - 256;
-    const size_t own_at = (static_cast<size_t>(bhk) * Sk + j0) * D;
-    const bool is_q = warp < 5;                            // converter warps: Q (and statistics), or dO
-    const float* const streamed = is_q ? Q : dO;
-    Converter<D, R, true> cv;
-    OwnRows<D> kr, vr;
-    if (warp >= 8) {
-        vr.load(V + own_at, Sk - j0, t_own);
-        if constexpr (D == 64) kr.load(K + own_at, Sk - j0, t_own);
-    } else if (warp >= 2) {
-        cv.start(tid - (is_q ? 64 : 160), streamed + (static_cast<size_t>(bhk) * G * Sq + static_cast<size_t>(m0) * R) * D, Sq - m0 * R);
-    }
 
     if (tid == 0) {
         for (int w = 0; w < 2; ++w) {
@@ -236,7 +222,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
+    const uint32_t tmem = lds32u(tmem_slot);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
@@ -246,67 +232,69 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
         if (warp == 0) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- S^T and dP^T
-            const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024), dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
-            const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024);
-            [[maybe_unused]] const uint64_t dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
-            if (leader) mbar_arrive(bar(C::S_GO));
-            if (leader) mbar_arrive(bar(C::P_GO));
-            mbar_wait(bar(C::KV), 0, status);
+            if (lane == 0) {
+                // -------------------------------------------------------------- S^T and dP^T
+                const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024), dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
+                const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024);
+                [[maybe_unused]] const uint64_t dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
+                mbar_arrive(bar(C::S_GO));
+                mbar_arrive(bar(C::P_GO));
+                mbar_wait(bar(C::KV), 0, status);
 #pragma unroll 1
-            for (int n = 0; n < n_blk; ++n) {
-                const int w = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                mbar_wait(bar(C::S_GO + w), ph, status);
-                tc_fence_after();
-                issue_scores<true, D, R, C::ST>(leader, tmem + C::TM_X, dKd, dQd + so);
-                umma_commit_warp(leader, bar(C::S_DONE));
-                mbar_wait(bar(C::P_GO + w), ph, status);
-                tc_fence_after();
-                if constexpr (C::V_TMEM) issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, tmem + C::TM_V, dOd + so);
-                else issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, dVd, dOd + so);
-                umma_commit_warp(leader, bar(C::P_DONE));
+                for (int n = 0; n < n_blk; ++n) {
+                    const int w = n & 1;
+                    const uint32_t ph = (n >> 1) & 1;
+                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                    mbar_wait(bar(C::S_GO + w), ph, status);
+                    tc_fence_after();
+                    issue_scores<true, D, R, C::ST>(tmem + C::TM_X, dKd, dQd + so);
+                    umma_commit(bar(C::S_DONE));
+                    mbar_wait(bar(C::P_GO + w), ph, status);
+                    tc_fence_after();
+                    if constexpr (C::V_TMEM) issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, tmem + C::TM_V, dOd + so);
+                    else issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, dVd, dOd + so);
+                    umma_commit(bar(C::P_DONE));
+                }
             }
             __syncwarp();
         } else if (warp == 1) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- dV and dK results
-            const uint64_t mQ = rows_desc<D, R>(base + C::OFF_Q), mO = rows_desc<D, R>(base + C::OFF_DO);
-            int m = 0;                                     // query block of the current head
+            if (lane == 0) {
+                // -------------------------------------------------------------- dV and dK results
+                const uint64_t mQ = rows_desc<D, R>(base + C::OFF_Q), mO = rows_desc<D, R>(base + C::OFF_DO);
 #pragma unroll 1
-            for (int n = 0; n < n_blk; ++n) {
-                const int w = n & 1;
-                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                const int steps = row_steps<R>(Sq - (m0 + m) * R);
-                if (++m == n_m) m = 0;
-                mbar_wait(bar(C::V_GO + w), (n >> 1) & 1, status);
-                tc_fence_after();
-                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_ZV, tmem + C::TM_X, mO + so, steps);
-                umma_commit_warp(leader, bar(C::V_DONE));
-                umma_commit_warp(leader, bar(C::S_GO + (w ^ 1)));
-                mbar_wait(bar(C::K_GO), n & 1, status);
-                tc_fence_after();
-                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so, steps);
-                umma_commit_warp(leader, bar(C::K_DONE + w));       // both products of the block: its tiles are free too
-                umma_commit_warp(leader, bar(C::P_GO + (w ^ 1)));
+                for (int n = 0; n < n_blk; ++n) {
+                    const int w = n & 1;
+                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                    mbar_wait(bar(C::V_GO + w), (n >> 1) & 1, status);
+                    tc_fence_after();
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZV, tmem + C::TM_X, mO + so);
+                    umma_commit(bar(C::V_DONE));
+                    umma_commit(bar(C::S_GO + (w ^ 1)));
+                    mbar_wait(bar(C::K_GO), n & 1, status);
+                    tc_fence_after();
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so);
+                    umma_commit(bar(C::K_DONE + w));       // both products of the block: its tiles are free too
+                    umma_commit(bar(C::P_GO + (w ^ 1)));
+                }
             }
             __syncwarp();
         } else {
             // ------------------------------------------------------------------ Q (and statistics), dO
+            const bool is_q = warp < 5;
             const int t = tid - (is_q ? 64 : 160);
+            const float* src = is_q ? Q : dO;
             const uint32_t stages = base + (is_q ? C::OFF_Q : C::OFF_DO);
             auto rows_of = [&](int n, int& g, int& i0) {   // n -> query head of the group, first query
                 g = n / n_m;
                 i0 = (m0 + n - g * n_m) * R;
             };
-            cv.run(n_blk, is_q ? c.hi : 1.f, is_q ? c.lo : 0.f,
+            Converter<D, R, true> cv(t, is_q ? c.hi : 1.f, is_q ? c.lo : 0.f);
+            cv.run(n_blk,
                    [&](int n, int& rows) {
                        int g, i0;
                        rows_of(n, g, i0);
                        rows = Sq - i0;
-                       return streamed + (static_cast<size_t>(bhk) * G + g) * Sq * D + static_cast<size_t>(i0) * D;
+                       return src + (static_cast<size_t>(bhk) * G + g) * Sq * D + static_cast<size_t>(i0) * D;
                    },
                    [&](int n) {
                        if (n >= 2) mbar_wait(bar(C::K_DONE + (n & 1)), ((n >> 1) & 1) ^ 1, status);
@@ -345,9 +333,12 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
         const uint32_t tl = tmem + lane_base;
         const int j = j0 + r;
-        const int t = t_own;
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bhk) * Sk + j0) * D;
         {
-            if constexpr (D != 64) kr.load(K + own_at, Sk - j0, t);
+            OwnRows<D> kr, vr;
+            vr.load(V + own_at, Sk - j0, t);
+            kr.load(K + own_at, Sk - j0, t);
             if constexpr (C::V_TMEM) {                     // by way of K's place
                 vr.to_exchange(base + C::OFF_K, t);
                 named_bar_sync(1, kCompute);
@@ -532,7 +523,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Heaviest (last) query tiles first when causal.
     const int item = static_cast<int>(blockIdx.x) / splits, part = static_cast<int>(blockIdx.x) % splits;
@@ -550,20 +541,6 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     if (n_blk <= 0) {
         pdl_wait();
         return;
-    }
-
-    // Own rows and the first streamed tile are asked for before the set-up.
-    const int t_own = tid - 256;
-    const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
-    const bool is_k = warp < 5;                            // converter warps: K, or V
-    const float* const head = (is_k ? K : V) + static_cast<size_t>(bhk) * Sk * D;
-    Converter<D, R> cv;
-    OwnRows<D> qr, orr;
-    if (warp >= 8) {
-        orr.load(dO + own_at, Sq - i0, t_own);
-        if constexpr (D == 64) qr.load(Q + own_at, Sq - i0, t_own);
-    } else if (warp >= 2) {
-        cv.start(tid - (is_k ? 64 : 160), head + static_cast<size_t>(b0) * R * D, Sk - b0 * R);
     }
 
     if (tid == 0) {
@@ -584,7 +561,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
+    const uint32_t tmem = lds32u(tmem_slot);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
@@ -595,51 +572,56 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
         if (warp == 0) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- S and dP
-            const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024), dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
-            const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024);
-            [[maybe_unused]] const uint64_t dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
-            if (leader) mbar_arrive(bar(C::S_GO));
-            if (leader) mbar_arrive(bar(C::S_GO + 1));
-            mbar_wait(bar(C::QDO), 0, status);
+            if (lane == 0) {
+                // -------------------------------------------------------------- S and dP
+                const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024), dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
+                const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024);
+                [[maybe_unused]] const uint64_t dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
+                mbar_arrive(bar(C::S_GO));
+                mbar_arrive(bar(C::S_GO + 1));
+                mbar_wait(bar(C::QDO), 0, status);
 #pragma unroll 1
-            for (int n = 0; n < n_blk; ++n) {
-                const int w = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                const uint32_t x = tmem + C::TM_X + w * C::X;
-                mbar_wait(bar(C::S_GO + w), ph, status);
-                tc_fence_after();
-                issue_scores<true, D, R, C::ST>(leader, x, dQd, dKd + so);
-                umma_commit_warp(leader, bar(C::S_DONE + w));
-                mbar_wait(bar(C::P_GO + w), ph, status);
-                tc_fence_after();
-                if constexpr (C::DO_TMEM) issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, tmem + C::TM_DO, dVd + so);
-                else issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, dOd, dVd + so);
-                umma_commit_warp(leader, bar(C::P_DONE));
+                for (int n = 0; n < n_blk; ++n) {
+                    const int w = n & 1;
+                    const uint32_t ph = (n >> 1) & 1;
+                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                    const uint32_t x = tmem + C::TM_X + w * C::X;
+                    mbar_wait(bar(C::S_GO + w), ph, status);
+                    tc_fence_after();
+                    issue_scores<true, D, R, C::ST>(x, dQd, dKd + so);
+                    umma_commit(bar(C::S_DONE + w));
+                    mbar_wait(bar(C::P_GO + w), ph, status);
+                    tc_fence_after();
+                    if constexpr (C::DO_TMEM) issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, tmem + C::TM_DO, dVd + so);
+                    else issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, dOd, dVd + so);
+                    umma_commit(bar(C::P_DONE));
+                }
             }
             __syncwarp();
         } else if (warp == 1) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- dQ results
-            const uint64_t mK = rows_desc<D, R>(base + C::OFF_K);
+            if (lane == 0) {
+                // -------------------------------------------------------------- dQ results
+                const uint64_t mK = rows_desc<D, R>(base + C::OFF_K);
 #pragma unroll 1
-            for (int n = 0; n < n_blk; ++n) {
-                const int w = n & 1;
-                mbar_wait(bar(C::Q_GO), n & 1, status);
-                tc_fence_after();
-                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
-                                    mK + static_cast<uint64_t>((w * C::STAGE) >> 4), row_steps<R>(Sk - (b0 + n) * R));
-                umma_commit_warp(leader, bar(C::Z_DONE + w));       // S, dP (whose results it was formed from) and dQ: tiles free
-                umma_commit_warp(leader, bar(C::S_GO + w));
+                for (int n = 0; n < n_blk; ++n) {
+                    const int w = n & 1;
+                    mbar_wait(bar(C::Q_GO), n & 1, status);
+                    tc_fence_after();
+                    issue_rows<D, R, C::STZ>(tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
+                                        mK + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                    umma_commit(bar(C::Z_DONE + w));       // S, dP (whose results it was formed from) and dQ: tiles free
+                    umma_commit(bar(C::S_GO + w));
+                }
             }
             __syncwarp();
         } else {
             // ------------------------------------------------------------------ K, V
+            const bool is_k = warp < 5;
+            const float* head = (is_k ? K : V) + static_cast<size_t>(bhk) * Sk * D;
             const uint32_t stages = base + (is_k ? C::OFF_K : C::OFF_V);
             const int go = is_k ? C::S_GO : C::P_GO;
-            cv.run(n_blk, 1.f, 0.f,
+            Converter<D, R> cv(tid - (is_k ? 64 : 160));
+            cv.run(n_blk,
                    [&](int n, int& rows) {
                        rows = Sk - (b0 + n) * R;
                        return head + static_cast<size_t>(b0 + n) * R * D;
@@ -658,10 +640,13 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
         const uint32_t tl = tmem + (static_cast<uint32_t>(r & ~31) << 16);
         const int i = i0 + r;
         const bool row_ok = i < Sq;
-        const int t = t_own;
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
         mbar_arrive(bar(C::P_GO));                         // block 0 has no dP before it
         {
-            if constexpr (D != 64) qr.load(Q + own_at, Sq - i0, t);
+            OwnRows<D> qr, orr;
+            orr.load(dO + own_at, Sq - i0, t);
+            qr.load(Q + own_at, Sq - i0, t);
             if constexpr (C::DO_TMEM) {                    // by way of Q's place
                 orr.to_exchange(base + C::OFF_Q, t);
                 named_bar_sync(1, kCompute);

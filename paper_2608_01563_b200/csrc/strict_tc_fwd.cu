@@ -18,10 +18,6 @@
 // product also tells the converters that its stage is free.  (One lane with a barrier per condition: 512
 // queries over 4096 keys, D = 128, 0.213 ms.)
 // Tensor memory: Q parts 3 D/2 columns, two score regions, one P V result.
-//   Grouped heads are packed where that saves tiles, and a tile's key blocks are dealt to a cluster of CTAs where few
-// tiles leave SMs idle (SPLIT), both as in fast_fwd.cu.  The CTAs of a cluster leave their unnormalised sums in their
-// exchange tiles; maxima are whole numbers, so the factors that put them together are exact.
-#include "parts.cuh"
 #include "strict_tc.cuh"
 
 namespace mgn {
@@ -39,7 +35,7 @@ struct Cfg {
     static constexpr int OFF_K = 0, OFF_V = NST * STAGE, OFF_EX = 2 * NST * STAGE,
                          OFF_BAR = OFF_EX + 128 * OwnRows<D>::PITCH + 2 * 128 * 4;      // exchange tile, row statistics
     static constexpr int SMEM = OFF_BAR + 512 + 1024;
-    static_assert(SMEM <= 232448 && kPartsScratch <= OFF_EX, "shared memory budget");
+    static_assert(SMEM <= 232448, "shared memory budget");
     static constexpr int ST = D == 64 ? 2 : 3, STO = D == 64 ? 2 : 1;       // column sets of scores, of results
     static constexpr uint32_t X = x_cols<R, ST>();
     static constexpr uint32_t TM_Q = 0, TM_X = 3 * D / 2, TM_O = TM_X + 2 * X;
@@ -54,7 +50,7 @@ struct Cfg {
 // against 0.18 for finite inputs and 0.86 of the FFMA kernel (53.7 when a thread walked over a row's keys).
 template <int D>
 __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float* Q, const float* K, const float* V, float* LSE,
-                                       size_t query0, int Sq, int Sk, int Sp, int H, int G, int causal, float scale)
+                                       size_t query0, int Sq, int Sk, int H, int G, int causal, float scale)
 {
     const int lane = threadIdx.x & 31;
     const int bh = static_cast<int>(query0 / Sq), i0 = static_cast<int>(query0 - static_cast<size_t>(bh) * Sq);
@@ -62,12 +58,12 @@ __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float*
     const float c2 = scale * kLog2e;
     for_flagged(flags, (static_cast<int>(threadIdx.x) >> 5) - 8, [&](uint32_t rows) {
         auto row = [&](int g) { return (rows >> (8 * g)) & 127u; };
-        auto end = [&](int g) { return causal ? (i0 + static_cast<int>(row(g))) % Sp + Sk - Sp + 1 : Sk; };
+        auto end = [&](int g) { return causal ? i0 + static_cast<int>(row(g)) + Sk - Sq + 1 : Sk; };
         RowGroup<D> q, o;
         q.load(Q + query0 * D, rows, lane);
         o.clear();
         float m = -INFINITY, l = 0.f;                      // the row's maximum, this lane's share of its sum
-        const int to = max(max(end(0), end(1)), max(end(2), end(3)));
+        const int to = end(3);                             // rows rise: the last one sees the most
         bool done = false;
         for (int j = 0; j < to && !done; j += 8) {
             const int n = min(8, to - j);
@@ -107,12 +103,11 @@ __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float*
     });
 }
 
-// Sp: rows of a head among the Sq of a packed one (Sq where heads are not packed).
-template <int D, bool SPLIT>
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
-                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int Sp, int BH, int H, int G, int n_qt, int Hg,
-                     int n_split, int causal, ScoreFactor c, float scale, unsigned* status)
+                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int BH, int H, int G, int n_qt, int Hg,
+                     int causal, ScoreFactor c, float scale, unsigned* status)
 {
     using C = Cfg<D>;
     constexpr int R = C::R;
@@ -121,32 +116,17 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Heaviest (last) query tiles first when causal.
     int tile, bh;
-    item_of_block(static_cast<int>(blockIdx.x) / (SPLIT ? n_split : 1), n_qt, BH, Hg, tile, bh);
-    const int part = SPLIT ? static_cast<int>(blockIdx.x) % n_split : 0;
+    item_of_block(static_cast<int>(blockIdx.x), n_qt, BH, Hg, tile, bh);
     const int qt = n_qt - 1 - tile;
     const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
-    const int off = Sk - Sp;                               // causal: key j visible to position i iff j <= i + off
-    const int i0 = qt * kBM, n_rows = min(kBM, Sq - i0);
-    int lo = i0 % Sp, hi = lo + n_rows - 1;                // positions of the tile's rows
-    if (hi >= Sp) { lo = 0; hi = Sp - 1; }                 // rows of two packed heads
-    // key blocks of this CTA (SPLIT: the last parts may be short, or empty)
-    const int n_all = causal ? (hi + off) / R + 1 : (Sk + R - 1) / R;
-    const int per = SPLIT ? (n_all + n_split - 1) / n_split : n_all, b0 = part * per;
-    const int n_kb = SPLIT ? max(0, min(per, n_all - b0)) : n_all;
-    // Own rows and the first streamed tile are asked for before the set-up.
-    const int t_own = tid - 256;
-    const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
-    const bool is_k = warp >= 4;                           // converter warps: K, or V
-    const float* const head = (is_k ? K : V) + static_cast<size_t>(bhk) * Sk * D;
-    Converter<D, R> cv;
-    OwnRows<D> qr;
-    if (warp >= 8) qr.load(Q + own_at, n_rows, t_own);
-    else if (warp != 0 && warp != 4) cv.start(is_k ? tid - 160 : tid - 32, head + static_cast<size_t>(b0) * R * D, Sk - b0 * R);
-
+    const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
+    const int i0 = qt * kBM;
+    const int i_last = min(i0 + kBM, Sq) - 1;
+    const int n_kb = causal ? (i_last + off) / R + 1 : (Sk + R - 1) / R;
     if (tid == 0) {
         mbar_init(bar(C::QFULL), 256);
         for (int w = 0; w < 2; ++w) {
@@ -160,64 +140,63 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     __syncwarp();
     if (warp == 0) tmem_alloc(tmem_slot, 512);
     if (tid == 32) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
-    if (SPLIT && tid >= 64 && tid < 72) sts32u(tmem_slot + 8 + 4 * (tid - 64), 0);        // flags of rows to do again
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
+    const uint32_t tmem = lds32u(tmem_slot);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
-        if constexpr (SPLIT) {                             // stays for its cluster
-            __syncwarp();
-            cluster_sync();
-            cluster_sync();
-        }
         return;
     }
 
     if (warp < 8) {
         reg_dealloc<56>();
         if (warp == 0) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- score products
-            const uint64_t dK = umma_smem_desc(base + C::OFF_K, 16, 1024);
-            if (leader) mbar_arrive(bar(C::SGO));                      // nothing to read yet in either score region
-            if (leader) mbar_arrive(bar(C::SGO + 1));
-            mbar_wait(bar(C::QFULL), 0, status);
+            if (lane == 0) {
+                // -------------------------------------------------------------- score products
+                const uint64_t dK = umma_smem_desc(base + C::OFF_K, 16, 1024);
+                mbar_arrive(bar(C::SGO));                      // nothing to read yet in either score region
+                mbar_arrive(bar(C::SGO + 1));
+                mbar_wait(bar(C::QFULL), 0, status);
 #pragma unroll 1
-            for (int n = 0; n < n_kb; ++n) {
-                const int w = n & 1;
-                mbar_wait(bar(C::SGO + w), (n >> 1) & 1, status);
-                tc_fence_after();
-                issue_scores<true, D, R, C::ST>(leader, tmem + C::TM_X + w * C::X, tmem + C::TM_Q,
-                                   dK + static_cast<uint64_t>((w * C::STAGE) >> 4));
-                umma_commit_warp(leader, bar(C::SDONE + w));
+                for (int n = 0; n < n_kb; ++n) {
+                    const int w = n & 1;
+                    mbar_wait(bar(C::SGO + w), (n >> 1) & 1, status);
+                    tc_fence_after();
+                    issue_scores<true, D, R, C::ST>(tmem + C::TM_X + w * C::X, tmem + C::TM_Q,
+                                       dK + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                    umma_commit(bar(C::SDONE + w));
+                }
             }
             __syncwarp();
         } else if (warp == 4) {
-            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
-            // -------------------------------------------------------------- P V products
-            const uint64_t mV = rows_desc<D, R>(base + C::OFF_V);
+            if (lane == 0) {
+                // -------------------------------------------------------------- P V products
+                const uint64_t mV = rows_desc<D, R>(base + C::OFF_V);
 #pragma unroll 1
-            for (int n = 0; n < n_kb; ++n) {
-                const int w = n & 1;
-                mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
-                tc_fence_after();
-                issue_rows<D, R, C::STO>(leader, tmem + C::TM_O, tmem + C::TM_X + w * C::X,
-                                 mV + static_cast<uint64_t>((w * C::STAGE) >> 4), row_steps<R>(Sk - (b0 + n) * R));
-                umma_commit_warp(leader, bar(C::PDONE + w));
-                umma_commit_warp(leader, bar(C::SGO + w));
+                for (int n = 0; n < n_kb; ++n) {
+                    const int w = n & 1;
+                    mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
+                    tc_fence_after();
+                    issue_rows<D, R, C::STO>(tmem + C::TM_O, tmem + C::TM_X + w * C::X,
+                                     mV + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                    umma_commit(bar(C::PDONE + w));
+                    umma_commit(bar(C::SGO + w));
+                }
             }
             __syncwarp();
         } else {
             // ------------------------------------------------------------------ K and V converters (one code)
+            const bool is_k = warp >= 4;
+            const float* head = (is_k ? K : V) + static_cast<size_t>(bhk) * Sk * D;
             const int full = is_k ? C::SGO : C::PGO, done = is_k ? C::SDONE : C::PDONE;
             const uint32_t stages = base + (is_k ? C::OFF_K : C::OFF_V);
-            cv.run(n_kb, 1.f, 0.f,
+            Converter<D, R> cv(is_k ? tid - 160 : tid - 32);
+            cv.run(n_kb,
                    [&](int i, int& rows) {
-                       rows = Sk - (b0 + i) * R;
-                       return head + static_cast<size_t>(b0 + i) * R * D;
+                       rows = Sk - i * R;
+                       return head + static_cast<size_t>(i) * R * D;
                    },
                    [&](int i) {
                        if (i >= 2) mbar_wait(bar(done + (i & 1)), ((i >> 1) & 1) ^ 1, status);
@@ -232,11 +211,14 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         const int r = tid & 127;                               // row within the tile = tensor-memory lane
         const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
         const uint32_t tX = tmem + lane_base + C::TM_X + w * C::X, tO = tmem + lane_base + C::TM_O;
-        const int i = (i0 + r) % Sp;                           // position
-        const bool row_ok = r < n_rows;
-        const int t = t_own;
+        const int i = i0 + r;
+        const bool row_ok = i < Sq;
+        const int t = tid - 256;
+        const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
         const uint32_t ex = base + C::OFF_EX;
         {
+            OwnRows<D> qr;
+            qr.load(Q + own_at, Sq - i0, t);
             qr.scale(c.hi, c.lo);
             qr.to_exchange(ex, t);
             named_bar_sync(1, 256);
@@ -252,12 +234,11 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
 #pragma unroll
         for (int d = 0; d < D; ++d) acc[d] = 0.f;
         const int vis = min(Sk, causal ? i + off + 1 : Sk);    // keys this row sees
-        const int all_see = min(Sk, causal ? lo + off + 1 : Sk);   // ... and every row of the tile
 
         for (int n = w; n < n_kb; n += 2) {
             const uint32_t ph = (n >> 1) & 1;
-            const int j0 = (b0 + n) * R, lim = vis - j0;   // first key; visible columns of this block
-            const bool masked = j0 + R > all_see;
+            const int lim = vis - n * R;                   // visible columns of this block
+            const bool masked = (causal && n * R + R - 1 > i0 + off) || n * R + R > Sk;
             mbar_wait(bar(C::SDONE + w), ph, status);
             tc_fence_after();
             // Blocks of 32 keep their scores in registers between the maximum and the exponentials; those of 64 are
@@ -337,124 +318,60 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         }
         named_bar_sync(1, 256);
         const uint32_t flags = tmem_slot + 8;
-        if constexpr (SPLIT) {
-            if (w == 0) {                                      // this part's sums, unnormalised
-                const float m1 = lds32f(stat), l1 = lds32f(stat + 4), mm = fmaxf(m, m1);
-                const float a0 = m == -INFINITY ? 0.f : ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+        bool redo = false;
+        if (w == 0) {
+            const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
+            const float mm = fmaxf(m, m1);
+            const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+            const float lt = fmaf(l, a0, l1 * a1);
+            const float inv = 1.0f / lt;
+            const float b0 = a0 * inv, b1 = a1 * inv;
+            // mm is a whole number: its share of the natural logarithm is formed with one rounding.  log2f, not the
+            // hardware approximation, whose error lies on one side (scores near 0: LSE off by -2.5 x 2^-24 on average and
+            // 3.9 rms over 200 keys; -0.3 and 2.9 with log2f; 3.3 rms in the FFMA kernel)
+            float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, log2f(lt) * kLn2));
+            float bad = 0.f;                                   // NaN once an output is not finite
 #pragma unroll
-                for (int d = 0; d < D; d += 4) {
-                    const float4 x = lds128(row + d * 4);
-                    sts128f(row + d * 4, fmaf(acc[d], a0, x.x * a1), fmaf(acc[d + 1], a0, x.y * a1), fmaf(acc[d + 2], a0, x.z * a1),
-                            fmaf(acc[d + 3], a0, x.w * a1));
-                }
-                sts32(stat, mm);
-                sts32(stat + 4, fmaf(l, a0, l1 * a1));
+            for (int d = 0; d < D; d += 4) {
+                float4 x = lds128(row + d * 4);
+                x = make_float4(fmaf(acc[d], b0, x.x * b1), fmaf(acc[d + 1], b0, x.y * b1), fmaf(acc[d + 2], b0, x.z * b1),
+                                fmaf(acc[d + 3], b0, x.w * b1));
+                sts128f(row + d * 4, x.x, x.y, x.z, x.w);
+                bad = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, bad))));
             }
-            const uint32_t stats = ex + 128 * OwnRows<D>::PITCH;
-            tc_fence_before();
-            __syncwarp();
-            cluster_sync();
-            // each CTA puts together a share of the tile's rows
-            const int share = (n_rows + n_split - 1) / n_split, first = part * share;
-            const size_t query0 = own_at / D;
-            combine_parts<D>(
-                ex, OwnRows<D>::PITCH, base, n_split, first, min(first + share, n_rows), t, 1,
-                [&](int rr, int k, float& mk, float& lk) {
-                    mk = lds_cluster_32(cluster_map(stats + rr * 8, k));
-                    lk = lds_cluster_32(cluster_map(stats + rr * 8 + 4, k));
-                },
-                [&](int rr, int c4, const float4& x, float mm, float lt) {
-                    const float inv = 1.0f / lt, lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, log2f(lt) * kLn2));
-                    const float4 y = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
-                    const float bad = fmaf(y.x, 0.f, fmaf(y.y, 0.f, fmaf(y.z, 0.f, y.w * 0.f)));
-                    if (bad != 0.f || !(fabsf(lse) < INFINITY)) or_shared(flags + 4 * (rr >> 5), 1u << (rr & 31));
-                    *reinterpret_cast<float4*>(O + (query0 + rr) * D + 4 * c4) = y;
-                    if (c4 == 0) LSE[query0 + rr] = lse;
-                });
-            __syncwarp();
-            cluster_sync();                                    // nobody leaves, or redoes rows, while its part is being read
-            if (any_flagged(flags)) {
-                redo_rows<D>(flags, ex, Q, K, V, LSE, query0, Sq, Sk, Sp, H, G, causal, scale);
-                named_bar_sync(1, 256);
-                for (int u = t; u < 128 * D / 4; u += 256) {
-                    const int rr = u / (D / 4), c4 = u % (D / 4);
-                    if (row_flagged(flags, rr))
-                        *reinterpret_cast<float4*>(O + (query0 + rr) * D + 4 * c4) = lds128(ex + rr * OwnRows<D>::PITCH + c4 * 16);
-                }
-            }
-        } else {
-            bool redo = false;
-            if (w == 0) {
-                const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
-                const float mm = fmaxf(m, m1);
-                const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
-                const float lt = fmaf(l, a0, l1 * a1);
-                const float inv = 1.0f / lt;
-                const float b0 = a0 * inv, b1 = a1 * inv;
-                // mm is a whole number: its share of the natural logarithm is formed with one rounding.  log2f, not the
-                // hardware approximation, whose error lies on one side (scores near 0: LSE off by -2.5 x 2^-24 on average and
-                // 3.9 rms over 200 keys; -0.3 and 2.9 with log2f; 3.3 rms in the FFMA kernel)
-                float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, log2f(lt) * kLn2));
-                float bad = 0.f;                                   // NaN once an output is not finite
-#pragma unroll
-                for (int d = 0; d < D; d += 4) {
-                    float4 x = lds128(row + d * 4);
-                    x = make_float4(fmaf(acc[d], b0, x.x * b1), fmaf(acc[d + 1], b0, x.y * b1), fmaf(acc[d + 2], b0, x.z * b1),
-                                    fmaf(acc[d + 3], b0, x.w * b1));
-                    sts128f(row + d * 4, x.x, x.y, x.z, x.w);
-                    bad = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, bad))));
-                }
-                redo = row_ok && (bad != 0.f || !(fabsf(lse) < INFINITY));
-                if (row_ok && !redo) LSE[static_cast<size_t>(bh) * Sq + i0 + r] = lse;
-            }
-            flag_rows(flags, warp - 8, redo);
-            named_bar_sync(1, 256);
-            if (any_flagged(flags)) {
-                redo_rows<D>(flags, ex, Q, K, V, LSE, own_at / D, Sq, Sk, Sp, H, G, causal, scale);
-                named_bar_sync(1, 256);
-            }
-            OwnRows<D>::store(O + own_at, Sq - i0, ex, t);
+            redo = row_ok && (bad != 0.f || !(fabsf(lse) < INFINITY));
+            if (row_ok && !redo) LSE[static_cast<size_t>(bh) * Sq + i] = lse;
         }
+        flag_rows(flags, warp - 8, redo);
+        named_bar_sync(1, 256);
+        if (any_flagged(flags)) {
+            redo_rows<D>(flags, ex, Q, K, V, LSE, own_at / D, Sq, Sk, H, G, causal, scale);
+            named_bar_sync(1, 256);
+        }
+        OwnRows<D>::store(O + own_at, Sq - i0, ex, t);
     }
 
     tc_fence_before();
-    if constexpr (SPLIT) {
-        if (warp < 8) {                                        // the softmax warps put the parts together
-            __syncwarp();
-            cluster_sync();
-            cluster_sync();
-        }
-    }
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// w: the problem with its heads packed; Sp: the rows of one head.
-template <int D, bool SPLIT>
-cudaError_t launch(const Problem& w, int Sp, int n_split, const float* q, const float* k, const float* v, float* o, float* lse,
+template <int D>
+cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse,
                    unsigned* status, cudaStream_t st)
 {
     using C = Cfg<D>;
-    auto kern = strict_tc_fwd_kernel<D, SPLIT>;
+    auto kern = strict_tc_fwd_kernel<D>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e == cudaSuccess && n_split > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_fwd attributes");
-    const int n_qt = (w.Sq + kBM - 1) / kBM;
-    const long long blocks = static_cast<long long>(n_qt) * w.BH() * n_split;
+    const int n_qt = (p.Sq + kBM - 1) / kBM;
+    const long long blocks = static_cast<long long>(n_qt) * p.BH();
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    e = launch_clusters(kern, static_cast<unsigned>(blocks), static_cast<unsigned>(n_split), kThreads, C::SMEM, st, q, k, v, o, lse, w.Sq,
-                        w.Sk, Sp, w.BH(), w.H, w.group(), n_qt, head_group(8.0 * w.Sk * D / w.group(), w.BH()), n_split, w.causal,
-                        score_factor(w.scale, D), w.scale, status);
-    return MGN_FAIL(e, "strict_tc_fwd launch");
-}
-template <int D>
-cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse, unsigned* status,
-                   cudaStream_t st)
-{
-    const Problem w = fwd_packed(p);
-    const int n_split = fwd_splits(static_cast<long long>((w.Sq + kBM - 1) / kBM) * w.BH(), p.Sk);
-    return n_split > 1 ? launch<D, true>(w, p.Sq, n_split, q, k, v, o, lse, status, st)
-                       : launch<D, false>(w, p.Sq, 1, q, k, v, o, lse, status, st);
+    kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(q, k, v, o, lse, p.Sq, p.Sk, p.BH(), p.H, p.group(),
+                                                                   n_qt, head_group(8.0 * p.Sk * D / p.group(), p.BH()), p.causal,
+                                                                   score_factor(p.scale, D), p.scale,
+                                                                   status);
+    return MGN_FAIL(cudaGetLastError(), "strict_tc_fwd launch");
 }
 
 }  // namespace
