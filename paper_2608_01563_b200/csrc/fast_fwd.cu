@@ -22,9 +22,15 @@
 // a limit (2^60; 2^15 with f16 probabilities), which is exact: any reference point works for a
 // softmax as long as nothing overflows.  The two threads of a row agree on that through a barrier
 // with an OR-reduction per block.
+//   Grouped heads: the query heads of a group are neighbours in memory and read the same keys, so where it saves tiles
+// (S_q not a multiple of 128) their rows are packed: one head of G S_q rows per key/value head, whose row x is position
+// x mod S_q.  One new token of 16 heads in groups of four is then four tiles, not sixteen.
+//   Few tiles over many keys (SPLIT): a tile's key blocks are dealt to a cluster of CTAs, which leave unnormalised O, row
+// sums and reference points in shared memory and put them together through distributed shared memory, in the order of
+// their ranks (see fwd_splits and parts.cuh).
 #include "kernels.h"
 #include "fast_items.cuh"
-#include "umma.cuh"
+#include "parts.cuh"
 
 namespace mgn {
 namespace {
@@ -34,6 +40,7 @@ constexpr int BM = 128;      // rows per query tile
 constexpr int BN = 128;      // keys per block
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+constexpr int kSplitWorth = 768;       // see fwd_splits
 // A thread's partial row sum (64 columns) above this limit moves the reference points.  Every p stays
 // below the limit and the sums of a row below 2^13 times it, so nothing overflows.  With f16
 // probabilities the limit is 2^15 (f16 ends at 65504).  With bf16 it is 2^60: bf16 and f32 share the
@@ -88,6 +95,8 @@ struct Cfg {
     static constexpr int OFF_BAR = OFF_MREF + 128 * 4;
     static constexpr int SMEM = OFF_BAR + 256 + 1024;
     static_assert(SMEM <= 232448, "shared memory budget");
+    static constexpr int PITCH = D * 4 + 16;                        // SPLIT: rows of a part's O
+    static_assert(128 * PITCH <= OFF_OST, "the parts of O lie over the dead tiles");
     static constexpr uint32_t TM_S = 0, TM_P = 256, TM_O = 384, TM_COLS = 512;
 };
 
@@ -108,6 +117,7 @@ enum { B_QFULL = 0, B_QEMPTY = 2, B_KEMPTY = 4, B_VEMPTY = 6, B_SFULL = 8, B_SGO
 // share the K, V of a few heads, which then stay in L2.  The launcher chooses (pick_schedule).
 struct Item {
     int bh, bhk, row0, nblk;
+    int blk0, lo;                              // GEN: first key block; lowest position of the tile's rows
 };
 // GEN = false is the square multi-head case (Sk == Sq, G == 1): offsets and the head mapping fold away.
 template <bool GEN>
@@ -127,20 +137,36 @@ __device__ __forceinline__ Item make_item(int it, const Dims& dm, int n_tiles, i
     w.bhk = GEN ? (w.bh / dm.H) * (dm.H / dm.G) + (w.bh % dm.H) / dm.G : w.bh;
     const int n_kb = (Sk + BN - 1) / BN;
     w.row0 = tile * BM;
-    w.nblk = causal ? min(n_kb, (min(w.row0 + BM, dm.Sq) - 1 + off) / BN + 1) : n_kb;
+    const int end = min(w.row0 + BM, dm.Sq);
+    int hi = end - 1;
+    w.lo = w.row0;
+    w.blk0 = 0;
+    if (GEN) {                                 // packed heads of Sp rows: a tile that holds rows of two sees all positions
+        w.lo = w.row0 % dm.Sp;
+        hi = w.lo + (end - w.row0) - 1;
+        if (hi >= dm.Sp) { w.lo = 0; hi = dm.Sp - 1; }
+    }
+    w.nblk = causal ? min(n_kb, (hi + off) / BN + 1) : n_kb;
     return w;
+}
+// Part `part` of n_split of an item's key blocks (the last parts may be short, or empty).
+__device__ __forceinline__ void take_part(Item& w, int part, int n_split) {
+    const int share = (w.nblk + n_split - 1) / n_split;
+    w.blk0 = part * share;
+    w.nblk = max(0, min(share, w.nblk - w.blk0));
 }
 
 // F16 = true is the forward of the accelerated policy (paper Section 4.2, table "Arithmetic
 // permissions"): operands are IEEE f16 copies of f32 tensors, P is packed as f16, and O leaves as f32
 // with plain stores (O32); otherwise operands and O are bf16 and O leaves through TMA (tmO).
-template <int D, bool GEN, bool F16>
+template <int D, bool GEN, bool F16, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                 float* __restrict__ LSE, float* __restrict__ O32, const Dims dm, int n_tiles, int causal, int order,
-                float c2, unsigned* status)
+                float c2, unsigned* status, int n_split, uint16_t* __restrict__ O16, int Dg)
 {
+    static_assert(!SPLIT || (GEN && !F16), "");
     using C = Cfg<D>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -150,12 +176,24 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     auto bar = [&](int i) { return bars + 8u * i; };
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
+    bool alive = true;                                     // false: an earlier wait on this device gave up
+    if constexpr (SPLIT) {                                 // the CTA stays for its cluster, and does nothing
+        if (tid == 0) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
+        __syncthreads();
+        alive = lds32u(tmem_slot + 4) == 0;
+    } else if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;
 
     const int n_items = n_tiles * dm.BH;
     const int Sq = dm.Sq, Sk = GEN ? dm.Sk : dm.Sq, coff = GEN ? dm.off : 0;
     const int G = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-    const int n_tiers = 2 * ((n_items + 2 * G - 1) / (2 * G));   // upper bound on items per CTA in either order
+    // upper bound on items per CTA in either order
+    const int n_tiers = SPLIT ? (alive ? 1 : 0) : 2 * ((n_items + 2 * G - 1) / (2 * G));
+    auto index_of = [&](int k) { return SPLIT ? cta / n_split : item_index(cta, k, G, n_items, order); };
+    auto item_of = [&](int it) {
+        Item w = make_item<GEN>(it, dm, n_tiles, causal, order);
+        if constexpr (SPLIT) take_part(w, cta % n_split, n_split);
+        return w;
+    };
 
     if (tid == 0) {
         for (int i = 0; i < B_COUNT; ++i) {
@@ -169,7 +207,7 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         fence_mbar_init();
     }
     __syncwarp();
-    if (warp == 0) tmem_alloc(tmem_slot, C::TM_COLS);
+    if (alive && warp == 0) tmem_alloc(tmem_slot, C::TM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -182,9 +220,9 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         {
             int g = 0;                                       // key blocks loaded so far (all items)
             for (int k = 0; k < n_tiers; ++k) {
-                const int it = item_index(cta, k, G, n_items, order);
+                const int it = index_of(k);
                 if (it < 0) break;
-                const Item w = make_item<GEN>(it, dm, n_tiles, causal, order);
+                const Item w = item_of(it);
                 const int qs = k & 1;
                 mbar_wait(bar(B_QEMPTY + qs), ((k >> 1) & 1) ^ 1, status);   // the last S product of item k - 2 is done
                 mbar_arrive_expect_tx(bar(B_QFULL + qs), C::TILE_BYTES);
@@ -198,7 +236,7 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     mbar_arrive_expect_tx(bar(B_SGO + st), C::TILE_BYTES);
 #pragma unroll
                     for (int ch = 0; ch < C::NCH; ++ch)
-                        tma_load_3d(sK + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmK, bar(B_SGO + st), ch * 64, n * BN, w.bhk);
+                        tma_load_3d(sK + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmK, bar(B_SGO + st), ch * 64, (w.blk0 + n) * BN, w.bhk);
                 }
             }
         }
@@ -209,16 +247,16 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         {
             int g = 0;
             for (int k = 0; k < n_tiers; ++k) {
-                const int it = item_index(cta, k, G, n_items, order);
+                const int it = index_of(k);
                 if (it < 0) break;
-                const Item w = make_item<GEN>(it, dm, n_tiles, causal, order);
+                const Item w = item_of(it);
                 for (int n = 0; n < w.nblk; ++n, ++g) {
                     const int st = g & 1;
                     mbar_wait(bar(B_VEMPTY + st), ((g >> 1) & 1) ^ 1, status);
                     mbar_arrive_expect_tx(bar(B_PVGO + st), C::TILE_BYTES);
 #pragma unroll
                     for (int ch = 0; ch < C::NCH; ++ch)
-                        tma_load_3d(sV + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmV, bar(B_PVGO + st), ch * 64, n * BN, w.bhk);
+                        tma_load_3d(sV + st * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmV, bar(B_PVGO + st), ch * 64, (w.blk0 + n) * BN, w.bhk);
                 }
             }
         }
@@ -240,9 +278,9 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 mbar_arrive(bar(B_SGO));         // blocks 0 and 1 have no product before them to wait for
                 mbar_arrive(bar(B_SGO + 1));
                 for (int k = 0; k < n_tiers; ++k) {
-                    const int it = item_index(cta, k, G, n_items, order);
+                    const int it = index_of(k);
                     if (it < 0) break;
-                    const int nblk = make_item<GEN>(it, dm, n_tiles, causal, order).nblk;
+                    const int nblk = item_of(it).nblk;
                     const int qs = k & 1;
                     const uint64_t qd = dQ0 + static_cast<uint64_t>((qs * C::TILE_BYTES) >> 4);
                     mbar_wait(bar(B_QFULL + qs), (k >> 1) & 1, status);
@@ -266,9 +304,9 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const uint64_t dV0 = umma_smem_desc(sV, C::CHUNK_BYTES, 1024);
                 const uint32_t tO = tmem + C::TM_O;
                 for (int k = 0; k < n_tiers; ++k) {
-                    const int it = item_index(cta, k, G, n_items, order);
+                    const int it = index_of(k);
                     if (it < 0) break;
-                    const int nblk = make_item<GEN>(it, dm, n_tiles, causal, order).nblk;
+                    const int nblk = item_of(it).nblk;
                     mbar_wait(bar(B_OEMPTY), (k & 1) ^ 1, status);   // the last item's O has been read out
                     for (int n = 0; n < nblk; ++n, ++g) {
                         const int b = g & 1;
@@ -299,11 +337,36 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const uint32_t xchg = base + C::OFF_XCHG, mref = base + C::OFF_MREF;
         const uint32_t ost = base + C::OFF_OST;
         for (int k = 0; k < n_tiers; ++k) {
-            const int it = item_index(cta, k, G, n_items, order);
+            const int it = index_of(k);
             if (it < 0) break;
-            const Item w = make_item<GEN>(it, dm, n_tiles, causal, order);
+            const Item w = item_of(it);
             const int i = w.row0 + r;
             mbar_wait(bar(B_STFULL), k & 1, status);
+            if constexpr (SPLIT) {
+                // this part's O, unnormalised, to the CTAs that own its rows
+                mbar_wait(bar(B_OFULL), 0, status);
+                tc_fence_after();
+                __syncwarp();
+                cluster_sync();
+                const int n_rows = min(BM, Sq - w.row0);
+                const RowShare rs(n_rows, n_split);
+                const uint32_t to = cluster_map(base + rs.slot(r, cta % n_split) * C::PITCH, min(rs.owner(r), n_split - 1));
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(tOr + 32 * c, v);
+                    tmem_ld_wait();
+                    if (r < n_rows && w.nblk > 0)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            sts_cluster_128(to + c * 128 + 16 * e, __uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]),
+                                            __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
+                }
+                tc_fence_before();
+                __syncwarp();
+                cluster_sync();
+                break;
+            }
             const float lt = lds32f(xchg + r * 4) + lds32f(xchg + (128 + r) * 4);
             const float mr = lds32f(mref + r * 4);
             mbar_arrive(bar(B_STEMPTY));                      // the softmax warps may use the exchange buffer again
@@ -359,7 +422,7 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 }
             }
         }
-        if (!F16 && r == 0) bulk_wait_group_read0();
+        if (!F16 && !SPLIT && r == 0) bulk_wait_group_read0();
     } else {
         // ------------------------------------------------------------------ softmax warps
         reg_alloc<176>();
@@ -385,10 +448,10 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         };
 
         for (int k = 0; k < n_tiers; ++k) {
-        const int it = item_index(cta, k, G, n_items, order);
+        const int it = index_of(k);
         if (it < 0) break;
-        const Item w = make_item<GEN>(it, dm, n_tiles, causal, order);
-        const int i = w.row0 + r;
+        const Item w = item_of(it);
+        const int i = GEN ? (w.row0 + r) % dm.Sp : w.row0 + r;      // position
         float m_ref = -INFINITY, l = 0.f;
         // the exchange buffer carried the row sums of the last item to the epilogue warps
         if (k > 0) mbar_wait(bar(B_STEMPTY), (k - 1) & 1, status);
@@ -400,8 +463,8 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             const uint32_t tP = tmem + lane_base + C::TM_P + b * 64 + 32 * h;    // ... and where their probabilities go
             mbar_wait(bar(B_SFULL + b), ph, status);
             tc_fence_after();
-            const int j0 = n * BN + 64 * h;
-            const bool masked = (causal && (j0 + 63 > w.row0 + coff)) || (j0 + 64 > Sk);
+            const int j0 = (w.blk0 + n) * BN + 64 * h;
+            const bool masked = (causal && (j0 + 63 > w.lo + coff)) || (j0 + 64 > Sk);
             const int jmax = min(Sk - 1, causal ? i + coff : Sk - 1) - j0;   // columns c <= jmax of this half are visible
 
             if (n == 0) {
@@ -432,6 +495,8 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 sts32(my_x, mine);
                 bar_or(false);
                 m_ref = fmaxf(mine, lds32f(peer_x)) + (F16 ? kMarginF16 : 0.f);      // finite: key 0 is visible to every row
+                // ... but not the first key of a part: a row that does not see it sees nothing of the part
+                if (SPLIT && m_ref == -INFINITY) m_ref = 0.f;
                 bar_or(false);                                // exchange buffer may be reused
             }
 
@@ -530,6 +595,41 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_arrive(bar(B_PVGO + b));
         }
 
+        if constexpr (SPLIT) {
+            // statistics to the owners of the rows (the epilogue warps send O), then the rows that this CTA owns
+            mbar_arrive(bar(B_STFULL));
+            tc_fence_before();
+            __syncwarp();
+            cluster_sync();
+            const int part = cta % n_split, n_rows = min(BM, Sq - w.row0);
+            const RowShare rs(n_rows, n_split);
+            if (r < n_rows) {
+                const uint32_t slot = rs.slot(r, part) * 4, owner = rs.owner(r);
+                sts_cluster_32(cluster_map(xchg + h * 512 + slot, owner), l);
+                if (h == 0) sts_cluster_32(cluster_map(base + C::OFF_MREF + slot, owner), m_ref);
+            }
+            __syncwarp();
+            cluster_sync();
+            const int first = part * rs.per;
+            const size_t at = static_cast<size_t>(w.bh) * Sq + w.row0 + first;
+            combine_parts<D>(
+                min(rs.per, n_rows - first), rs.per, n_split, tid - 128, 256,
+                [&](int slot, float& m, float& lk) {
+                    m = lds32f(base + C::OFF_MREF + slot * 4);
+                    lk = lds32f(xchg + slot * 4) + lds32f(xchg + 512 + slot * 4);
+                    if (lk == 0.f) m = -INFINITY;              // sees no key of this part
+                },
+                [&](int slot, int c) { return lds128(base + slot * C::PITCH + c * 16); },
+                [&](int row, int c, const float4& o, float m, float lk) {
+                    const float inv = 1.0f / lk;
+                    if (c == 0) LSE[at + row] = (m + log2f(lk)) * kLn2;
+                    if (4 * c < Dg)
+                        *reinterpret_cast<uint2*>(O16 + (at + row) * Dg + 4 * c) =
+                            make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+                });
+            break;
+        }
+
         // row sums (one per half) and reference points for the epilogue warps
         sts32(my_x, l);
         if (h == 0) sts32(base + C::OFF_MREF + r * 4, m_ref);
@@ -538,13 +638,20 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
 
     tc_fence_before();
+    if constexpr (SPLIT) {
+        if (warp < 4 || !alive) {                              // the two meetings of the cluster (see parts.cuh)
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
+    }
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, C::TM_COLS);
+    if (alive && warp == 0) tmem_dealloc(tmem, C::TM_COLS);
 }
 
-template <int D, bool GEN, bool F16>
+template <int D, bool GEN, bool F16, bool SPLIT = false>
 cudaError_t launch_gen(const Problem& p, const void* q, const void* k, const void* v, void* o, float* lse,
-                       unsigned* status, cudaStream_t st)
+                       unsigned* status, cudaStream_t st, int off, int Sp)
 {
     using C = Cfg<D>;
     CUtensorMap tq, tk, tv, to;
@@ -553,7 +660,7 @@ cudaError_t launch_gen(const Problem& p, const void* q, const void* k, const voi
     if (make_tmap_3d(&tv, v, 2, 1, p.BHkv(), p.Sk, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map v");
     // with f32 output the kernel stores O itself; the map then only has to be a valid one
     if (make_tmap_3d(&to, F16 ? q : o, 2, 1, p.BH(), p.Sq, p.D, 64, 128)) return MGN_FAIL(cudaErrorInvalidValue, "tensor map o");
-    auto kern = fast_fwd_kernel<D, GEN, F16>;
+    auto kern = fast_fwd_kernel<D, GEN, F16, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return MGN_FAIL(e, "cudaFuncSetAttribute");
     int dev = 0, sms = 0;
@@ -564,21 +671,35 @@ cudaError_t launch_gen(const Problem& p, const void* q, const void* k, const voi
     const long long items = static_cast<long long>(n_tiles) * p.BH();
     if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
     const long long blocks = items < sms ? items : sms;       // persistent: one CTA per SM
-    const Dims dm{p.Sq, p.Sk, p.BH(), p.H, p.group(), p.off()};
-    // streamed per block and shared between the query tiles of a head: K, V
-    const int order = pick_schedule(items, sms, static_cast<double>(p.BHkv()) * p.Sk * D * (2 + 2), dev);
-    kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(tq, tk, tv, to, lse, F16 ? static_cast<float*>(o) : nullptr, dm,
-                                                                   n_tiles, p.causal, order,
-                                                                   p.scale * kLog2e, status);
-    return MGN_FAIL(cudaGetLastError(), "forward launch");
+    const Dims dm{p.Sq, p.Sk, p.BH(), p.H, p.group(), off, Sp};
+    if constexpr (SPLIT) {
+        const int n_split = fwd_splits(items, p.Sk, kSplitWorth);
+        if (n_split > 8) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return MGN_FAIL(e, "cudaFuncSetAttribute");
+        }
+        e = launch_clusters(kern, static_cast<unsigned>(items) * n_split, static_cast<unsigned>(n_split), kThreads, C::SMEM, st, tq, tk, tv,
+                            to, lse, nullptr, dm, n_tiles, p.causal, 0, p.scale * kLog2e, status, n_split, static_cast<uint16_t*>(o), p.D);
+        return MGN_FAIL(e, "split forward launch");
+    } else {
+        // streamed per block and shared between the query tiles of a head: K, V
+        const int order = pick_schedule(items, sms, static_cast<double>(p.BHkv()) * p.Sk * D * (2 + 2), dev);
+        kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(tq, tk, tv, to, lse, F16 ? static_cast<float*>(o) : nullptr, dm,
+                                                                       n_tiles, p.causal, order, p.scale * kLog2e, status, 1, nullptr, p.D);
+        return MGN_FAIL(cudaGetLastError(), "forward launch");
+    }
 }
 
 template <int D>
 cudaError_t launch(const Problem& p, const void* q, const void* k, const void* v, void* o, float* lse,
                    unsigned* status, cudaStream_t st)
 {
-    return (p.Hkv != p.H || p.Sq != p.Sk) ? launch_gen<D, true, false>(p, q, k, v, o, lse, status, st)
-                                          : launch_gen<D, false, false>(p, q, k, v, o, lse, status, st);
+    // heads packed; the offset of the causal mask and the rows of a head stay those of the call
+    const Problem w = fwd_packed(p, 3, 4);
+    if (fwd_splits(static_cast<long long>((w.Sq + BM - 1) / BM) * w.BH(), p.Sk, kSplitWorth) > 1)
+        return launch_gen<D, true, false, true>(w, q, k, v, o, lse, status, st, p.off(), p.Sq);
+    return (p.Hkv != p.H || p.Sq != p.Sk) ? launch_gen<D, true, false>(w, q, k, v, o, lse, status, st, p.off(), p.Sq)
+                                          : launch_gen<D, false, false>(p, q, k, v, o, lse, status, st, 0, p.Sq);
 }
 
 // f32 -> IEEE f16, round to nearest even (HBM-bound, 8 elements per thread and step)
@@ -606,8 +727,8 @@ cudaError_t launch_fast_fwd_f16(const Problem& p, const void* q16, const void* k
                                 float* lse, unsigned* status, cudaStream_t st)
 {
     switch (p.D) {
-        case 64:  return launch_gen<64, true, true>(p, q16, k16, v16, o, lse, status, st);
-        case 128: return launch_gen<128, true, true>(p, q16, k16, v16, o, lse, status, st);
+        case 64:  return launch_gen<64, true, true>(p, q16, k16, v16, o, lse, status, st, p.off(), p.Sq);
+        case 128: return launch_gen<128, true, true>(p, q16, k16, v16, o, lse, status, st, p.off(), p.Sq);
         default:  return cudaErrorNotSupported;
     }
 }

@@ -7,6 +7,7 @@ namespace mgn {
 // key/value head h / G; causal: key j is visible to query i iff j <= i + off, off = Sk - Sq >= 0.
 struct Dims {
     int Sq, Sk, BH, H, G, off;
+    int Sp = 0;      // forward: rows of a head within the Sq rows of a packed one (Sq where heads are not packed)
 };
 
 // k-th item of CTA c out of G, -1 past the end (then also for every larger k).

@@ -41,6 +41,30 @@ inline double tiled_work(const Problem& p, int BM, int BN) {
     }
     return static_cast<double>(pairs) * BM * BN;
 }
+// The SM count is a constant: the library runs on one chip, and mgn_attn_strict_tiles has to answer without a device.
+constexpr int kSms = 148;
+
+// Forward over grouped heads: one head of group() * Sq rows per key/value head (see fast_fwd.cu), where that leaves at most
+// num/den of the 128-row tiles.  (A tile that holds rows of two heads sees the keys of both heads' last row.)
+inline Problem fwd_packed(Problem p, int num, int den) {
+    const int g = p.group();
+    const long long rows = static_cast<long long>(g) * p.Sq;
+    if (g > 1 && rows <= (1 << 24) && (rows + 127) / 128 * den <= static_cast<long long>(g) * ((p.Sq + 127) / 128) * num) {
+        p.H = p.Hkv;
+        p.Sq = static_cast<int>(rows);
+    }
+    return p;
+}
+// Forward: CTAs (a power of two, at most a cluster) that the keys of a 128-row query tile are dealt to, where the tiles leave
+// half of the SMs idle, at least 256 keys each.  `worth`: keys that a CTA has to be spared, or the parts cost more to put
+// together (4 us in fast mode) than they save: 8 heads of 1024 x 1024, D = 128, two parts 18.6 -> 22.5 us; one token of 16
+// heads in groups of four over 1024 keys, four parts 16.4 -> 14.3, over 16384 keys 117 -> 23 (strict 899 -> 79).
+inline int fwd_splits(long long tiles, int Sk, int worth) {
+    int n = 1;
+    while (n < 16 && tiles * n * 2 <= kSms && Sk / (2 * n) >= 256) n *= 2;
+    return Sk - Sk / n >= worth ? n : 1;
+}
+
 // Per-device set-up shared by every entry point: checks the architecture of the current device and
 // returns the device address of its status word.  Returns an mgn_status code.
 int device_status_word(unsigned** status);
@@ -60,6 +84,24 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned bl
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+// Launches `kern` in clusters of `cluster` CTAs (`grid` a multiple of it).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_clusters(void (*kern)(KArgs...), unsigned grid, unsigned cluster, unsigned block, size_t smem, cudaStream_t st,
+                                   Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
@@ -102,8 +144,6 @@ inline bool strict_on_tensor_cores(const Problem& p) {
 //   40-row query tiles (and 112-key tiles forward) by more than a seventh: 40 queries of 300 keys execute 40 x 336 and
 //   40 x 320 instead of 64 x 384 and 64 x 320.
 // - Otherwise 64 x 128 forward (64 x 64 at D = 128) and 64 x 64 backward (32 x 64).
-// The SM count is a constant: the library runs on one chip, and the query has to answer without a device.
-constexpr int kSms = 148;
 inline bool strict_few_tiles(long long tiles64) { return tiles64 <= kSms / 2; }
 inline bool prefer_alt_tiles(const Problem& p, int BM, int BN, int BM_alt, int BN_alt) {
     if (p.D != 64 || p.Sq > 512 || p.Sk > 512) return false;

@@ -18,6 +18,10 @@
 // product also tells the converters that its stage is free.  (One lane with a barrier per condition: 512
 // queries over 4096 keys, D = 128, 0.213 ms.)
 // Tensor memory: Q parts 3 D/2 columns, two score regions, one P V result.
+//   Grouped heads are packed where that saves tiles, and a tile's key blocks are dealt to a cluster of CTAs where few
+// tiles leave SMs idle (SPLIT), both as in fast_fwd.cu.  The CTAs of a cluster leave their unnormalised sums in their
+// exchange tiles; maxima are whole numbers, so the factors that put them together are exact.
+#include "parts.cuh"
 #include "strict_tc.cuh"
 
 namespace mgn {
@@ -50,7 +54,7 @@ struct Cfg {
 // against 0.18 for finite inputs and 0.86 of the FFMA kernel (53.7 when a thread walked over a row's keys).
 template <int D>
 __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float* Q, const float* K, const float* V, float* LSE,
-                                       size_t query0, int Sq, int Sk, int H, int G, int causal, float scale)
+                                       size_t query0, int Sq, int Sk, int Sp, int H, int G, int causal, float scale)
 {
     const int lane = threadIdx.x & 31;
     const int bh = static_cast<int>(query0 / Sq), i0 = static_cast<int>(query0 - static_cast<size_t>(bh) * Sq);
@@ -58,12 +62,12 @@ __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float*
     const float c2 = scale * kLog2e;
     for_flagged(flags, (static_cast<int>(threadIdx.x) >> 5) - 8, [&](uint32_t rows) {
         auto row = [&](int g) { return (rows >> (8 * g)) & 127u; };
-        auto end = [&](int g) { return causal ? i0 + static_cast<int>(row(g)) + Sk - Sq + 1 : Sk; };
+        auto end = [&](int g) { return causal ? (i0 + static_cast<int>(row(g))) % Sp + Sk - Sp + 1 : Sk; };
         RowGroup<D> q, o;
         q.load(Q + query0 * D, rows, lane);
         o.clear();
         float m = -INFINITY, l = 0.f;                      // the row's maximum, this lane's share of its sum
-        const int to = end(3);                             // rows rise: the last one sees the most
+        const int to = max(max(end(0), end(1)), max(end(2), end(3)));
         bool done = false;
         for (int j = 0; j < to && !done; j += 8) {
             const int n = min(8, to - j);
@@ -103,11 +107,12 @@ __device__ __noinline__ void redo_rows(uint32_t flags, uint32_t ex, const float*
     });
 }
 
-template <int D>
+// Sp: rows of a head among the Sq of a packed one (Sq where heads are not packed).
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V,
-                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int BH, int H, int G, int n_qt, int Hg,
-                     int causal, ScoreFactor c, float scale, unsigned* status)
+                     float* __restrict__ O, float* __restrict__ LSE, int Sq, int Sk, int Sp, int BH, int H, int G, int n_qt, int Hg,
+                     int n_split, int causal, ScoreFactor c, float scale, unsigned* status)
 {
     using C = Cfg<D>;
     constexpr int R = C::R;
@@ -120,13 +125,18 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
 
     // Heaviest (last) query tiles first when causal.
     int tile, bh;
-    item_of_block(static_cast<int>(blockIdx.x), n_qt, BH, Hg, tile, bh);
+    item_of_block(static_cast<int>(blockIdx.x) / (SPLIT ? n_split : 1), n_qt, BH, Hg, tile, bh);
+    const int part = SPLIT ? static_cast<int>(blockIdx.x) % n_split : 0;
     const int qt = n_qt - 1 - tile;
     const int bhk = (bh / H) * (H / G) + (bh % H) / G;     // key/value head of this query head
-    const int off = Sk - Sq;                               // causal: key j visible to query i iff j <= i + off
-    const int i0 = qt * kBM;
-    const int i_last = min(i0 + kBM, Sq) - 1;
-    const int n_kb = causal ? (i_last + off) / R + 1 : (Sk + R - 1) / R;
+    const int off = Sk - Sp;                               // causal: key j visible to position i iff j <= i + off
+    const int i0 = qt * kBM, n_rows = min(kBM, Sq - i0);
+    int lo = i0 % Sp, hi = lo + n_rows - 1;                // positions of the tile's rows
+    if (hi >= Sp) { lo = 0; hi = Sp - 1; }                 // rows of two packed heads
+    // key blocks of this CTA (SPLIT: the last parts may be short, or empty)
+    const int n_all = causal ? (hi + off) / R + 1 : (Sk + R - 1) / R;
+    const int per = SPLIT ? (n_all + n_split - 1) / n_split : n_all, b0 = part * per;
+    const int n_kb = SPLIT ? max(0, min(per, n_all - b0)) : n_all;
     if (tid == 0) {
         mbar_init(bar(C::QFULL), 256);
         for (int w = 0; w < 2; ++w) {
@@ -140,6 +150,7 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     __syncwarp();
     if (warp == 0) tmem_alloc(tmem_slot, 512);
     if (tid == 32) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
+    if (SPLIT && tid >= 64 && tid < 72) sts32u(tmem_slot + 8 + 4 * (tid - 64), 0);        // flags of rows to do again
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -147,6 +158,11 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
+        if constexpr (SPLIT) {                             // stays for its cluster
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
         return;
     }
 
@@ -195,8 +211,8 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
             Converter<D, R> cv(is_k ? tid - 160 : tid - 32);
             cv.run(n_kb,
                    [&](int i, int& rows) {
-                       rows = Sk - i * R;
-                       return head + static_cast<size_t>(i) * R * D;
+                       rows = Sk - (b0 + i) * R;
+                       return head + static_cast<size_t>(b0 + i) * R * D;
                    },
                    [&](int i) {
                        if (i >= 2) mbar_wait(bar(done + (i & 1)), ((i >> 1) & 1) ^ 1, status);
@@ -211,8 +227,8 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         const int r = tid & 127;                               // row within the tile = tensor-memory lane
         const uint32_t lane_base = static_cast<uint32_t>(r & ~31) << 16;
         const uint32_t tX = tmem + lane_base + C::TM_X + w * C::X, tO = tmem + lane_base + C::TM_O;
-        const int i = i0 + r;
-        const bool row_ok = i < Sq;
+        const int i = (i0 + r) % Sp;                           // position
+        const bool row_ok = r < n_rows;
         const int t = tid - 256;
         const size_t own_at = (static_cast<size_t>(bh) * Sq + i0) * D;
         const uint32_t ex = base + C::OFF_EX;
@@ -234,11 +250,12 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
 #pragma unroll
         for (int d = 0; d < D; ++d) acc[d] = 0.f;
         const int vis = min(Sk, causal ? i + off + 1 : Sk);    // keys this row sees
+        const int all_see = min(Sk, causal ? lo + off + 1 : Sk);   // ... and every row of the tile
 
         for (int n = w; n < n_kb; n += 2) {
             const uint32_t ph = (n >> 1) & 1;
-            const int lim = vis - n * R;                   // visible columns of this block
-            const bool masked = (causal && n * R + R - 1 > i0 + off) || n * R + R > Sk;
+            const int j0 = (b0 + n) * R, lim = vis - j0;   // first key; visible columns of this block
+            const bool masked = j0 + R > all_see;
             mbar_wait(bar(C::SDONE + w), ph, status);
             tc_fence_after();
             // Blocks of 32 keep their scores in registers between the maximum and the exponentials; those of 64 are
@@ -318,60 +335,138 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
         }
         named_bar_sync(1, 256);
         const uint32_t flags = tmem_slot + 8;
-        bool redo = false;
-        if (w == 0) {
-            const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
-            const float mm = fmaxf(m, m1);
-            const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
-            const float lt = fmaf(l, a0, l1 * a1);
-            const float inv = 1.0f / lt;
-            const float b0 = a0 * inv, b1 = a1 * inv;
-            // mm is a whole number: its share of the natural logarithm is formed with one rounding.  log2f, not the
-            // hardware approximation, whose error lies on one side (scores near 0: LSE off by -2.5 x 2^-24 on average and
-            // 3.9 rms over 200 keys; -0.3 and 2.9 with log2f; 3.3 rms in the FFMA kernel)
-            float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, log2f(lt) * kLn2));
-            float bad = 0.f;                                   // NaN once an output is not finite
+        if constexpr (SPLIT) {
+            // this part's sums, unnormalised, to the CTAs that own its rows; then the rows that this CTA owns
+            const RowShare rs(n_rows, n_split);
+            const int first = part * rs.per, owned = min(rs.per, n_rows - first);
+            float mm = 0.f, ll = 0.f;
+            if (w == 0) {
+                const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
+                mm = fmaxf(m, m1);
+                const float a0 = m == -INFINITY ? 0.f : ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+                ll = fmaf(l, a0, l1 * a1);
 #pragma unroll
-            for (int d = 0; d < D; d += 4) {
-                float4 x = lds128(row + d * 4);
-                x = make_float4(fmaf(acc[d], b0, x.x * b1), fmaf(acc[d + 1], b0, x.y * b1), fmaf(acc[d + 2], b0, x.z * b1),
-                                fmaf(acc[d + 3], b0, x.w * b1));
-                sts128f(row + d * 4, x.x, x.y, x.z, x.w);
-                bad = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, bad))));
+                for (int d = 0; d < D; d += 4) {
+                    const float4 x = lds128(row + d * 4);
+                    acc[d] = fmaf(acc[d], a0, x.x * a1);
+                    acc[d + 1] = fmaf(acc[d + 1], a0, x.y * a1);
+                    acc[d + 2] = fmaf(acc[d + 2], a0, x.z * a1);
+                    acc[d + 3] = fmaf(acc[d + 3], a0, x.w * a1);
+                }
             }
-            redo = row_ok && (bad != 0.f || !(fabsf(lse) < INFINITY));
-            if (row_ok && !redo) LSE[static_cast<size_t>(bh) * Sq + i] = lse;
-        }
-        flag_rows(flags, warp - 8, redo);
-        named_bar_sync(1, 256);
-        if (any_flagged(flags)) {
-            redo_rows<D>(flags, ex, Q, K, V, LSE, own_at / D, Sq, Sk, H, G, causal, scale);
+            tc_fence_before();
+            __syncwarp();
+            cluster_sync();
+            if (w == 0 && row_ok) {
+                const uint32_t slot = rs.slot(r, part), to = cluster_map(ex + slot * OwnRows<D>::PITCH, rs.owner(r)),
+                               to_stat = cluster_map(ex + 128 * OwnRows<D>::PITCH + slot * 8, rs.owner(r));
+#pragma unroll
+                for (int d = 0; d < D; d += 4) sts_cluster_128(to + d * 4, acc[d], acc[d + 1], acc[d + 2], acc[d + 3]);
+                sts_cluster_32(to_stat, mm);
+                sts_cluster_32(to_stat + 4, ll);
+            }
+            __syncwarp();
+            cluster_sync();
+            const size_t query0 = own_at / D;
+            combine_parts<D>(
+                owned, rs.per, n_split, t, 256,
+                [&](int slot, float& mk, float& lk) {
+                    mk = lds32f(ex + 128 * OwnRows<D>::PITCH + slot * 8);
+                    lk = lds32f(ex + 128 * OwnRows<D>::PITCH + slot * 8 + 4);
+                },
+                [&](int slot, int c4) { return lds128(ex + slot * OwnRows<D>::PITCH + c4 * 16); },
+                [&](int rr, int c4, const float4& x, float top, float lt) {
+                    const float inv = 1.0f / lt, lse = fmaf(top, kLn2, fmaf(top, kLn2Lo, log2f(lt) * kLn2));
+                    const float4 y = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
+                    const float bad = fmaf(y.x, 0.f, fmaf(y.y, 0.f, fmaf(y.z, 0.f, y.w * 0.f)));
+                    rr += first;
+                    if (bad != 0.f || !(fabsf(lse) < INFINITY)) or_shared(flags + 4 * (rr >> 5), 1u << (rr & 31));
+                    *reinterpret_cast<float4*>(O + (query0 + rr) * D + 4 * c4) = y;
+                    if (c4 == 0) LSE[query0 + rr] = lse;
+                });
             named_bar_sync(1, 256);
+            if (any_flagged(flags)) {
+                redo_rows<D>(flags, ex, Q, K, V, LSE, query0, Sq, Sk, Sp, H, G, causal, scale);
+                named_bar_sync(1, 256);
+                for (int u = t; u < 128 * D / 4; u += 256) {
+                    const int rr = u / (D / 4), c4 = u % (D / 4);
+                    if (row_flagged(flags, rr))
+                        *reinterpret_cast<float4*>(O + (query0 + rr) * D + 4 * c4) = lds128(ex + rr * OwnRows<D>::PITCH + c4 * 16);
+                }
+            }
+        } else {
+            bool redo = false;
+            if (w == 0) {
+                const float m1 = lds32f(stat), l1 = lds32f(stat + 4);
+                const float mm = fmaxf(m, m1);
+                const float a0 = ex2(m - mm), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+                const float lt = fmaf(l, a0, l1 * a1);
+                const float inv = 1.0f / lt;
+                const float b0 = a0 * inv, b1 = a1 * inv;
+                // mm is a whole number: its share of the natural logarithm is formed with one rounding.  log2f, not the
+                // hardware approximation, whose error lies on one side (scores near 0: LSE off by -2.5 x 2^-24 on average and
+                // 3.9 rms over 200 keys; -0.3 and 2.9 with log2f; 3.3 rms in the FFMA kernel)
+                float lse = fmaf(mm, kLn2, fmaf(mm, kLn2Lo, log2f(lt) * kLn2));
+                float bad = 0.f;                                   // NaN once an output is not finite
+#pragma unroll
+                for (int d = 0; d < D; d += 4) {
+                    float4 x = lds128(row + d * 4);
+                    x = make_float4(fmaf(acc[d], b0, x.x * b1), fmaf(acc[d + 1], b0, x.y * b1), fmaf(acc[d + 2], b0, x.z * b1),
+                                    fmaf(acc[d + 3], b0, x.w * b1));
+                    sts128f(row + d * 4, x.x, x.y, x.z, x.w);
+                    bad = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, bad))));
+                }
+                redo = row_ok && (bad != 0.f || !(fabsf(lse) < INFINITY));
+                if (row_ok && !redo) LSE[static_cast<size_t>(bh) * Sq + i0 + r] = lse;
+            }
+            flag_rows(flags, warp - 8, redo);
+            named_bar_sync(1, 256);
+            if (any_flagged(flags)) {
+                redo_rows<D>(flags, ex, Q, K, V, LSE, own_at / D, Sq, Sk, Sp, H, G, causal, scale);
+                named_bar_sync(1, 256);
+            }
+            OwnRows<D>::store(O + own_at, Sq - i0, ex, t);
         }
-        OwnRows<D>::store(O + own_at, Sq - i0, ex, t);
     }
 
     tc_fence_before();
+    if constexpr (SPLIT) {
+        if (warp < 8) {                                        // the two meetings of the cluster (see parts.cuh)
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
+    }
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int D>
-cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse,
+// w: the problem with its heads packed; Sp: the rows of one head.
+template <int D, bool SPLIT>
+cudaError_t launch(const Problem& w, int Sp, int n_split, const float* q, const float* k, const float* v, float* o, float* lse,
                    unsigned* status, cudaStream_t st)
 {
     using C = Cfg<D>;
-    auto kern = strict_tc_fwd_kernel<D>;
+    auto kern = strict_tc_fwd_kernel<D, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (e == cudaSuccess && n_split > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return MGN_FAIL(e, "strict_tc_fwd attributes");
-    const int n_qt = (p.Sq + kBM - 1) / kBM;
-    const long long blocks = static_cast<long long>(n_qt) * p.BH();
+    const int n_qt = (w.Sq + kBM - 1) / kBM;
+    const long long blocks = static_cast<long long>(n_qt) * w.BH() * n_split;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(q, k, v, o, lse, p.Sq, p.Sk, p.BH(), p.H, p.group(),
-                                                                   n_qt, head_group(8.0 * p.Sk * D / p.group(), p.BH()), p.causal,
-                                                                   score_factor(p.scale, D), p.scale,
-                                                                   status);
-    return MGN_FAIL(cudaGetLastError(), "strict_tc_fwd launch");
+    e = launch_clusters(kern, static_cast<unsigned>(blocks), static_cast<unsigned>(n_split), kThreads, C::SMEM, st, q, k, v, o, lse, w.Sq,
+                        w.Sk, Sp, w.BH(), w.H, w.group(), n_qt, head_group(8.0 * w.Sk * D / w.group(), w.BH()), n_split, w.causal,
+                        score_factor(w.scale, D), w.scale, status);
+    return MGN_FAIL(e, "strict_tc_fwd launch");
+}
+template <int D>
+cudaError_t launch(const Problem& p, const float* q, const float* k, const float* v, float* o, float* lse, unsigned* status,
+                   cudaStream_t st)
+{
+    const Problem w = fwd_packed(p, 19, 20);
+    const int n_split = fwd_splits(static_cast<long long>((w.Sq + kBM - 1) / kBM) * w.BH(), p.Sk, 256);
+    return n_split > 1 ? launch<D, true>(w, p.Sq, n_split, q, k, v, o, lse, status, st)
+                       : launch<D, false>(w, p.Sq, 1, q, k, v, o, lse, status, st);
 }
 
 }  // namespace

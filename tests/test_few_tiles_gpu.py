@@ -1,0 +1,64 @@
+"""Forward over few query tiles and many keys: the keys of a tile dealt to a cluster of CTAs, the rows of a group's heads
+packed into one tile (csrc/fast_fwd.cu, csrc/strict_tc_fwd.cu), against the f64 oracle in both modes."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_01563_b200 import binding as mgn
+
+import helpers as hp
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # B, H, Hkv, Sq, Sk, D, causal
+    (1, 16, 4, 1, 4096, 128, True),        # one new token: four packed tiles, sixteen parts
+    (1, 8, 2, 1, 1025, 64, True),          # parts of unequal length; the last key in a block of its own
+    (2, 8, 2, 50, 700, 128, True),         # tiles that hold the rows of three heads
+    (1, 6, 6, 130, 2100, 64, True),        # nothing to pack; two tiles a head, the second of two rows
+    (1, 4, 1, 300, 1111, 128, False),
+    (1, 2, 2, 1000, 1000, 64, True),       # square causal: the first tiles see no key of the later parts
+    (3, 32, 8, 33, 520, 32, True),         # head size 32 (the 64-wide build)
+]
+
+
+@pytest.mark.parametrize("mode,dtype", [(mgn.MODE_FAST_BF16, torch.bfloat16), (mgn.MODE_STRICT_F32, torch.float32)])
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", CASES)
+def test_matches_the_oracle(mode, dtype, B, H, Hkv, Sq, Sk, D, causal):
+    g = torch.Generator().manual_seed(Sq + Sk)
+    q = torch.randn(B, H, Sq, D, generator=g).to(dtype)
+    k, v = (torch.randn(B, Hkv, Sk, D, generator=g).to(dtype) for _ in range(2))
+    q[:, :, ::3] *= 6.0                                    # rows whose maxima differ between the parts
+    scale = 1.0 / math.sqrt(D)
+    got = hp.run_cuda_ext(q, k, v, torch.zeros_like(q), causal, scale, mode, run_bwd=False)
+    ref = hp.run_oracle_ext(q, k, v, torch.zeros_like(q), causal, scale)
+    if mode == mgn.MODE_STRICT_F32:
+        hp.check_strict(got, ref, names=("O", "LSE"), literal_max_abs=False)
+    else:
+        hp.check_fast(got, ref, names=("O",))
+    again = hp.run_cuda_ext(q, k, v, torch.zeros_like(q), causal, scale, mode, run_bwd=False)
+    for n in ("O", "LSE"):
+        assert np.array_equal(got[n], again[n]), f"{n} differs between runs"
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_strict_rows_that_are_not_finite_across_parts(D):
+    """An infinite value of one key: the rows that see it are infinite in that column alone, the others untouched."""
+    B, H, Hkv, Sq, Sk = 1, 8, 2, 40, 1024
+    g = torch.Generator().manual_seed(3)
+    q = torch.randn(B, H, Sq, D, generator=g)
+    k, v = (torch.randn(B, Hkv, Sk, D, generator=g) for _ in range(2))
+    v[0, 1, 1000, 5] = math.inf                            # seen by the queries from position 1000 - (Sk - Sq) on
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    o, lse = torch.empty_like(qd), torch.empty(B, H, Sq, device="cuda")
+    mgn.mgn_attn_fwd_ext(qd, kd, vd, o, lse, True, D ** -0.5, mgn.MODE_STRICT_F32)
+    mgn.mgn_attn_check()
+    inf = torch.zeros(B, H, Sq, D, dtype=torch.bool)
+    inf[0, 4:, 1000 - (Sk - Sq):, 5] = True
+    assert torch.equal(o.cpu() == math.inf, inf)
+    v[0, 1, 1000, 5] = 0.0
+    ref = hp.run_oracle_ext(q, k, v, torch.zeros_like(q), True, D ** -0.5)
+    got = np.where(inf.numpy(), ref["O"], o.cpu().double().numpy())
+    hp.check_strict({"O": got, "LSE": lse.cpu().double().numpy()}, ref, names=("O", "LSE"), literal_max_abs=False)
