@@ -18,6 +18,10 @@
 // operand); the column sets that come out are added in registers.  Stacked scores of 64 rows cost four
 // steps of 228 clocks together per 16 columns of D instead of six of 300.  f32 tensors are read with plain 16-byte
 // loads and split by converter warps.
+//   The warp that issues walks along in step and one elected lane issues: with a single lane in a branch of its own the
+// operands of every step went from that lane's registers to the uniform ones first, and a step took 80 to 110 clocks.
+// Forward and backward, in us: (8,12,1024,64) causal 484 -> 458, (32,12,197,64) 281 -> 259, (4,32,1024,128) causal
+// 1259 -> 1152.
 #pragma once
 #include "kernels.h"
 #include "umma.cuh"
@@ -333,19 +337,19 @@ template <int N> __device__ __forceinline__ void store_half_parts(uint32_t x, in
 // Sets of D[128 x R] = A B^T over D columns, at tensor-memory column d; B a split tile of R rows.  A in tensor
 // memory (part p at a + p * D / 2) or a split tile of 128 rows (a: its descriptor).  SCORE: see term().
 template <bool SCORE, int D, int R, int ST, typename A>
-__device__ __forceinline__ void issue_scores(uint32_t d, A a_at, uint64_t b_desc) {
+__device__ __forceinline__ void issue_scores(uint32_t leader, uint32_t d, A a_at, uint64_t b_desc) {
 #pragma unroll 1
     for (int t = 0; t < n_terms<SCORE, ST>(); ++t) {
         const Term m = term<SCORE, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, R, false, false) + (m.n - 1) * ((R >> 3) << 17);
-        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
+        const uint64_t b = desc_at(b_desc, m.b * part_bytes<R>());
         const uint32_t dt = d + m.set * R;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t bk = b + (((kk >> 2) * block_bytes<R>() + (kk & 3) * 32) >> 4);
+            const uint64_t bk = desc_at(b, (kk >> 2) * block_bytes<R>() + (kk & 3) * 32);
             const uint32_t add = (t > 0 || kk > 0) ? 1u : 0u;
-            if constexpr (sizeof(A) == 4) umma_ts(dt, a_at + m.a * (D / 2) + kk * 8, bk, idesc, add);
-            else umma_ss(dt, a_at + ((m.a * part_bytes<128>() + (kk >> 2) * block_bytes<128>() + (kk & 3) * 32) >> 4), bk, idesc, add);
+            if constexpr (sizeof(A) == 4) umma_ts_warp(leader, dt, a_at + m.a * (D / 2) + kk * 8, bk, idesc, add);
+            else umma_ss_warp(leader, dt, desc_at(a_at, m.a * part_bytes<128>() + (kk >> 2) * block_bytes<128>() + (kk & 3) * 32), bk, idesc, add);
         }
     }
 }
@@ -355,17 +359,17 @@ template <int D, int R> __device__ __forceinline__ uint64_t rows_desc(uint32_t t
     return umma_smem_desc(tile, D == 64 ? part_bytes<R>() : block_bytes<R>(), 1024);
 }
 template <int D, int R, int ST>
-__device__ __forceinline__ void issue_rows(uint32_t d, uint32_t x, uint64_t b_desc) {
+__device__ __forceinline__ void issue_rows(uint32_t leader, uint32_t d, uint32_t x, uint64_t b_desc) {
     static_assert(ST == 1 || D == 64, "");
 #pragma unroll 1
     for (int t = 0; t < n_terms<false, ST>(); ++t) {
         const Term m = term<false, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, D, false, true) + (m.n - 1) * ((D >> 3) << 17);
-        const uint64_t b = b_desc + ((m.b * part_bytes<R>()) >> 4);
+        const uint64_t b = desc_at(b_desc, m.b * part_bytes<R>());
         const uint32_t dt = d + m.set * D;
 #pragma unroll
         for (int kk = 0; kk < R / 16; ++kk)
-            umma_ts(dt, x + x_part_col<R>(m.a, kk), b + ((kk * 2048) >> 4), idesc, (t > 0 || kk > 0) ? 1u : 0u);
+            umma_ts_warp(leader, dt, x + x_part_col<R>(m.a, kk), desc_at(b, kk * 2048), idesc, (t > 0 || kk > 0) ? 1u : 0u);
     }
 }
 

@@ -190,7 +190,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     pdl_launch_dependents();                               // the dQ kernel may fill SMs as this one drains
 
     // First key blocks first: under a causal mask they see the most queries.
@@ -222,7 +222,7 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
@@ -232,50 +232,48 @@ strict_tc_dkv_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
         if (warp == 0) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- S^T and dP^T
-                const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024), dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
-                const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024);
-                [[maybe_unused]] const uint64_t dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
-                mbar_arrive(bar(C::S_GO));
-                mbar_arrive(bar(C::P_GO));
-                mbar_wait(bar(C::KV), 0, status);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- S^T and dP^T
+            const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024), dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
+            const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024);
+            [[maybe_unused]] const uint64_t dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
+            if (leader) mbar_arrive(bar(C::S_GO));
+            if (leader) mbar_arrive(bar(C::P_GO));
+            mbar_wait(bar(C::KV), 0, status);
 #pragma unroll 1
-                for (int n = 0; n < n_blk; ++n) {
-                    const int w = n & 1;
-                    const uint32_t ph = (n >> 1) & 1;
-                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                    mbar_wait(bar(C::S_GO + w), ph, status);
-                    tc_fence_after();
-                    issue_scores<true, D, R, C::ST>(tmem + C::TM_X, dKd, dQd + so);
-                    umma_commit(bar(C::S_DONE));
-                    mbar_wait(bar(C::P_GO + w), ph, status);
-                    tc_fence_after();
-                    if constexpr (C::V_TMEM) issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, tmem + C::TM_V, dOd + so);
-                    else issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, dVd, dOd + so);
-                    umma_commit(bar(C::P_DONE));
-                }
+            for (int n = 0; n < n_blk; ++n) {
+                const int w = n & 1;
+                const uint32_t ph = (n >> 1) & 1;
+                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                mbar_wait(bar(C::S_GO + w), ph, status);
+                tc_fence_after();
+                issue_scores<true, D, R, C::ST>(leader, tmem + C::TM_X, dKd, dQd + so);
+                umma_commit_warp(leader, bar(C::S_DONE));
+                mbar_wait(bar(C::P_GO + w), ph, status);
+                tc_fence_after();
+                if constexpr (C::V_TMEM) issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, tmem + C::TM_V, dOd + so);
+                else issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, dVd, dOd + so);
+                umma_commit_warp(leader, bar(C::P_DONE));
             }
             __syncwarp();
         } else if (warp == 1) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- dV and dK results
-                const uint64_t mQ = rows_desc<D, R>(base + C::OFF_Q), mO = rows_desc<D, R>(base + C::OFF_DO);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- dV and dK results
+            const uint64_t mQ = rows_desc<D, R>(base + C::OFF_Q), mO = rows_desc<D, R>(base + C::OFF_DO);
 #pragma unroll 1
-                for (int n = 0; n < n_blk; ++n) {
-                    const int w = n & 1;
-                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                    mbar_wait(bar(C::V_GO + w), (n >> 1) & 1, status);
-                    tc_fence_after();
-                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZV, tmem + C::TM_X, mO + so);
-                    umma_commit(bar(C::V_DONE));
-                    umma_commit(bar(C::S_GO + (w ^ 1)));
-                    mbar_wait(bar(C::K_GO), n & 1, status);
-                    tc_fence_after();
-                    issue_rows<D, R, C::STZ>(tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so);
-                    umma_commit(bar(C::K_DONE + w));       // both products of the block: its tiles are free too
-                    umma_commit(bar(C::P_GO + (w ^ 1)));
-                }
+            for (int n = 0; n < n_blk; ++n) {
+                const int w = n & 1;
+                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                mbar_wait(bar(C::V_GO + w), (n >> 1) & 1, status);
+                tc_fence_after();
+                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_ZV, tmem + C::TM_X, mO + so);
+                umma_commit_warp(leader, bar(C::V_DONE));
+                umma_commit_warp(leader, bar(C::S_GO + (w ^ 1)));
+                mbar_wait(bar(C::K_GO), n & 1, status);
+                tc_fence_after();
+                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_ZK, tmem + C::TM_Y, mQ + so);
+                umma_commit_warp(leader, bar(C::K_DONE + w));       // both products of the block: its tiles are free too
+                umma_commit_warp(leader, bar(C::P_GO + (w ^ 1)));
             }
             __syncwarp();
         } else {
@@ -523,7 +521,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
 
     // Heaviest (last) query tiles first when causal.
     const int item = static_cast<int>(blockIdx.x) / splits, part = static_cast<int>(blockIdx.x) % splits;
@@ -561,7 +559,7 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
@@ -572,46 +570,44 @@ strict_tc_dq_kernel(const float* __restrict__ Q, const float* __restrict__ K, co
     if (warp < 8) {
         reg_dealloc<kRegsIssue>();
         if (warp == 0) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- S and dP
-                const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024), dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
-                const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024);
-                [[maybe_unused]] const uint64_t dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
-                mbar_arrive(bar(C::S_GO));
-                mbar_arrive(bar(C::S_GO + 1));
-                mbar_wait(bar(C::QDO), 0, status);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- S and dP
+            const uint64_t dKd = umma_smem_desc(base + C::OFF_K, 16, 1024), dVd = umma_smem_desc(base + C::OFF_V, 16, 1024);
+            const uint64_t dQd = umma_smem_desc(base + C::OFF_Q, 16, 1024);
+            [[maybe_unused]] const uint64_t dOd = umma_smem_desc(base + C::OFF_DO, 16, 1024);
+            if (leader) mbar_arrive(bar(C::S_GO));
+            if (leader) mbar_arrive(bar(C::S_GO + 1));
+            mbar_wait(bar(C::QDO), 0, status);
 #pragma unroll 1
-                for (int n = 0; n < n_blk; ++n) {
-                    const int w = n & 1;
-                    const uint32_t ph = (n >> 1) & 1;
-                    const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
-                    const uint32_t x = tmem + C::TM_X + w * C::X;
-                    mbar_wait(bar(C::S_GO + w), ph, status);
-                    tc_fence_after();
-                    issue_scores<true, D, R, C::ST>(x, dQd, dKd + so);
-                    umma_commit(bar(C::S_DONE + w));
-                    mbar_wait(bar(C::P_GO + w), ph, status);
-                    tc_fence_after();
-                    if constexpr (C::DO_TMEM) issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, tmem + C::TM_DO, dVd + so);
-                    else issue_scores<false, D, R, C::ST>(tmem + C::TM_Y, dOd, dVd + so);
-                    umma_commit(bar(C::P_DONE));
-                }
+            for (int n = 0; n < n_blk; ++n) {
+                const int w = n & 1;
+                const uint32_t ph = (n >> 1) & 1;
+                const uint64_t so = static_cast<uint64_t>((w * C::STAGE) >> 4);
+                const uint32_t x = tmem + C::TM_X + w * C::X;
+                mbar_wait(bar(C::S_GO + w), ph, status);
+                tc_fence_after();
+                issue_scores<true, D, R, C::ST>(leader, x, dQd, dKd + so);
+                umma_commit_warp(leader, bar(C::S_DONE + w));
+                mbar_wait(bar(C::P_GO + w), ph, status);
+                tc_fence_after();
+                if constexpr (C::DO_TMEM) issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, tmem + C::TM_DO, dVd + so);
+                else issue_scores<false, D, R, C::ST>(leader, tmem + C::TM_Y, dOd, dVd + so);
+                umma_commit_warp(leader, bar(C::P_DONE));
             }
             __syncwarp();
         } else if (warp == 1) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- dQ results
-                const uint64_t mK = rows_desc<D, R>(base + C::OFF_K);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- dQ results
+            const uint64_t mK = rows_desc<D, R>(base + C::OFF_K);
 #pragma unroll 1
-                for (int n = 0; n < n_blk; ++n) {
-                    const int w = n & 1;
-                    mbar_wait(bar(C::Q_GO), n & 1, status);
-                    tc_fence_after();
-                    issue_rows<D, R, C::STZ>(tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
-                                        mK + static_cast<uint64_t>((w * C::STAGE) >> 4));
-                    umma_commit(bar(C::Z_DONE + w));       // S, dP (whose results it was formed from) and dQ: tiles free
-                    umma_commit(bar(C::S_GO + w));
-                }
+            for (int n = 0; n < n_blk; ++n) {
+                const int w = n & 1;
+                mbar_wait(bar(C::Q_GO), n & 1, status);
+                tc_fence_after();
+                issue_rows<D, R, C::STZ>(leader, tmem + C::TM_Z, tmem + C::TM_X + w * C::X,
+                                    mK + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                umma_commit_warp(leader, bar(C::Z_DONE + w));       // S, dP (whose results it was formed from) and dQ: tiles free
+                umma_commit_warp(leader, bar(C::S_GO + w));
             }
             __syncwarp();
         } else {

@@ -121,7 +121,7 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     const uint32_t base = smem_u32(smem);
     const uint32_t bars = base + C::OFF_BAR, tmem_slot = bars + C::COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
 
     // Heaviest (last) query tiles first when causal.
     int tile, bh;
@@ -154,7 +154,7 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
     if (lds32u(tmem_slot + 4) != 0) {                      // an earlier wait on this device gave up
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, 512);
@@ -169,37 +169,35 @@ strict_tc_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ K, c
     if (warp < 8) {
         reg_dealloc<56>();
         if (warp == 0) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- score products
-                const uint64_t dK = umma_smem_desc(base + C::OFF_K, 16, 1024);
-                mbar_arrive(bar(C::SGO));                      // nothing to read yet in either score region
-                mbar_arrive(bar(C::SGO + 1));
-                mbar_wait(bar(C::QFULL), 0, status);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- score products
+            const uint64_t dK = umma_smem_desc(base + C::OFF_K, 16, 1024);
+            if (leader) mbar_arrive(bar(C::SGO));                      // nothing to read yet in either score region
+            if (leader) mbar_arrive(bar(C::SGO + 1));
+            mbar_wait(bar(C::QFULL), 0, status);
 #pragma unroll 1
-                for (int n = 0; n < n_kb; ++n) {
-                    const int w = n & 1;
-                    mbar_wait(bar(C::SGO + w), (n >> 1) & 1, status);
-                    tc_fence_after();
-                    issue_scores<true, D, R, C::ST>(tmem + C::TM_X + w * C::X, tmem + C::TM_Q,
-                                       dK + static_cast<uint64_t>((w * C::STAGE) >> 4));
-                    umma_commit(bar(C::SDONE + w));
-                }
+            for (int n = 0; n < n_kb; ++n) {
+                const int w = n & 1;
+                mbar_wait(bar(C::SGO + w), (n >> 1) & 1, status);
+                tc_fence_after();
+                issue_scores<true, D, R, C::ST>(leader, tmem + C::TM_X + w * C::X, tmem + C::TM_Q,
+                                   dK + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                umma_commit_warp(leader, bar(C::SDONE + w));
             }
             __syncwarp();
         } else if (warp == 4) {
-            if (lane == 0) {
-                // -------------------------------------------------------------- P V products
-                const uint64_t mV = rows_desc<D, R>(base + C::OFF_V);
+            const uint32_t leader = elect_one();       // the whole warp walks along, one lane issues
+            // -------------------------------------------------------------- P V products
+            const uint64_t mV = rows_desc<D, R>(base + C::OFF_V);
 #pragma unroll 1
-                for (int n = 0; n < n_kb; ++n) {
-                    const int w = n & 1;
-                    mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
-                    tc_fence_after();
-                    issue_rows<D, R, C::STO>(tmem + C::TM_O, tmem + C::TM_X + w * C::X,
-                                     mV + static_cast<uint64_t>((w * C::STAGE) >> 4));
-                    umma_commit(bar(C::PDONE + w));
-                    umma_commit(bar(C::SGO + w));
-                }
+            for (int n = 0; n < n_kb; ++n) {
+                const int w = n & 1;
+                mbar_wait(bar(C::PGO + w), (n >> 1) & 1, status);
+                tc_fence_after();
+                issue_rows<D, R, C::STO>(leader, tmem + C::TM_O, tmem + C::TM_X + w * C::X,
+                                 mV + static_cast<uint64_t>((w * C::STAGE) >> 4));
+                umma_commit_warp(leader, bar(C::PDONE + w));
+                umma_commit_warp(leader, bar(C::SGO + w));
             }
             __syncwarp();
         } else {

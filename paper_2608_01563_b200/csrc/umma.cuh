@@ -59,6 +59,30 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// The same issued by a whole warp in step, of which the lane with `leader` set issues: operands that are computed by
+// uniform code need not be moved out of one lane's registers first, and an issuing lane has few instructions to spare (see
+// strict_tc.cuh).
+__device__ __forceinline__ void umma_ss_warp(uint32_t leader, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred P, L;\n\tsetp.ne.b32 P, %4, 0;\n\tsetp.ne.b32 L, %5, 0;\n\t"
+        "@L tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, P;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
+}
+__device__ __forceinline__ void umma_ts_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred P, L;\n\tsetp.ne.b32 P, %4, 0;\n\tsetp.ne.b32 L, %5, 0;\n\t"
+        "@L tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, P;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
+}
+__device__ __forceinline__ void umma_commit_warp(uint32_t leader, uint32_t bar) {
+    asm volatile("{\n\t.reg .pred L;\n\tsetp.ne.b32 L, %1, 0;\n\t"
+                 "@L tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader) : "memory");
+}
+// Descriptor of a tile `bytes` further on (the address field cannot carry out of its 14 bits within shared memory).
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) {
+    return (desc & 0xffffffff00000000ull) | (static_cast<uint32_t>(desc) + (bytes >> 4));
+}
+
 // ---- tensor memory --------------------------------------------------------------------------------
 // Address = (lane << 16) | column.  A warp may touch lanes [32*(warp%4), 32*(warp%4)+32).
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_slot, uint32_t ncols) {   // whole warp
