@@ -56,13 +56,17 @@ inline Problem fwd_packed(Problem p, int num, int den) {
     return p;
 }
 // Forward: CTAs (a power of two, at most a cluster) that the keys of a 128-row query tile are dealt to, where the tiles leave
-// half of the SMs idle, at least 256 keys each.  `worth`: keys that a CTA has to be spared, or the parts cost more to put
-// together (4 us in fast mode) than they save: 8 heads of 1024 x 1024, D = 128, two parts 18.6 -> 22.5 us; one token of 16
-// heads in groups of four over 1024 keys, four parts 16.4 -> 14.3, over 16384 keys 117 -> 23 (strict 899 -> 79).
+// half of the SMs idle, at least 256 keys each.
+// - Clusters of 8 and 16 find room on 64 SMs at a time, not more: 16 tiles over 8192 keys, D = 128, in 4 / 8 parts 29.7 /
+//   37.0 us (strict 142 / 146), 8 tiles over 4096 keys in 8 / 16 parts 18.3 / 28.7 (47 / 55), 4 tiles over 16384 keys in 8 / 16
+//   parts 26.8 / 22.7 (137 / 80); 32 tiles over 3000 keys, D = 64, in 1 / 2 / 4 parts 30.8 / 24.6 / 20.6.
+// - `worth`: keys that a CTA has to be spared (two parts: 256 more), or the parts cost more to put together (4 us in fast
+//   mode) than they save: 8 heads of 1024 x 1024, D = 128, two parts 18.6 -> 22.5 us, 56 tiles over 2000 keys 25.6 -> 26.6;
+//   one token of 16 heads in groups of four over 1024 keys, four parts 16.4 -> 14.3.
 inline int fwd_splits(long long tiles, int Sk, int worth) {
     int n = 1;
-    while (n < 16 && tiles * n * 2 <= kSms && Sk / (2 * n) >= 256) n *= 2;
-    return Sk - Sk / n >= worth ? n : 1;
+    while (n < 16 && tiles * n * 2 <= (n < 4 ? kSms : 64) && Sk / (2 * n) >= 256) n *= 2;
+    return Sk - Sk / n >= worth + (n == 2 ? 256 : 0) ? n : 1;
 }
 
 // Per-device set-up shared by every entry point: checks the architecture of the current device and
