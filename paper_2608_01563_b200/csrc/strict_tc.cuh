@@ -334,11 +334,14 @@ template <int N> __device__ __forceinline__ void store_half_parts(uint32_t x, in
     }
 }
 
+// Unrolled over terms and steps: with uniform operands they are constants and a step is few instructions (forward and
+// backward, terms rolled / unrolled: (8,12,1024,64) causal 449 / 444 us, (32,12,197,64) 258 / 254, (4,32,1024,128) causal
+// 1134 / 1125).
 // Sets of D[128 x R] = A B^T over D columns, at tensor-memory column d; B a split tile of R rows.  A in tensor
 // memory (part p at a + p * D / 2) or a split tile of 128 rows (a: its descriptor).  SCORE: see term().
 template <bool SCORE, int D, int R, int ST, typename A>
 __device__ __forceinline__ void issue_scores(uint32_t leader, uint32_t d, A a_at, uint64_t b_desc) {
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < n_terms<SCORE, ST>(); ++t) {
         const Term m = term<SCORE, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, R, false, false) + (m.n - 1) * ((R >> 3) << 17);
@@ -361,7 +364,7 @@ template <int D, int R> __device__ __forceinline__ uint64_t rows_desc(uint32_t t
 template <int D, int R, int ST>
 __device__ __forceinline__ void issue_rows(uint32_t leader, uint32_t d, uint32_t x, uint64_t b_desc) {
     static_assert(ST == 1 || D == 64, "");
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < n_terms<false, ST>(); ++t) {
         const Term m = term<false, ST>(t);
         const uint32_t idesc = umma_idesc_bf16(128, D, false, true) + (m.n - 1) * ((D >> 3) << 17);
