@@ -1,0 +1,398 @@
+// Fast-mode attention backward for one block of keys (S_k <= 128): the latency path.
+//
+// The paper's own cross-attention shapes (50 action tokens over 16 context tokens, 77-token text; Section 4.1,
+// workload table) have a single key block, where the persistent kernel of fast_bwd.cu is one dependent chain per
+// item and SM, behind a preprocess launch.  Here a small CTA (two per SM at D = 64) owns 128-row query tiles of one
+// key/value head, scores are NOT transposed (lanes = queries, columns = the keys that exist, rounded up to 16), and one
+// kernel is the whole backward:
+//     delta = rowsum(dO o O)  (or given)
+//     S = Q K^T, dP = dO V^T            -> P = exp2(S c - LSE), dS = P (dP - delta), bf16, rows of shared memory
+//     dV += P^T dO, dK += dS^T Q        (P, dS as MN-major operands)       dQ = dS K   (the same dS, K-major)
+// dQ of a tile is complete and leaves through the dO tile and a TMA store.  dK and dV gather in tensor memory over the
+// tiles of a CTA; the tiles of a head may be dealt to a cluster of up to eight CTAs, which add their parts up through
+// distributed shared memory in the order of their ranks: no atomics, bit-identical from run to run.
+//   warp 0, one lane   TMA loads and all tensor-core issue
+//   warps 1-8          element-wise work, two threads per query row: 16-key pieces in turn
+// Tensor memory: S [0,128), at D = 128 dP [128,256), dV, dK behind.  At D = 64 (256 columns, two CTAs per SM) dP has
+// columns of its own only where at most 64 keys leave them; else it takes S's, once S has been read.  dQ takes S's.
+// Bound by the chain of a tile: load, two products, exponentials, product, product, store; two CTAs per SM overlap it.
+#include <cuda_bf16.h>
+
+#include "fast_items.cuh"
+#include "kernels.h"
+#include "umma.cuh"
+
+namespace mgn {
+namespace {
+
+constexpr int kThreads = 288, BM = 128, kCompute = 256;
+constexpr float kLog2e = 1.4426950408889634f;
+
+// KC: 64-key chunks of a tile (1: at most 64 keys).
+template <int D, int KC>
+struct Cfg {
+    static constexpr int NCH = D / 64;
+    static constexpr int P_CHUNK = BM * 128, P_BYTES = KC * P_CHUNK;             // P, dS: 128 rows, chunks of 64 keys
+    static constexpr bool SHARED_P = D == 64 && KC == 2;                         // dS takes P's place (for two CTAs per SM)
+    static constexpr int Q_CHUNK = BM * 128, Q_BYTES = NCH * Q_CHUNK;            // Q, dO
+    static constexpr int K_CHUNK = KC * 64 * 128, K_BYTES = NCH * K_CHUNK;       // K, V
+    // P and dS first: with one chunk the products' A operand still spans two, the second one lying in what follows
+    // (its rows of dV, dK are those of keys that do not exist)
+    static constexpr int OFF_P = 0, OFF_DS = SHARED_P ? 0 : P_BYTES, OFF_Q = OFF_DS + P_BYTES, OFF_DO = OFF_Q + Q_BYTES,
+                         OFF_K = OFF_DO + Q_BYTES, OFF_V = OFF_K + K_BYTES, OFF_DELTA = OFF_V + K_BYTES,
+                         OFF_BAR = OFF_DELTA + 2 * BM * 4;                       // delta: a share of each thread of a row
+    static constexpr int PAYLOAD = OFF_BAR + 96, SMEM = PAYLOAD + 1024;
+    static constexpr int PITCH = D * 4 + 16;                                     // rows of the f32 parts of dK, dV
+    static_assert(2 * 64 * KC * PITCH <= OFF_DELTA, "the parts lie over the dead tiles");
+    static constexpr bool DP_APART = D == 128 || KC == 1;
+    static constexpr uint32_t TM_S = 0, TM_DP = D == 128 ? 128 : KC == 1 ? 64 : 0, TM_DV = D == 128 ? 256 : 128,
+                              TM_DK = TM_DV + D, TM_COLS = D == 128 ? 512 : 256;
+    static constexpr int CTAS = D == 64 ? 2 : 1;
+};
+enum { B_KV = 0, B_QO = 1, B_S = 2, B_DP = 3, B_P = 4, B_DV = 5, B_DS = 6, B_DQ = 7, B_R = 8, B_DQR = 9, B_COUNT = 10 };
+
+template <int D, int KC>
+__global__ void __launch_bounds__(kThreads, Cfg<D, KC>::CTAS)
+fast_bwd_small_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
+                      const __grid_constant__ CUtensorMap tmdQ, const __nv_bfloat16* __restrict__ O,
+                      const float* __restrict__ LSE, const float* __restrict__ DELTA, __nv_bfloat16* __restrict__ dK,
+                      __nv_bfloat16* __restrict__ dV, const Dims dm, int n_share, int causal, float scale, int Dg,
+                      unsigned* status)
+{
+    using C = Cfg<D, KC>;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;       // the same offset in every CTA of a cluster
+    const uint32_t sP = base + C::OFF_P, sDS = base + C::OFF_DS, sQ = base + C::OFF_Q, sdO = base + C::OFF_DO,
+                   sK = base + C::OFF_K, sV = base + C::OFF_V, bars = base + C::OFF_BAR, tmem_slot = bars + B_COUNT * 8;
+    auto bar = [&](int i) { return bars + 8u * i; };
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    // Share `share` of n_share of the query tiles of key/value head bhk: tiles share, share + n_share, ... of
+    // (query head of the group, 128 rows).
+    const int Sq = dm.Sq, Sk = dm.Sk, n_qt = (Sq + BM - 1) / BM, n_tiles = n_qt * dm.G;
+    const int bhk = static_cast<int>(blockIdx.x) / n_share, share = static_cast<int>(blockIdx.x) % n_share;
+    const int Hkv = dm.H / dm.G, bh0 = (bhk / Hkv) * dm.H + (bhk % Hkv) * dm.G;
+    const int n_own = (n_tiles - share + n_share - 1) / n_share;       // >= 1: n_share <= n_tiles
+    auto tile_at = [&](int t, int& bh, int& i0) {
+        const int x = share + t * n_share;
+        bh = bh0 + x / n_qt;
+        i0 = (x % n_qt) * BM;
+    };
+    // An earlier wait on this device gave up: nothing is computed or stored, but the CTA stays for its cluster.
+    if (tid == 0) {
+        sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
+        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), (i == B_P || i == B_DS || i == B_DQR) ? 8 : 1);   // one arrival per warp
+        fence_mbar_init();
+    }
+    __syncthreads();
+    const bool alive = lds32u(tmem_slot + 4) == 0;
+    uint32_t tmem = 0;
+    if (alive) {
+        if (warp == 0) tmem_alloc(tmem_slot, C::TM_COLS);
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        tmem = lds32u(tmem_slot);
+    }
+    const int ksteps = (Sk + 15) >> 4;                                 // 16-key steps that hold keys
+
+    if (alive && warp == 0) {
+        if (lane == 0) {
+            // ---------------------------------------------------------------- loads and tensor-core issue
+            const uint32_t idesc_s = umma_idesc_bf16(BM, 16 * ksteps, false, false);
+            constexpr uint32_t idesc_kv = umma_idesc_bf16(128, D, true, true), idesc_q = umma_idesc_bf16(BM, D, false, true);
+            const uint64_t kQ = umma_smem_desc(sQ, 16, 1024), kO = umma_smem_desc(sdO, 16, 1024), kK = umma_smem_desc(sK, 16, 1024),
+                           kV = umma_smem_desc(sV, 16, 1024), kDS = umma_smem_desc(sDS, 16, 1024);
+            const uint64_t mP = umma_smem_desc(sP, C::P_CHUNK, 1024), mDS = umma_smem_desc(sDS, C::P_CHUNK, 1024),
+                           mQ = umma_smem_desc(sQ, C::Q_CHUNK, 1024), mO = umma_smem_desc(sdO, C::Q_CHUNK, 1024),
+                           mK = umma_smem_desc(sK, C::K_CHUNK, 1024);
+            auto at = [](uint64_t desc, int bytes) { return desc + static_cast<uint64_t>(bytes >> 4); };
+            auto load_tile = [&](int t) {
+                int bh, i0;
+                tile_at(t, bh, i0);
+                mbar_arrive_expect_tx(bar(B_QO), 2 * C::Q_BYTES);
+#pragma unroll
+                for (int ch = 0; ch < C::NCH; ++ch) {
+                    tma_load_3d(sQ + ch * C::Q_CHUNK, &tmQ, bar(B_QO), ch * 64, i0, bh);
+                    tma_load_3d(sdO + ch * C::Q_CHUNK, &tmdO, bar(B_QO), ch * 64, i0, bh);
+                }
+            };
+            mbar_arrive_expect_tx(bar(B_KV), 2 * C::K_BYTES);
+#pragma unroll
+            for (int ch = 0; ch < C::NCH; ++ch) {
+                tma_load_3d(sK + ch * C::K_CHUNK, &tmK, bar(B_KV), ch * 64, 0, bhk);
+                tma_load_3d(sV + ch * C::K_CHUNK, &tmV, bar(B_KV), ch * 64, 0, bhk);
+            }
+            load_tile(0);
+            mbar_wait(bar(B_KV), 0, status);
+            auto issue_dp = [&]() {
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk)
+                    umma_ss(tmem + C::TM_DP, at(kO, (kk >> 2) * C::Q_CHUNK + (kk & 3) * 32), at(kV, (kk >> 2) * C::K_CHUNK + (kk & 3) * 32),
+                            idesc_s, kk > 0);
+                umma_commit(bar(B_DP));
+            };
+            for (int t = 0; t < n_own; ++t) {
+                const uint32_t ph = t & 1;
+                int bh, i0;
+                tile_at(t, bh, i0);
+                const int qsteps = (min(Sq - i0, BM) + 15) >> 4;       // 16-query steps that hold queries
+                mbar_wait(bar(B_QO), ph, status);
+                tc_fence_after();
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk)
+                    umma_ss(tmem + C::TM_S, at(kQ, (kk >> 2) * C::Q_CHUNK + (kk & 3) * 32), at(kK, (kk >> 2) * C::K_CHUNK + (kk & 3) * 32),
+                            idesc_s, kk > 0);
+                umma_commit(bar(B_S));
+                if (C::DP_APART) issue_dp();
+                mbar_wait(bar(B_P), ph, status);
+                tc_fence_after();
+                if (!C::DP_APART) issue_dp();
+                for (int kk = 0; kk < qsteps; ++kk)
+                    umma_ss(tmem + C::TM_DV, at(mP, kk * 2048), at(mO, kk * 2048), idesc_kv, (t > 0 || kk > 0) ? 1u : 0u);
+                if (C::SHARED_P) umma_commit(bar(B_DV));
+                mbar_wait(bar(B_DS), ph, status);
+                tc_fence_after();
+                for (int kk = 0; kk < ksteps; ++kk)
+                    umma_ss(tmem + C::TM_S, at(kDS, (kk >> 2) * C::P_CHUNK + (kk & 3) * 32), at(mK, kk * 2048), idesc_q, kk > 0);
+                umma_commit(bar(B_DQ));
+                for (int kk = 0; kk < qsteps; ++kk)
+                    umma_ss(tmem + C::TM_DK, at(mDS, kk * 2048), at(mQ, kk * 2048), idesc_kv, (t > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(bar(B_R));
+                if (t + 1 < n_own) {
+                    mbar_wait(bar(B_R), ph, status);                   // every product of the tile has completed
+                    mbar_wait(bar(B_DQR), ph, status);                 // dQ has been read and has left the dO tile
+                    load_tile(t + 1);
+                }
+            }
+        }
+        __syncwarp();
+    } else if (alive) {
+        // -------------------------------------------------------------------- element-wise, two threads per query row
+        const int h = (warp - 1) >> 2, q4 = warp & 3, r = 32 * q4 + lane;
+        const uint32_t tl = tmem + (static_cast<uint32_t>(32 * q4) << 16);
+        const float c2 = scale * kLog2e;
+        auto swz = [&](uint32_t tile, int chunk_bytes, int col) {      // 16-byte piece of this row that holds column col
+            return tile + (col >> 6) * chunk_bytes + r * 128 + ((((col & 63) >> 3) ^ (r & 7)) << 4);
+        };
+        for (int t = 0; t < n_own; ++t) {
+            const uint32_t ph = t & 1;
+            int bh, i0;
+            tile_at(t, bh, i0);
+            const int i = i0 + r;
+            const bool row_ok = i < Sq;
+            const size_t row = static_cast<size_t>(bh) * Sq + i;
+            const int vis = !row_ok ? 0 : causal ? min(Sk, i + dm.off + 1) : Sk;      // columns c < vis are visible
+            const float nlse = row_ok ? -__ldg(LSE + row) * kLog2e : 0.f;
+            float ndelta = 0.f;
+            if (DELTA != nullptr) {
+                if (row_ok) ndelta = -__ldg(DELTA + row);
+            } else {
+                // this thread's half of the row: O straight from global memory, asked for before the wait for the tiles, dO from its tile
+                uint4 o[D / 16];
+                const uint4* orow = reinterpret_cast<const uint4*>(O + row * Dg) + h * (D / 16);
+#pragma unroll
+                for (int p = 0; p < D / 16; ++p) o[p] = row_ok && h * (D / 2) + 8 * p < Dg ? __ldg(orow + p) : make_uint4(0, 0, 0, 0);
+                mbar_wait(bar(B_QO), ph, status);
+                float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                for (int p = 0; p < D / 16; ++p) {
+                    const float4 x = lds128(swz(sdO, C::Q_CHUNK, h * (D / 2) + 8 * p));
+                    const uint32_t a[4] = {__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z), __float_as_uint(x.w)};
+                    const uint32_t b[4] = {o[p].x, o[p].y, o[p].z, o[p].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        d0 = fmaf(__uint_as_float(a[e] << 16), __uint_as_float(b[e] << 16), d0);
+                        d1 = fmaf(__uint_as_float(a[e] & 0xffff0000u), __uint_as_float(b[e] & 0xffff0000u), d1);
+                    }
+                }
+                sts32(base + C::OFF_DELTA + (h * BM + r) * 4, d0 + d1);
+            }
+            uint32_t pk[2 * KC * 8];                                   // P of this thread's pieces, packed bf16
+            mbar_wait(bar(B_S), ph, status);
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 2 * KC; ++c) {
+                const int col = 16 * (2 * c + h);
+                if (col < Sk) {
+                    uint32_t v[16];
+                    tmem_ld16(tl + C::TM_S + col, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 2) {
+                        const float y0 = fmaf(__uint_as_float(v[e]), c2, nlse), y1 = fmaf(__uint_as_float(v[e + 1]), c2, nlse);
+                        pk[8 * c + e / 2] = pack_bf16(col + e < vis ? ex2(y0) : 0.f, col + e + 1 < vis ? ex2(y1) : 0.f);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        sts128(swz(sP, C::P_CHUNK, col + 8 * q), pk[8 * c + 4 * q], pk[8 * c + 4 * q + 1], pk[8 * c + 4 * q + 2],
+                               pk[8 * c + 4 * q + 3]);
+                }
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_P));
+            if (DELTA == nullptr) {
+                named_bar_sync(2, kCompute);                           // both halves of delta are there
+                ndelta = -(lds32f(base + C::OFF_DELTA + r * 4) + lds32f(base + C::OFF_DELTA + (BM + r) * 4));
+            }
+            mbar_wait(bar(B_DP), ph, status);
+            if (C::SHARED_P) mbar_wait(bar(B_DV), ph, status);         // dV has read P, whose place dS takes
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 2 * KC; ++c) {
+                const int col = 16 * (2 * c + h);
+                if (col < Sk) {
+                    uint32_t v[16], u[8];
+                    tmem_ld16(tl + C::TM_DP + col, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 2) {
+                        const uint32_t k = pk[8 * c + e / 2];
+                        const float a = __uint_as_float(k << 16) * (__uint_as_float(v[e]) + ndelta);
+                        const float b = __uint_as_float(k & 0xffff0000u) * (__uint_as_float(v[e + 1]) + ndelta);
+                        u[e / 2] = pack_bf16(col + e < vis ? a : 0.f, col + e + 1 < vis ? b : 0.f);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) sts128(swz(sDS, C::P_CHUNK, col + 8 * q), u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+                }
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_DS));
+            // dQ -> bf16 -> the dO tile (dead: dV was issued before dQ) -> TMA store
+            mbar_wait(bar(B_DQ), ph, status);
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c) {
+                const int col = h * (D / 2) + 32 * c;
+                uint32_t v[32], u[16];
+                tmem_ld32(tl + C::TM_S + col, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) u[e] = pack_bf16(__uint_as_float(v[2 * e]) * scale, __uint_as_float(v[2 * e + 1]) * scale);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    sts128(swz(sdO, C::Q_CHUNK, col + 8 * q), u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            named_bar_sync(1, kCompute);
+            if (r == 0 && h == 0) {
+#pragma unroll
+                for (int ch = 0; ch < C::NCH; ++ch) tma_store_3d(&tmdQ, sdO + ch * C::Q_CHUNK, ch * 64, i0, bh);
+                tma_store_commit_and_wait_read();
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_DQR));
+        }
+
+        // ---- this CTA's part of dV and dK (lanes = keys now), as f32 rows over the dead tiles
+        mbar_wait(bar(B_R), (n_own - 1) & 1, status);
+        tc_fence_after();
+        named_bar_sync(1, kCompute);                                   // the last dQ tile has been read by its store
+        if (r < 64 * KC) {
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t v[32];
+                tmem_ld32(tl + (h ? C::TM_DK : C::TM_DV) + 32 * c, v);
+                tmem_ld_wait();
+                const uint32_t to = base + (h * 64 * KC + r) * C::PITCH + c * 128;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) sts128(to + 16 * e, v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            }
+        }
+        tc_fence_before();
+    }
+    __syncwarp();
+    cluster_sync();
+    // ---- the parts of the cluster's CTAs added up, each CTA a range of the key rows, two tensors
+    if (alive) {
+        const int per = (Sk + n_share - 1) / n_share, j0 = share * per, nj = min(per, Sk - j0);
+        const int quads = Dg / 4;
+        for (int x = tid; x < 2 * max(nj, 0) * quads; x += kThreads) {
+            const int w = x / (nj * quads), rem = x - w * nj * quads, j = j0 + rem / quads, c = rem % quads;
+            const uint32_t at = base + (w * 64 * KC + j) * C::PITCH + c * 16;
+            float4 y[8];                                               // asked for together: a load takes about a thousand clocks
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k < n_share) y[k] = lds_cluster_128(cluster_map(at, k));
+            float4 s = y[0];
+#pragma unroll
+            for (int k = 1; k < 8; ++k)
+                if (k < n_share) s = make_float4(s.x + y[k].x, s.y + y[k].y, s.z + y[k].z, s.w + y[k].w);
+            const float f = w ? scale : 1.f;
+            *reinterpret_cast<uint2*>((w ? dK : dV) + (static_cast<size_t>(bhk) * Sk + j) * Dg + 4 * c) =
+                make_uint2(pack_bf16(s.x * f, s.y * f), pack_bf16(s.z * f, s.w * f));
+        }
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tmem, C::TM_COLS);
+    }
+    __syncwarp();
+    cluster_sync();                                                    // nobody leaves while its part is being read
+}
+
+// CTAs per head.  A head's tiles run one after the other in a CTA; dealing them to more CTAs shortens that chain until
+// the CTAs take turns on the SMs.  A CTA's set-up, its share of the reduction included, counts as one tile.
+inline int shares(int tiles, long long heads, long long slots) {
+    int best = 1;
+    long long best_cost = -1;
+    for (int n = 1; n <= 8 && n <= tiles; n *= 2) {
+        const long long cost = (heads * n + slots - 1) / slots * (1 + (tiles + n - 1) / n);
+        if (best_cost < 0 || cost < best_cost) {
+            best = n;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+template <int D, int KC>
+cudaError_t launch(const Problem& p, const void* q, const void* k, const void* v, const void* o, const void* d_o,
+                   const float* lse, const float* delta, void* dq, void* dk, void* dv, unsigned* status, cudaStream_t st)
+{
+    using C = Cfg<D, KC>;
+    CUtensorMap tq, tk, tv, tdo, tdq;
+    if (make_tmap_3d(&tq, q, 2, 1, p.BH(), p.Sq, p.D, 64, BM)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tk, k, 2, 1, p.BHkv(), p.Sk, p.D, 64, 64 * KC)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tv, v, 2, 1, p.BHkv(), p.Sk, p.D, 64, 64 * KC)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tdo, d_o, 2, 1, p.BH(), p.Sq, p.D, 64, BM)) return cudaErrorInvalidValue;
+    if (make_tmap_3d(&tdq, dq, 2, 1, p.BH(), p.Sq, p.D, 64, BM)) return cudaErrorInvalidValue;
+    auto kern = fast_bwd_small_kernel<D, KC>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (e != cudaSuccess) return MGN_FAIL(e, "cudaFuncSetAttribute");
+    const long long tiles = static_cast<long long>((p.Sq + BM - 1) / BM) * p.group();
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const int n_share = shares(static_cast<int>(tiles), p.BHkv(), kSms * C::CTAS);
+    const long long blocks = static_cast<long long>(p.BHkv()) * n_share;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const Dims dm{p.Sq, p.Sk, p.BH(), p.H, p.group(), p.off()};
+    e = launch_clusters(kern, static_cast<unsigned>(blocks), static_cast<unsigned>(n_share), kThreads, C::SMEM, st, tq, tk, tv, tdo, tdq,
+                        static_cast<const __nv_bfloat16*>(o), lse, delta, static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv),
+                        dm, n_share, p.causal, p.scale, p.D, status);
+    return MGN_FAIL(e, "small backward launch");
+}
+
+}  // namespace
+
+cudaError_t launch_fast_bwd_small(const Problem& p, const void* q, const void* k, const void* v, const void* o,
+                                  const void* d_o, const float* lse, const float* delta, void* dq, void* dk, void* dv,
+                                  unsigned* status, cudaStream_t st)
+{
+    const bool one = p.Sk <= 64;
+    switch (p.D) {
+        case 32:  // the 64-wide build on zero-filled 32-element rows (see fast_fwd.cu)
+        case 64:
+            return one ? launch<64, 1>(p, q, k, v, o, d_o, lse, delta, dq, dk, dv, status, st)
+                       : launch<64, 2>(p, q, k, v, o, d_o, lse, delta, dq, dk, dv, status, st);
+        case 128:
+            return one ? launch<128, 1>(p, q, k, v, o, d_o, lse, delta, dq, dk, dv, status, st)
+                       : launch<128, 2>(p, q, k, v, o, d_o, lse, delta, dq, dk, dv, status, st);
+        default: return cudaErrorNotSupported;
+    }
+}
+
+}  // namespace mgn

@@ -264,6 +264,27 @@ cudaError_t launch_fast_bwd(const Problem& p, const void* q, const void* k, cons
                             float* dq_acc, void* dq, void* dk, void* dv,
                             unsigned* sched, unsigned* status, cudaStream_t st);
 
+// The latency path of the backward: one block of keys, small CTAs, no preprocess pass (delta may be null: it is then formed
+// from o) and no atomics.  The lines, in us of a backward, persistent kernel / this one:
+// - Deterministic, where the persistent dK+dV kernel and the dQ pass stand behind the preprocess pass: always (16 x 8 heads of
+//   1024 x 77, D = 64: 71 / 39; 64 x 16 of 2048 x 128, D = 128: 1131 / 763), but for many heads of one tile at D = 128,
+//   where one CTA fits an SM (512 heads of 100 x 100: 67 / 78).
+// - Otherwise D <= 64 with at most 64 keys (64 x 8 heads of 50 x 16: 29.7 / 19.5; 1024 heads of 2048 x 16: 386 / 259), or, with
+//   more, eight tiles a head and heads for one round of CTAs (8 heads of 2048 x 128: 48 / 21; 128 of 1024 x 77: 39.8 / 38.9;
+//   but 128 of 512 x 100: 25.6 / 28.7, of 100 x 100: 15.3 / 18.4; 1024 of 2048 x 128: 388 / 416).
+// - D = 128: heads that leave half of the SMs idle, with four tiles a head (eight beyond 64 keys): 8 heads of 2048 x 128
+//   69 / 27, 64 of 2048 x 100 81 / 69, 64 of 500 x 50 29.7 / 25.5; but 32 of 300 x 100 23.5 / 26.6, 128 of 1024 x 77 54 / 66.
+inline bool fast_bwd_is_small(const Problem& p, bool deterministic) {
+    if (p.Sk > 128) return false;
+    const long long tiles = static_cast<long long>(p.group()) * ((p.Sq + 127) / 128);
+    if (deterministic) return !(p.D == 128 && p.Sk > 64 && tiles == 1 && p.BHkv() > kSms);
+    if (p.D == 128) return p.BHkv() <= kSms / 2 && tiles >= (p.Sk <= 64 ? 4 : 8);
+    return p.Sk <= 64 || (tiles >= 8 && p.BHkv() <= 2 * kSms);
+}
+cudaError_t launch_fast_bwd_small(const Problem& p, const void* q, const void* k, const void* v, const void* o,
+                                  const void* d_o, const float* lse, const float* delta, void* dq, void* dk, void* dv,
+                                  unsigned* status, cudaStream_t st);
+
 // Deterministic fast backward: launch_fast_bwd with dq_acc == nullptr runs the fused dK+dV kernel
 // without the dQ product and reductions (dq is not touched), and this separate pass computes dQ.
 cudaError_t launch_fast_dq(const Problem& p, const void* q, const void* k, const void* v, const void* d_o,

@@ -1,0 +1,55 @@
+"""Fast backward over one block of keys (S_k <= 128; csrc/fast_bwd_small.cu): against the f64 oracle at the edges of its
+16-key steps, 64-key chunks and 128-row tiles, with a head's tiles on one CTA and dealt to a cluster, grouped heads, a
+causal offset, and delta formed by the kernel or given."""
+import math
+
+import pytest
+import torch
+
+from paper_2608_01563_b200 import binding as mgn
+
+import helpers as hp
+
+pytestmark = pytest.mark.gpu
+MODE, BF = mgn.MODE_FAST_BF16, torch.bfloat16
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal", [
+    (1, 2, 2, 1, 1, 64, False),
+    (1, 2, 2, 129, 15, 128, False),
+    (2, 3, 3, 128, 17, 32, False),
+    (1, 4, 2, 300, 64, 64, False),        # six tiles of a group: a cluster of several CTAs
+    (1, 4, 4, 60, 65, 64, True),          # the second chunk holds one key
+    (1, 2, 1, 1100, 77, 128, False),      # eighteen tiles over eight CTAs: shares of two and three
+    (2, 2, 2, 127, 128, 128, True),
+    (40, 8, 8, 260, 60, 64, False),       # more heads than CTAs at a time: one CTA walks over a head's three tiles
+])
+def test_matches_the_oracle(B, H, Hkv, Sq, Sk, D, causal):
+    g = torch.Generator().manual_seed(Sq + Sk)
+    q, d_o = (torch.randn(B, H, Sq, D, generator=g).to(BF) for _ in range(2))
+    k, v = (torch.randn(B, Hkv, Sk, D, generator=g).to(BF) for _ in range(2))
+    scale = 1.0 / math.sqrt(D)
+    qd, kd, vd, dod = (t.cuda() for t in (q, k, v, d_o))
+    o, lse = torch.empty_like(qd), torch.empty(B, H, Sq, device="cuda")
+    mgn.mgn_attn_fwd_ext(qd, kd, vd, o, lse, causal, scale, MODE)
+    delta = (o.float() * dod.float()).sum(-1).contiguous()
+    ws = mgn.alloc_workspace(B, H, Sq, D, MODE)
+    heads = slice(0, 2) if B > 2 else slice(None)          # the oracle on two batch elements at most
+    ref = hp.run_oracle_ext(q[heads], k[heads], v[heads], d_o[heads], causal, scale)
+
+    def run(call):
+        ws.fill_(0xFF)
+        dq = hp.Guarded((B, H, Sq, D), BF)
+        dk, dv = (hp.Guarded((B, Hkv, Sk, D), BF) for _ in range(2))
+        call(dq.view, dk.view, dv.view)
+        mgn.mgn_attn_check()
+        got = {"dQ": dq.check("dQ"), "dK": dk.check("dK"), "dV": dv.check("dV")}
+        hp.check_fast({n: t[heads].double().numpy() for n, t in got.items()}, ref, names=("dQ", "dK", "dV"))
+        return got
+
+    run(lambda x, y, z: mgn.mgn_attn_bwd_ext(qd, kd, vd, o, dod, lse, x, y, z, ws, causal, scale, MODE))
+    a = run(lambda x, y, z: mgn.mgn_attn_bwd_deterministic(qd, kd, vd, o, dod, lse, x, y, z, ws, causal, scale, MODE))
+    b = run(lambda x, y, z: mgn.mgn_attn_bwd_deterministic(qd, kd, vd, o, dod, lse, x, y, z, ws, causal, scale, MODE))
+    run(lambda x, y, z: mgn.mgn_attn_bwd_given_delta(qd, kd, vd, dod, lse, delta, x, y, z, ws, causal, scale, MODE))
+    for n in a:
+        assert torch.equal(a[n], b[n]), f"{n} differs between runs"
