@@ -23,7 +23,9 @@
 //         Global f32 reduce-add runs at about 20 bytes per clock per SM on this part (3300 clocks
 //         for one 64 KB partial), and issued from the load/store unit it stalls every shared-memory
 //         access of the SM; so it goes through TMA and is waited for only by the drain warps.
-// Two issuing threads share the tensor core.  Issuer A runs MMA4(n), MMA1(n+1) as soon as P^T(n)
+// Two issuing warps share the tensor core (a warp computes the operands in step and an elected lane issues: a lane in a
+// branch of its own has to move them to the uniform registers first; (2,16,4096,128) causal, forward and backward, both
+// kernels 616 -> 607 us, the deterministic backward of (4,32,1024,128) 274 -> 267).  Issuer A runs MMA4(n), MMA1(n+1) as soon as P^T(n)
 // is in tensor memory (before dS(n) exists), so the next scores are ready when the compute warps
 // come back for them; issuer B runs MMA6(n), MMA2(n+1), MMA5(n) once dS(n) is in shared memory
 // (the dQ partial first so its drain starts early, dP^T of the next pair as soon as Y has been
@@ -162,7 +164,7 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     // dS(g) complete: one barrier per parity of g, so that a waiter two pairs behind cannot alias phases
     auto pds_bar = [&](int g) { return bars + 8u * ((g & 1) ? B_PDSFULL1 : B_PDSFULL); };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
     if (base + C::PAYLOAD > smem_u32(smem_raw) + C::SMEM) {           // alignment slack ran out
         if (tid == 0) atomicMax(status, kStatusSmemLayout);
@@ -191,8 +193,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         return it;
     };
     auto read_item = [&](int k) -> int {
-        if (!mbar_wait(bar(B_ITEM + (k & 3)), (k >> 2) & 1, status)) return -1;
-        return static_cast<int>(lds32u(item_slot + 4u * (k & 3)));
+        if (!__all_sync(0xffffffffu, mbar_wait(bar(B_ITEM + (k & 3)), (k >> 2) & 1, status))) return -1;
+        return static_cast<int>(__shfl_sync(0xffffffffu, lds32u(item_slot + 4u * (k & 3)), 0));
     };
     const float c2 = scale * kLog2e;
 
@@ -212,7 +214,7 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
     // Launched as a programmatic dependent of the preprocess kernel: everything above overlapped its
     // tail; delta, the cleared accumulator and the work-item counter are read only after this wait.
     pdl_launch_dependents();
@@ -251,7 +253,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 }
             }
         }
-        } else if ((warp == 1 || warp == 2) && lane == 0) {
+        } else if (warp == 1 || warp == 2) {
+        const uint32_t leader = elect_one();               // the whole warp walks along, one lane issues
         // ------------------------------------------------------------------ MMA issuers
         {
             constexpr uint32_t idesc_st = umma_idesc_bf16(BLK, BLK, false, false);   // S^T, dP^T
@@ -259,8 +262,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             constexpr uint32_t idesc_dq = umma_idesc_bf16(BLK, D, true, true);       // A MN-major, B MN-major
             // Descriptors are built once; inside the loops only the start-address field moves (it
             // holds address >> 4 and cannot carry out of its 14 bits within shared memory).
-            auto kmajor_off = [](int kk) { return static_cast<uint64_t>(((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32) >> 4); };
-            auto mn_off = [](int kk) { return static_cast<uint64_t>((kk * 2048) >> 4); };
+            auto kmajor_off = [](int kk) { return static_cast<uint32_t>((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32); };
+            auto mn_off = [](int kk) { return static_cast<uint32_t>(kk * 2048); };
             const uint32_t tXa = tmem + C::TM_X, tYa = tmem + C::TM_Y, tDK = tmem + C::TM_DK, tDV = tmem + C::TM_DV;
             if (warp == 1) {
                 // ---- issuer A: dV += P^T dO (MMA4), then the next S^T = K Q^T (MMA1) into X
@@ -269,8 +272,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 auto mma1 = [&](int g) {
                     const uint64_t qd = kQ + static_cast<uint64_t>(((g & 1) * C::TILE_BYTES) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) umma_ss(tXa, kK + kmajor_off(kk), qd + kmajor_off(kk), idesc_st, kk > 0);
-                    umma_commit(bar(B_SFULL));
+                    for (int kk = 0; kk < D / 16; ++kk) umma_ss_warp(leader, tXa, desc_at(kK, kmajor_off(kk)), desc_at(qd, kmajor_off(kk)), idesc_st, kk > 0);
+                    umma_commit_warp(leader, bar(B_SFULL));
                 };
                 int g = 0;
                 for (int k = 0;; ++k) {
@@ -292,17 +295,17 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         // P^T: queries 0-63 at X[0,32), queries 64-127 at X[64,96)
 #pragma unroll
                         for (int kk = 0; kk < BLK / 16; ++kk)
-                            umma_ts(tDV, tXa + (kk >> 2) * 64 + (kk & 3) * 8, mdO + mn_off(kk), idesc_dv,
+                            umma_ts_warp(leader, tDV, tXa + (kk >> 2) * 64 + (kk & 3) * 8, desc_at(mdO, mn_off(kk)), idesc_dv,
                                     (kk > 0 || n > 0) ? 1u : 0u);
-                        umma_commit(bar(B_DOEMPTY));
+                        umma_commit_warp(leader, bar(B_DOEMPTY));
                         if (n + 1 < w.N) {
                             mbar_wait(bar(B_QFULL + ((g + 1) & 1)), ((g + 1) >> 1) & 1, status);
                             tc_fence_after();
                             mma1(g + 1);      // X is free once MMA4 has read P^T (same issuer: in order)
                         }
                     }
-                    umma_commit(bar(B_DVFULL));
-                    umma_commit(bar(B_KVEMPTY));      // this issuer's last product with K of this item is done
+                    umma_commit_warp(leader, bar(B_DVFULL));
+                    umma_commit_warp(leader, bar(B_KVEMPTY));      // this issuer's last product with K of this item is done
                 }
             } else {
                 // ---- issuer B: dQ partial (MMA6), dP^T of the next pair (MMA2), dK (MMA5)
@@ -311,9 +314,9 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const uint64_t mK = umma_smem_desc(sK, C::CHUNK_BYTES, 1024), mQ = umma_smem_desc(sQ, C::CHUNK_BYTES, 1024);
                 auto mma2 = [&]() {
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) umma_ss(tYa, kV + kmajor_off(kk), kdO + kmajor_off(kk), idesc_st, kk > 0);
-                    umma_commit(bar(B_DPFULL));
-                    umma_commit(bar(B_DOEMPTY));     // with issuer A's arrival after dV: both readers of dO are done
+                    for (int kk = 0; kk < D / 16; ++kk) umma_ss_warp(leader, tYa, desc_at(kV, kmajor_off(kk)), desc_at(kdO, kmajor_off(kk)), idesc_st, kk > 0);
+                    umma_commit_warp(leader, bar(B_DPFULL));
+                    umma_commit_warp(leader, bar(B_DOEMPTY));     // with issuer A's arrival after dV: both readers of dO are done
                 };
                 int g = 0;
                 for (int k = 0;; ++k) {
@@ -331,8 +334,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         tc_fence_after();
                         if constexpr (WITH_DQ) {
 #pragma unroll
-                            for (int kk = 0; kk < BLK / 16; ++kk) umma_ss(tYa, mdS + mn_off(kk), mK + mn_off(kk), idesc_dq, kk > 0);
-                            umma_commit(bar(B_DQFULL));
+                            for (int kk = 0; kk < BLK / 16; ++kk) umma_ss_warp(leader, tYa, desc_at(mdS, mn_off(kk)), desc_at(mK, mn_off(kk)), idesc_dq, kk > 0);
+                            umma_commit_warp(leader, bar(B_DQFULL));
                         }
                         if (n + 1 < w.N) {
                             mbar_wait(bar(B_DOFULL), (g + 1) & 1, status);
@@ -343,12 +346,12 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         if (n == 0) mbar_wait(bar(B_DKVEMPTY), (k & 1) ^ 1, status);   // last item's dK has been read out
 #pragma unroll
                         for (int kk = 0; kk < BLK / 16; ++kk)
-                            umma_ss(tDK, kdS + kmajor_off(kk), qm + mn_off(kk), idesc_dv, (kk > 0 || n > 0) ? 1u : 0u);
-                        umma_commit(bar(B_QEMPTY + (g & 1)));
-                        umma_commit(bar(B_DSEMPTY));                             // dS(n) buffer may be rewritten
+                            umma_ss_warp(leader, tDK, desc_at(kdS, kmajor_off(kk)), desc_at(qm, mn_off(kk)), idesc_dv, (kk > 0 || n > 0) ? 1u : 0u);
+                        umma_commit_warp(leader, bar(B_QEMPTY + (g & 1)));
+                        umma_commit_warp(leader, bar(B_DSEMPTY));                             // dS(n) buffer may be rewritten
                     }
-                    umma_commit(bar(B_DKFULL));
-                    umma_commit(bar(B_KVEMPTY));
+                    umma_commit_warp(leader, bar(B_DKFULL));
+                    umma_commit_warp(leader, bar(B_KVEMPTY));
                 }
             }
         }

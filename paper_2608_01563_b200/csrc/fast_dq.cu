@@ -66,7 +66,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const uint32_t tmem_slot = bars + B_COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
 
     // Heaviest (last) query tiles first when causal.
@@ -87,7 +87,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
 
     if (warp < 4) {
         reg_dealloc<96>();
@@ -113,15 +113,16 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 for (int ch = 0; ch < C::NCH; ++ch)
                     tma_load_3d(sV + sv * C::TILE_BYTES + ch * C::CHUNK_BYTES, &tmV, bar(B_PGO + sv), ch * 64, n * BLK, bhk);
             }
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1) {
+            const uint32_t leader = elect_one();           // the whole warp walks along, one lane issues
             // ------------------------------------------------------------------ S and dP
             constexpr uint32_t idesc_s = umma_idesc_bf16(BLK, BLK, false, false);    // both operands K-major
             const uint64_t dQd = umma_smem_desc(sQ, 16, 1024), dOd = umma_smem_desc(sdO, 16, 1024);
             const uint64_t dK0 = umma_smem_desc(sK, 16, 1024), dV0 = umma_smem_desc(sV, 16, 1024);
             const uint32_t tP = tmem + C::TM_P;
-            auto koff = [](int kk) { return static_cast<uint64_t>(((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32) >> 4); };
-            mbar_arrive(bar(B_SFREE));
-            mbar_arrive(bar(B_SFREE + 1));
+            auto koff = [](int kk) { return static_cast<uint32_t>((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32); };
+            if (leader) mbar_arrive(bar(B_SFREE));
+            if (leader) mbar_arrive(bar(B_SFREE + 1));
             mbar_wait(bar(B_Q), 0, status);
             for (int n = 0; n < n_kb; ++n) {
                 const int w = n & 1;
@@ -132,15 +133,16 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 mbar_wait(bar(B_SFREE + w), (n >> 1) & 1, status);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tS, dQd + koff(kk), kst + koff(kk), idesc_s, kk > 0);
-                umma_commit(bar(B_SDONE + w));
+                for (int kk = 0; kk < D / 16; ++kk) umma_ss_warp(leader, tS, desc_at(dQd, koff(kk)), desc_at(kst, koff(kk)), idesc_s, kk > 0);
+                umma_commit_warp(leader, bar(B_SDONE + w));
                 mbar_wait(bar(B_PGO + w), (n >> 1) & 1, status);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) umma_ss(tP, dOd + koff(kk), vst + koff(kk), idesc_s, kk > 0);
-                umma_commit(bar(B_PDONE));
+                for (int kk = 0; kk < D / 16; ++kk) umma_ss_warp(leader, tP, desc_at(dOd, koff(kk)), desc_at(vst, koff(kk)), idesc_s, kk > 0);
+                umma_commit_warp(leader, bar(B_PDONE));
             }
-        } else if (warp == 2 && lane == 0) {
+        } else if (warp == 2) {
+            const uint32_t leader = elect_one();
             // ------------------------------------------------------------------ dQ
             constexpr uint32_t idesc_q = umma_idesc_bf16(BLK, D, false, true);       // A from tensor memory, B MN-major
             const uint64_t mK0 = umma_smem_desc(sK, C::CHUNK_BYTES, 1024);
@@ -152,10 +154,10 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 tc_fence_after();
 #pragma unroll
                 for (int kk = 0; kk < BLK / 16; ++kk)
-                    umma_ts(tDQ, tS + (kk >> 2) * 64 + (kk & 3) * 8, kst + static_cast<uint64_t>((kk * 2048) >> 4), idesc_q,
+                    umma_ts_warp(leader, tDQ, tS + (kk >> 2) * 64 + (kk & 3) * 8, desc_at(kst, kk * 2048), idesc_q,
                             (kk > 0 || n > 0) ? 1u : 0u);
-                umma_commit(bar(B_QDONE + n % 3));
-                umma_commit(bar(B_SFREE + (n & 1)));
+                umma_commit_warp(leader, bar(B_QDONE + n % 3));
+                umma_commit_warp(leader, bar(B_SFREE + (n & 1)));
             }
         }
         __syncwarp();

@@ -175,7 +175,7 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t tmem_slot = bars + B_COUNT * 8;
     auto bar = [&](int i) { return bars + 8u * i; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     bool alive = true;                                     // false: an earlier wait on this device gave up
     if constexpr (SPLIT) {                                 // the CTA stays for its cluster, and does nothing
         if (tid == 0) sts32u(tmem_slot + 4, *reinterpret_cast<volatile unsigned*>(status));
@@ -211,7 +211,7 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = lds32u(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
 
     if (warp < 4) {
         reg_dealloc<72>();
@@ -260,7 +260,8 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 }
             }
         }
-        } else if ((warp == 1 || warp == 3) && lane == 0) {
+        } else if (warp == 1 || warp == 3) {
+        const uint32_t leader = elect_one();               // the whole warp walks along, one lane issues
         // ------------------------------------------------------------------ MMA issuers
         // Two lanes, each walking over this CTA's blocks (all items in sequence): warp 1 issues the score
         // products, which run up to two blocks ahead of the softmax warps, warp 3 the P V products.
@@ -275,8 +276,8 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (warp == 1) {
                 const uint64_t dQ0 = umma_smem_desc(sQ, 16, 1024);
                 const uint64_t dK0 = umma_smem_desc(sK, 16, 1024);
-                mbar_arrive(bar(B_SGO));         // blocks 0 and 1 have no product before them to wait for
-                mbar_arrive(bar(B_SGO + 1));
+                if (leader) mbar_arrive(bar(B_SGO));         // blocks 0 and 1 have no product before them to wait for
+                if (leader) mbar_arrive(bar(B_SGO + 1));
                 for (int k = 0; k < n_tiers; ++k) {
                     const int it = index_of(k);
                     if (it < 0) break;
@@ -292,13 +293,13 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         const uint32_t tS = tmem + C::TM_S + b * 128;
 #pragma unroll
                         for (int kk = 0; kk < D / 16; ++kk) {
-                            const uint64_t off = static_cast<uint64_t>(((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32) >> 4);
-                            umma_ss(tS, qd + off, kd + off, idesc_s, kk > 0);
+                            const uint32_t off = static_cast<uint32_t>((kk >> 2) * C::CHUNK_BYTES + (kk & 3) * 32);
+                            umma_ss_warp(leader, tS, desc_at(qd, off), desc_at(kd, off), idesc_s, kk > 0);
                         }
-                        umma_commit(bar(B_SFULL + b));
-                        umma_commit(bar(B_KEMPTY + b));
+                        umma_commit_warp(leader, bar(B_SFULL + b));
+                        umma_commit_warp(leader, bar(B_KEMPTY + b));
                     }
-                    umma_commit(bar(B_QEMPTY + qs));      // that was this item's last S product
+                    umma_commit_warp(leader, bar(B_QEMPTY + qs));      // that was this item's last S product
                 }
             } else {
                 const uint64_t dV0 = umma_smem_desc(sV, C::CHUNK_BYTES, 1024);
@@ -316,12 +317,12 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                         const uint32_t tP = tmem + C::TM_P + b * 64;
 #pragma unroll
                         for (int kk = 0; kk < BN / 16; ++kk)
-                            umma_ts(tO, tP + kk * 8, vd + static_cast<uint64_t>((kk * 2048) >> 4), idesc_o, (kk > 0 || n > 0) ? 1u : 0u);
-                        umma_commit(bar(B_SGO + b));          // with K(g+2): S(g+2) may go
-                        umma_commit(bar(B_VEMPTY + b));
-                        umma_commit(bar(B_PVDONE + b));
+                            umma_ts_warp(leader, tO, tP + kk * 8, desc_at(vd, kk * 2048), idesc_o, (kk > 0 || n > 0) ? 1u : 0u);
+                        umma_commit_warp(leader, bar(B_SGO + b));          // with K(g+2): S(g+2) may go
+                        umma_commit_warp(leader, bar(B_VEMPTY + b));
+                        umma_commit_warp(leader, bar(B_PVDONE + b));
                     }
-                    umma_commit(bar(B_OFULL));
+                    umma_commit_warp(leader, bar(B_OFULL));
                 }
             }
         }
