@@ -202,7 +202,7 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int i = 0; i < B_COUNT; ++i) {
             uint32_t cnt = 1;
             if (i == B_PDSFULL || i == B_PDSFULL1 || i == B_PFULL || i == B_DKVEMPTY) cnt = 256;
-            if (i == B_DQEMPTY) cnt = 128;
+            if (i == B_DQEMPTY || (!WITH_DQ && i == B_DKVEMPTY)) cnt = 128;
             if (i == B_STATFULL || i == B_STATFULL + 1) cnt = 32;
             if (i == B_KVEMPTY || i == B_DOEMPTY) cnt = 2;   // one arrival per issuer
             mbar_init(bar(i), cnt);
@@ -217,8 +217,8 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t tmem = __shfl_sync(0xffffffffu, lds32u(tmem_slot), 0);
     // Launched as a programmatic dependent of the preprocess kernel: everything above overlapped its
     // tail; delta, the cleared accumulator and the work-item counter are read only after this wait.
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();   // behind the wait: the separate dQ pass reads delta without a wait of its own
 
     if (warp < 4) {
         reg_dealloc<104>();
@@ -392,6 +392,56 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const int r = tid - 384;                           // query row of the block = tensor-memory lane
         const uint32_t tY = tmem + (static_cast<uint32_t>(r & ~31) << 16) + C::TM_Y;
         const uint32_t stage = base + C::OFF_DQ;
+        if constexpr (!WITH_DQ) {
+            // Without a dQ partial to drain these warps write out dK and dV, so that the compute warps go on with the next
+            // item: tensor memory -> bf16 -> the staging area, one tensor at a time -> coalesced 16-byte stores.
+            const uint32_t tl = tmem + (static_cast<uint32_t>(r & ~31) << 16);
+            constexpr int PCS = D / 8;                     // 16-byte pieces of a row
+            auto at = [&](int row, int piece) { return stage + (piece >> 3) * C::CHUNK_BYTES + row * 128 + (((piece & 7) ^ (row & 7)) << 4); };
+            for (int k = 0;; ++k) {
+                const int it = read_item(k);
+                if (it < 0) break;
+                const Item<GEN> w = make_item<GEN>(it, dm, causal);
+                mbar_wait(bar(B_DVFULL), k & 1, status);
+                mbar_wait(bar(B_DKFULL), k & 1, status);
+                tc_fence_after();
+                uint32_t u[D / 2];
+                auto read = [&](uint32_t col, float mul) {
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c) {
+                        uint32_t v[32];
+                        tmem_ld32(tl + col + 32 * c, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e)
+                            u[16 * c + e] = pack_bf16(__uint_as_float(v[2 * e]) * mul, __uint_as_float(v[2 * e + 1]) * mul);
+                    }
+                };
+                auto put = [&]() {
+#pragma unroll
+                    for (int p = 0; p < PCS; ++p) sts128(at(r, p), u[4 * p], u[4 * p + 1], u[4 * p + 2], u[4 * p + 3]);
+                };
+                auto store = [&](__nv_bfloat16* out) {
+                    named_bar_sync(4, 128);
+                    out += (static_cast<size_t>(w.bhk) * Sk + w.j0) * Dg;
+#pragma unroll 4
+                    for (int i = 0; i < PCS; ++i) {
+                        const int idx = i * 128 + r, row = idx / PCS, piece = idx % PCS;   // a warp covers whole rows
+                        if (piece * 8 < Dg && w.j0 + row < Sk)
+                            *reinterpret_cast<float4*>(out + static_cast<size_t>(row) * Dg + piece * 8) = lds128(at(row, piece));
+                    }
+                    named_bar_sync(4, 128);                // the slab has been read: the staging area may be rewritten
+                };
+                read(C::TM_DV, 1.0f);
+                put();
+                read(C::TM_DK, scale);
+                tc_fence_before();
+                mbar_arrive(bar(B_DKVEMPTY));              // the next item may accumulate into dK, dV
+                store(dV);
+                put();
+                store(dK);
+            }
+        }
         int g = 0;
         for (int k = 0; WITH_DQ; ++k) {
         const int it = read_item(k);
@@ -559,11 +609,11 @@ fast_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (n + 1 < w.N) exp_phase(w, n + 1, g + 1);
         }
 
-        // ---- item epilogue.  Each warpgroup writes D/2 columns of dV, then D/2 columns of dK (scaled):
+        // ---- item epilogue (without a dQ partial: the drain warps').  Each warpgroup writes D/2 columns of dV, then D/2 columns of dK (scaled):
         // tensor memory -> bf16 registers -> this warpgroup's half of the dS buffer (idle here) ->
         // coalesced 16-byte global stores.  Not a TMA store: it would queue behind the dQ reductions
         // of the last pairs in the copy engine.
-        {
+        if constexpr (WITH_DQ) {
             constexpr int HC = D / 2;                      // columns per warpgroup and tensor
             constexpr int PCS = HC / 8;                    // 16-byte pieces per staged row
             const uint32_t stage = sdS + half * C::CHUNK_BYTES;

@@ -13,6 +13,8 @@
 // S has two regions: S(n+1) and dQ(n-1) run while the arithmetic of block n does, and dP(n+1) follows
 // as soon as dP(n) has been read, so a block costs its arithmetic; with one S region the products and the
 // arithmetic took turns.  (4,32,1024,128) causal, forward and deterministic backward: 261 -> 253 us.
+// Heads in groups whose tensors stay in L2, launched beside the draining dK+dV kernel, arithmetic on pairs of columns; and the
+// dK+dV kernel's results written by its otherwise idle drain warps: 274 -> 268 us.
 // Epilogue: dQ * scale -> bf16 -> shared memory (the dead Q tile) -> TMA store.
 // Warp roles (384 threads): warp 0 TMA producer, warps 1 and 2 one MMA-issuing lane each (S and dP; dQ),
 // warps 4-11 compute.
@@ -56,7 +58,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                const __grid_constant__ CUtensorMap tmdQ,
                const float* __restrict__ LSE, const float* __restrict__ DELTA,
-               const Dims dm, int n_qt, int causal, float scale, unsigned* status)
+               const Dims dm, int n_qt, int Hg, int causal, float scale, unsigned* status)
 {
     using C = Cfg<D>;
     extern __shared__ uint8_t smem_raw[];
@@ -67,11 +69,15 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     auto bar = [&](int i) { return bars + 8u * i; };
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    if (*reinterpret_cast<volatile unsigned*>(status) != 0) return;   // an earlier wait on this device gave up
+    if (*reinterpret_cast<volatile unsigned*>(status) != 0) {         // an earlier wait on this device gave up
+        pdl_wait();
+        return;
+    }
 
     // Heaviest (last) query tiles first when causal.
-    const int qt = n_qt - 1 - static_cast<int>(blockIdx.x) / dm.BH;
-    const int bh = static_cast<int>(blockIdx.x) % dm.BH;
+    int tile, bh;
+    item_of_block(static_cast<int>(blockIdx.x), n_qt, dm.BH, Hg, tile, bh);
+    const int qt = n_qt - 1 - tile;
     const int bhk = (bh / dm.H) * (dm.H / dm.G) + (bh % dm.H) / dm.G;   // key/value head of this query head
     const int i0 = qt * BLK;
     const int n_kb_all = (dm.Sk + BLK - 1) / BLK;
@@ -179,6 +185,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // K is NaN.
         const int tile_last = causal ? i0 + dm.off : dm.Sk - 1, row_last = causal ? i + dm.off : dm.Sk - 1;
 
+        const uint64_t c2x2 = f2_pack(c2, c2), nlse = f2_pack(-lse2, -lse2), ndl = f2_pack(-dl, -dl);
         for (int n = 0; n < n_kb; ++n) {
             const int j0 = n * BLK + 64 * h;
             const bool masked = j0 + 63 > tile_last;
@@ -193,10 +200,17 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 tmem_ld32(tS + 32 * c, s);
                 tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    p[32 * c + e] = ex2(fmaf(__uint_as_float(s[e]), c2, -lse2));
-                    if (masked && 32 * c + e > jmax) p[32 * c + e] = 0.f;
+                for (int e = 0; e < 32; e += 2) {
+                    float y0, y1;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2x2, nlse), y0, y1);
+                    p[32 * c + e] = ex2(y0);
+                    p[32 * c + e + 1] = ex2(y1);
                 }
+            }
+            if (masked) {
+#pragma unroll
+                for (int e = 0; e < 64; ++e)
+                    if (e > jmax) p[e] = 0.f;
             }
             mbar_wait(bar(B_PDONE), n & 1, status);
             tc_fence_after();
@@ -210,9 +224,12 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             for (int c = 0; c < 2; ++c) {
                 uint32_t u[16];
 #pragma unroll
-                for (int e = 0; e < 32; e += 2)
-                    u[e / 2] = pack_bf16(p[32 * c + e] * (__uint_as_float(dp[c][e]) - dl),
-                                         p[32 * c + e + 1] * (__uint_as_float(dp[c][e + 1]) - dl));
+                for (int e = 0; e < 32; e += 2) {
+                    float a, b;
+                    f2_unpack(f2_mul(f2_pack(p[32 * c + e], p[32 * c + e + 1]),
+                                     f2_add(f2_pack(__uint_as_float(dp[c][e]), __uint_as_float(dp[c][e + 1])), ndl)), a, b);
+                    u[e / 2] = pack_bf16(a, b);
+                }
                 tmem_st16(tS + 16 * c, u);                 // dS of this half: packed columns [64h, 64h + 32)
             }
             tmem_st_wait();
@@ -255,6 +272,7 @@ fast_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, C::TM_COLS);
+    pdl_wait();     // this grid must not complete before the one it may have started beside
 }
 
 template <int D>
@@ -275,9 +293,8 @@ cudaError_t launch(const Problem& p, const void* q, const void* k, const void* v
     const long long blocks = static_cast<long long>(n_qt) * p.BH();
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     const Dims dm{p.Sq, p.Sk, p.BH(), p.H, p.group(), p.off()};
-    kern<<<static_cast<unsigned>(blocks), kThreads, C::SMEM, st>>>(tq, tk, tv, tdo, tdq, lse, delta, dm, n_qt, p.causal,
-                                                                   p.scale, status);
-    return cudaGetLastError();
+    return launch_pdl(kern, static_cast<unsigned>(blocks), kThreads, C::SMEM, st, tq, tk, tv, tdo, tdq, lse, delta, dm, n_qt,
+                      head_group(4.0 * p.Sk * D / p.group(), p.BH()), p.causal, p.scale, status);
 }
 
 }  // namespace

@@ -23,6 +23,7 @@
 // Forward and backward, in us: (8,12,1024,64) causal 484 -> 458, (32,12,197,64) 281 -> 259, (4,32,1024,128) causal
 // 1259 -> 1152.
 #pragma once
+#include "fast_items.cuh"
 #include "kernels.h"
 #include "umma.cuh"
 
@@ -92,26 +93,6 @@ __device__ __forceinline__ void store_quad(uint32_t at, const float4 x) {
     sts64(at, h[0], h[1]);
     sts64(at + part_bytes<R>(), m[0], m[1]);
     sts64(at + 2 * part_bytes<R>(), l[0], l[1]);
-}
-
-// CTA -> (tile in order of falling weight, head).  Heads come in groups whose streamed tensors stay in L2 while the
-// group's CTAs run; within a group every head's heaviest tile comes first.
-__device__ __forceinline__ void item_of_block(int block, int n_tiles, int heads, int group, int& tile, int& head) {
-    const int g = block / (n_tiles * group), rem = block - g * n_tiles * group;
-    const int size = min(group, heads - g * group);
-    tile = rem / size;
-    head = g * group + rem % size;
-}
-// `bytes`: what the CTAs of one head share.  One group while everything fits half of L2; else a quarter of L2 a
-// group, equal groups ((4,32,1024,128) causal forward 0.282 -> 0.261 ms; its K and V are 134 MB).
-inline int head_group(double bytes, int heads) {
-    int dev = 0, l2 = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || l2 <= 0)
-        l2 = 126 << 20;
-    if (bytes * heads <= 0.5 * l2) return heads;
-    const double n = 0.25 * l2 / bytes;
-    const int most = n < 1.0 ? 1 : static_cast<int>(n), groups = (heads + most - 1) / most;
-    return (heads + groups - 1) / groups;
 }
 
 // A team of kTeam threads turns a stream of R x D f32 tiles into split operand tiles, 2048 values at a time
