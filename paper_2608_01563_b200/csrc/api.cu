@@ -179,9 +179,7 @@ int mgn_attn_fwd_accel(const float* q, const float* k, const float* v, float* o,
     void* q16 = w;
     void* k16 = w + align_up(nq * 2, 256);
     void* v16 = static_cast<char*>(k16) + align_up(nk * 2, 256);
-    if (mgn::launch_to_f16(q, q16, nq, st) != cudaSuccess || mgn::launch_to_f16(k, k16, nk, st) != cudaSuccess ||
-        mgn::launch_to_f16(v, v16, nk, st) != cudaSuccess)
-        return MGN_ERR_CUDA;
+    if (mgn::launch_to_f16(q, k, v, q16, k16, v16, nq, nk, st) != cudaSuccess) return MGN_ERR_CUDA;
     MainKernelTimer timer(st);
     return mgn::launch_fast_fwd_f16(p, q16, k16, v16, o, lse, status, st) == cudaSuccess ? MGN_OK : MGN_ERR_CUDA;
 }

@@ -253,7 +253,8 @@ cudaError_t launch_fast_fwd_small(const Problem& p, const void* q, const void* k
                                   unsigned* status, cudaStream_t st);
 // Forward of the accelerated policy: q16, k16, v16 are IEEE f16 copies (launch_to_f16) of f32
 // tensors, tensor-core products with f32 accumulation, O and LSE stored as f32.
-cudaError_t launch_to_f16(const float* in, void* out, size_t n, cudaStream_t st);
+cudaError_t launch_to_f16(const float* q, const float* k, const float* v, void* q16, void* k16, void* v16, size_t nq, size_t nk,
+                          cudaStream_t st);       // nq, nk: elements of q, of k and v
 cudaError_t launch_fast_fwd_f16(const Problem& p, const void* q16, const void* k16, const void* v16, float* o,
                                 float* lse, unsigned* status, cudaStream_t st);
 // With a single 128-key block every dQ tile receives one partial: the fused kernel then stores dq itself
