@@ -272,7 +272,8 @@ cudaError_t launch_fast_bwd(const Problem& p, const void* q, const void* k, cons
 //   where one CTA fits an SM (512 heads of 100 x 100: 67 / 78).
 // - Otherwise D <= 64 with at most 64 keys (64 x 8 heads of 50 x 16: 29.7 / 19.5; 1024 heads of 2048 x 16: 386 / 259), or, with
 //   more, eight tiles a head and heads for one round of CTAs (8 heads of 2048 x 128: 48 / 21; 128 of 1024 x 77: 39.8 / 38.9;
-//   but 128 of 512 x 100: 25.6 / 28.7, of 100 x 100: 15.3 / 18.4; 1024 of 2048 x 128: 388 / 416).
+//   but 128 of 512 x 100: 25.6 / 28.7, of 100 x 100: 15.3 / 18.4; 256 of 1024 x 120: 58.7 / 67.7, 288 of 1500 x 100:
+//   86.9 / 89.2; 1024 of 2048 x 128: 388 / 416).
 // - D = 128: heads that leave half of the SMs idle, with four tiles a head (eight beyond 64 keys): 8 heads of 2048 x 128
 //   69 / 27, 64 of 2048 x 100 81 / 69, 64 of 500 x 50 29.7 / 25.5; but 32 of 300 x 100 23.5 / 26.6, 128 of 1024 x 77 54 / 66.
 inline bool fast_bwd_is_small(const Problem& p, bool deterministic) {
@@ -280,7 +281,7 @@ inline bool fast_bwd_is_small(const Problem& p, bool deterministic) {
     const long long tiles = static_cast<long long>(p.group()) * ((p.Sq + 127) / 128);
     if (deterministic) return !(p.D == 128 && p.Sk > 64 && tiles == 1 && p.BHkv() > kSms);
     if (p.D == 128) return p.BHkv() <= kSms / 2 && tiles >= (p.Sk <= 64 ? 4 : 8);
-    return p.Sk <= 64 || (tiles >= 8 && p.BHkv() <= 2 * kSms);
+    return p.Sk <= 64 || (tiles >= 8 && p.BHkv() <= kSms);
 }
 cudaError_t launch_fast_bwd_small(const Problem& p, const void* q, const void* k, const void* v, const void* o,
                                   const void* d_o, const float* lse, const float* delta, void* dq, void* dk, void* dv,
