@@ -141,7 +141,7 @@ __device__ __forceinline__ Item make_item(int it, const Dims& dm, int n_tiles, i
     int hi = end - 1;
     w.lo = w.row0;
     w.blk0 = 0;
-    if (GEN) {                                 // packed heads of Sp rows: a tile that holds rows of two sees all positions
+    if (GEN && dm.Sp != dm.Sq) {               // packed heads of Sp rows: a tile that holds rows of two sees all positions
         w.lo = w.row0 % dm.Sp;
         hi = w.lo + (end - w.row0) - 1;
         if (hi >= dm.Sp) { w.lo = 0; hi = dm.Sp - 1; }
@@ -452,7 +452,8 @@ fast_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const int it = index_of(k);
         if (it < 0) break;
         const Item w = item_of(it);
-        const int i = GEN ? (w.row0 + r) % dm.Sp : w.row0 + r;      // position
+        // position (the division only where heads are packed: 512 heads of 500 x 300, D = 64, 64.1 -> 62.1 us)
+        const int i = GEN && dm.Sp != dm.Sq ? (w.row0 + r) % dm.Sp : w.row0 + r;
         float m_ref = -INFINITY, l = 0.f;
         // the exchange buffer carried the row sums of the last item to the epilogue warps
         if (k > 0) mbar_wait(bar(B_STEMPTY), (k - 1) & 1, status);
